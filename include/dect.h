@@ -478,7 +478,7 @@ dect_status dect_adm_tv_ex(const dect_plan *plan, const float *m, float *x, int 
  * c channels uses the next of these widths >= min(c, 64)), and the measured
  * median time of each variant in microseconds (-1 = not available):
  *   0-2 L1-cached gather with 4x4 / 8x8 / 16x16 pixel tiles per 256-thread block,
- *   3   shared-memory sinogram windows (cp.async staged),
+ *   3   none (falls back to 1),
  *   4-5 L1-cached gather, one 1024-thread block per SM, tiles of two / four
  *       block steps (8x8 / 16x8 pixels at 32 and 64 channels, 8x16 / 16x16 below),
  *   6-7 (16, 32 or 64 channels; otherwise 4 is used) each lane gathers 8
@@ -494,25 +494,28 @@ dect_status dect_plan_get_tuning(const dect_plan *plan, int images, int *choice,
 
 /* Fix the A^T variant used for batch width `images` (skipping the timing),
  * or pass choice = -1 to let the next ADM call time the candidates again.
- * Variant 3 falls back to 1 where the windows do not fit shared memory. */
+ * Variant 3 falls back to 1. */
 dect_status dect_plan_set_tuning(dect_plan *plan, int images, int choice);
 
 /*
  * Autotuner record of the forward projector A G inside dect_adm_tv, as
  * dect_plan_get_tuning gives it for A^T: the variant chosen for batch width
  * `images` and the measured median time of each (microseconds; -1 = not
- * timed).  All variants run one 1024-thread block per SM and a warp per ray:
+ * timed).  Variants 0-2 run one 1024-thread block per SM and a warp per ray:
  *   0 each lane gathers 4 channels of an entry (one 16-byte load); the row's
  *     table entries are loaded by the warp together and handed to the lanes
  *     by shuffles,
  *   1 each lane gathers 8 channels of an entry (two 16-byte loads), so fewer
  *     lanes receive each entry's (index, length), four entries per lane in
  *     flight; 16, 32 or 64 channels only (otherwise 0 is used),
- *   2 as 1 with two entries per lane in flight.
+ *   2 as 1 with two entries per lane in flight,
+ *   3 the plan's line table, a lane per ray and four channels; up to 16
+ *     channels, where the geometry has the table (otherwise 2, or 0 below 16
+ *     channels).
  * Timed on the set-up projection r = A f - beta m of the first ADM call
  * with that width.  Host memory: us has DECT_FWD_VARIANTS elements.
  */
-#define DECT_FWD_VARIANTS 3
+#define DECT_FWD_VARIANTS 4
 dect_status dect_plan_get_fwd_tuning(const dect_plan *plan, int images, int *choice,
                                      float us[DECT_FWD_VARIANTS]);
 

@@ -25,6 +25,9 @@
 //   k_fwd    q = A G  (ray-major table)                  ; |grad G|^2, |q|^2,
 //            then the last block forms Phi^k, the stopping test and
 //            alpha^k in FP64.
+// Up to 16 channels k_line_fwd may take the place of k_fwd: A G from the line
+// table (lines.cuh), gathering from G and from a transposed copy that k_bwd
+// writes beside it.
 //
 // Optional joint TV over the stacked image (both energies of a slice, channels
 // 2s and 2s + 1, which one thread always holds together): the TV norm and the
@@ -48,6 +51,7 @@
 
 #include "dect_internal.cuh"
 #include "kernels.cuh"
+#include "lines.cuh"
 
 namespace dect {
 namespace {
@@ -59,6 +63,13 @@ constexpr int kGrid = kSMs * 8;  // fixed grid of every reducing kernel
 constexpr int kFwdBlock = 1024;
 constexpr int kFwdGrid = kSMs;
 
+// block partials held per kernel: the grid of k_line_fwd goes beyond kGrid
+template <int NB>
+__host__ __device__ constexpr int part_blocks()
+{
+    return NB <= kLineMaxImages ? kSMs * 16 : kGrid;
+}
+
 // reduction slots; (TV, RR) and (DD, QQ) are reduced together
 enum { R_TV = 0, R_RR = 1, R_DD = 2, R_QQ = 3, R_GG = 4, R_COUNT = 5 };
 enum { C_TV = 0, C_BWD = 1, C_FWD = 2, C_RES = 3, C_COUNT = 4 };
@@ -66,7 +77,7 @@ enum { C_TV = 0, C_BWD = 1, C_FWD = 2, C_RES = 3, C_COUNT = 4 };
 struct AdmDev {
     // per-channel scalars
     double *red;       // [R_COUNT][NB] reduction results
-    double *part;      // [C_COUNT][2][kGrid][NB] block partials, per kernel
+    double *part;      // [C_COUNT][2][part_blocks][NB] block partials, per kernel
     unsigned *ctr;     // [C_COUNT] last-block counters, then the k_tv tile counter
     double *alpha;     // [NB] step applied by the next k_tv
     double *c_prev;    // [NB]
@@ -96,7 +107,7 @@ struct AdmConst {
 template <int NB>
 __device__ __forceinline__ double *part_of(const AdmDev &D, int kernel)
 {
-    return D.part + (size_t)kernel * 2 * kGrid * NB;
+    return D.part + (size_t)kernel * 2 * part_blocks<NB>() * NB;
 }
 
 // z-shrink of Eq. (8) per pixel on the 4-vector of both channels' gradients
@@ -599,12 +610,13 @@ __global__ void __launch_bounds__(TvTmaShape<NB>::THREADS) k_tv_tma(
 // sinogram lines its pixels gather are shared in L1.
 // VWL = 4: lanes gather 4 images of an entry, entries broadcast through a
 // per-warp shared-memory slot; VWL = 8 or 16: lanes gather VWL images of an
-// entry, R rounds in flight (row_dot_w; NB >= 16 only).
+// entry, R rounds in flight (row_dot_w; NB >= 16 only).  GT (may be
+// null): a transposed copy of G for k_line_fwd.
 template <int NB, int G_, int TW, int TH, int BLK, int VWL = 4, int R = 2>
 __global__ void __launch_bounds__(BLK) k_bwd(const int64_t *__restrict__ colptr,
                                                 const Entry *__restrict__ tent,
                                                 const float *__restrict__ r, const float *__restrict__ p,
-                                                float *__restrict__ G, AdmConst C, AdmDev D)
+                                                float *__restrict__ G, AdmConst C, AdmDev D, float *__restrict__ GT)
 {
     constexpr int VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
     constexpr int RPS = BLK / G_;  // pixels per block step
@@ -647,173 +659,11 @@ __global__ void __launch_bounds__(BLK) k_bwd(const int64_t *__restrict__ colptr,
                     nrm[0].v[c] = fmaf(out.v[c], out.v[c], nrm[0].v[c]);
                 }
                 st_keep<VW>(G + o, out, pol);
+                if (NB <= kLineMaxImages && GT) st_v<VW>(GT + ((int64_t)j * C.n + i) * NB + vl * VW, out);
             }
         }
     }
     reduce_images<NB, 1, BLK>(nrm, part_of<NB>(D, C_BWD), D.red + R_GG * NB, D.ctr + C_BWD, smem);
-}
-
-// G = mu A^T r + grad^T p with everything a tile needs staged in shared
-// memory: a block takes kWinTH x kWinTW pixel tiles; per tile, the block
-// copies the tile's entries (tile-major table, tile-local ray indices) and,
-// per view, the window of sinogram bins the tile meets into shared memory
-// with 16-byte cp.async copies, double-buffered so that the copies of the
-// next tile overlap the gathers of this one; the tile's pixels then read
-// only shared memory.
-
-template <int NB, int G>
-__device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_smem(const Entry *sent, int b, int e, int lr,
-                                                           const float *win)
-{
-    constexpr int VW = Batch<NB>::VW, LPE = Batch<NB>::CPB, EG = G / LPE;
-    const int grp = lr / LPE, vl = lr % LPE;
-    Vec<VW> acc;
-    acc.zero();
-#pragma unroll 4
-    for (int k = b + grp; k < e; k += EG) {
-        const Entry t = sent[k];
-        const Vec<VW> xv = ld_v<VW>(win + t.x * NB + vl * VW);
-        const float w = __int_as_float(t.y);
-#pragma unroll
-        for (int c = 0; c < VW; ++c) acc.v[c] = fmaf(w, xv.v[c], acc.v[c]);
-    }
-#pragma unroll
-    for (int off = LPE; off < G; off <<= 1)
-#pragma unroll
-        for (int c = 0; c < VW; ++c) acc.v[c] += __shfl_xor_sync(0xffffffffu, acc.v[c], off);
-    return acc;
-}
-
-constexpr int kWinBlock = 32 * kWinTP;  // one warp per pixel of a tile
-constexpr int kWinWarps = kWinBlock / 32;
-
-struct WinArgs {
-    const Entry *tmaj;
-    const int64_t *tbase;
-    const int *tpo, *wray0, *wcnt, *woff, *wtot;
-    int nv, nvp;
-    int win_floats;  // floats of one stage's sinogram window
-    int ent_max;     // entries of one stage's table part
-};
-
-// Data stage st in dynamic shared memory: [window floats][entries]; after the
-// two data stages, two descriptor stages of [wray0 | wcnt | woff] x nvp ints.
-__device__ __forceinline__ float *win_stage(float *dyn, const WinArgs &A, int st)
-{
-    return dyn + (size_t)st * (A.win_floats + 2 * A.ent_max);
-}
-__device__ __forceinline__ int *desc_stage(float *dyn, const WinArgs &A, int st)
-{
-    return reinterpret_cast<int *>(win_stage(dyn, A, 2)) + (size_t)st * 3 * A.nvp;
-}
-
-// Copies of tile `tile`'s view descriptors into descriptor stage ds (16-byte cp.async).
-__device__ __forceinline__ void win_copy_desc(const WinArgs &A, float *dyn, int tile, int ds)
-{
-    int *d = desc_stage(dyn, A, ds);
-    const int q = A.nvp / 4;  // 16-byte chunks per array
-    const int64_t o = (int64_t)tile * A.nvp;
-    for (int c = threadIdx.x; c < 3 * q; c += blockDim.x) {
-        const int a = c / q, k = (c % q) * 4;
-        const int *src = a == 0 ? A.wray0 : (a == 1 ? A.wcnt : A.woff);
-        cp_async16(d + a * A.nvp + k, src + o + k);
-    }
-}
-
-// Copies of tile `tile`'s entries and sinogram windows into data stage st,
-// using the descriptors already in descriptor stage ds; pixel offsets to spo.
-template <int NB>
-__device__ __forceinline__ void win_copy_data(const WinArgs &A, float *dyn, int (*spo)[kWinTP + 1],
-                                              const float *r, int tile, int st, int ds)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float *win = win_stage(dyn, A, st);
-    Entry *sent = reinterpret_cast<Entry *>(win + A.win_floats);
-    const int64_t e0 = A.tbase[tile], e1 = A.tbase[tile + 1];
-    const int nch = (int)((e1 - e0) / 2);
-    for (int c = threadIdx.x; c < nch; c += blockDim.x) cp_async16(sent + 2 * c, A.tmaj + e0 + 2 * c);
-    const int *d = desc_stage(dyn, A, ds);
-    for (int v = warp; v < A.nv; v += kWinWarps) {
-        const int ray0 = d[v], cnt = d[A.nvp + v], off = d[2 * A.nvp + v];
-        const int nc = cnt * NB / 4;
-        const float *src = r + (int64_t)ray0 * NB;
-        float *dst = win + (int64_t)off * NB;
-        for (int c = lane; c < nc; c += 32) cp_async16(dst + 4 * c, src + 4 * c);
-    }
-    if (threadIdx.x <= kWinTP) spo[st][threadIdx.x] = A.tpo[(int64_t)tile * (kWinTP + 1) + threadIdx.x];
-}
-
-template <int NB>
-__global__ void __launch_bounds__(kWinBlock, 1) k_bwd_win(WinArgs A, const float *__restrict__ r,
-                                                          const float *__restrict__ p,
-                                                          float *__restrict__ G, AdmConst C, AdmDev D)
-{
-    constexpr int VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
-    constexpr int G_ = 32;
-    extern __shared__ __align__(128) float dyn[];
-    __shared__ int spo[2][kWinTP + 1];
-    __shared__ double smem[reduce_smem_doubles<NB, kWinBlock>(1)];
-    const int lr = threadIdx.x & 31, grp = lr / LPE, vl = lr % LPE;
-    const int slot = threadIdx.x >> 5;  // pixel of the tile handled by this warp
-    const int64_t sN = C.N * NB;
-    const int tiles_x = (C.n + kWinTW - 1) / kWinTW;
-    const int ntiles = tiles_x * ((C.n + kWinTH - 1) / kWinTH);
-    Vec<VW> nrm[1];
-    nrm[0].zero();
-    // pipeline: at the top of the loop for tile t the group holding
-    // (data of t, descriptors of t + 1) is awaited; then the group
-    // (descriptors of t + 2, data of t + 1) is issued and overlaps compute(t)
-    const int g = gridDim.x;
-    int t0 = blockIdx.x;
-    if (t0 < ntiles) {
-        win_copy_desc(A, dyn, t0, 0);
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-        if (t0 + g < ntiles) win_copy_desc(A, dyn, t0 + g, 1);
-        win_copy_data<NB>(A, dyn, spo, r, t0, 0, 0);
-        cp_async_commit();
-    }
-    int it = 0;
-    for (int tile = t0; tile < ntiles; tile += g, ++it) {
-        const int st = it & 1;
-        cp_async_wait<0>();
-        __syncthreads();
-        const int next = tile + g, next2 = tile + 2 * g;
-        if (next2 < ntiles) win_copy_desc(A, dyn, next2, st);        // desc stage of t+2 = t % 2
-        if (next < ntiles) win_copy_data<NB>(A, dyn, spo, r, next, st ^ 1, st ^ 1);
-        cp_async_commit();
-        const int ty = tile / tiles_x, tx = tile % tiles_x;
-        const int i = ty * kWinTH + slot / kWinTW, j = tx * kWinTW + slot % kWinTW;
-        const bool ok = i < C.n && j < C.n;
-        const int64_t pix = (int64_t)i * C.n + j;
-        const int64_t o = pix * NB + vl * VW;
-        Vec<VW> p0, p1, pd, pr;
-        p0.zero(); p1.zero(); pd.zero(); pr.zero();
-        if (ok && grp == 0) {
-            p0 = ld_v<VW>(p + o);
-            p1 = ld_v<VW>(p + sN + o);
-            if (i + 1 < C.n) pd = ld_v<VW>(p + o + (int64_t)C.n * NB);
-            if (j + 1 < C.n) pr = ld_v<VW>(p + sN + o + NB);
-        }
-        const float *win = win_stage(dyn, A, st);
-        const Entry *sent = reinterpret_cast<const Entry *>(win + A.win_floats);
-        const int b = ok ? spo[st][slot] : 0, e = ok ? spo[st][slot + 1] : 0;
-        Vec<VW> acc = row_dot_smem<NB, G_>(sent, b, e, lr, win);
-        if (ok && grp == 0) {
-            Vec<VW> out;
-#pragma unroll
-            for (int c = 0; c < VW; ++c) {
-                float gt = (i > 0 ? p0.v[c] : 0.f) - pd.v[c] + (j > 0 ? p1.v[c] : 0.f) - pr.v[c];
-                out.v[c] = fmaf(C.mu, acc.v[c], gt);
-                nrm[0].v[c] = fmaf(out.v[c], out.v[c], nrm[0].v[c]);
-            }
-            st_keep<VW>(G + o, out, l2_evict_last_policy());
-        }
-        __syncthreads();  // every read of this stage precedes its next copies
-    }
-    cp_async_wait<0>();
-    reduce_images<NB, 1, kWinBlock>(nrm, part_of<NB>(D, C_BWD), D.red + R_GG * NB, D.ctr + C_BWD, smem);
 }
 
 // Step size and stopping test, FP64, one thread per channel (last block of k_fwd).
@@ -980,10 +830,142 @@ __global__ void __launch_bounds__(BLK) k_fwd(const int64_t *__restrict__ rowptr,
     }
 }
 
-// Exact residual of the current f (f_cur) against the carried one, for the
-// reports: QQ <- |A f - beta m|^2, GG <- |r - (A f - beta m)|^2 (q is
-// overwritten; call only where q is no longer needed).
+// ---------------------------------------------------------------------------
+// A on the line table (NB <= 16 channels).
+// ---------------------------------------------------------------------------
 
+// Sums of K quantities of the thread's channel (threadIdx.x % NB) over the
+// grid: as reduce_images, for kernels whose threads hold one channel each.
+// part holds K * gridDim.x * NB doubles.
+template <int NB, int K, int BLOCK>
+__device__ __forceinline__ bool reduce_channels(float (&v)[K], double *__restrict__ part, double *__restrict__ out,
+                                                unsigned *counter)
+{
+    constexpr int NW = BLOCK / 32, KN = K * NB, SUB = BLOCK / KN;
+    static_assert(NB <= 32 && KN <= BLOCK, "reduce_channels: block shape");
+    __shared__ double sm[NW * KN > BLOCK ? NW * KN : BLOCK];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+#pragma unroll
+        for (int off = NB; off < 32; off <<= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
+        if (lane < NB) sm[warp * KN + q * NB + lane] = (double)v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < KN) {
+        double s = 0.0;
+        for (int w = 0; w < NW; ++w) s += sm[w * KN + threadIdx.x];
+        part[(size_t)blockIdx.x * KN + threadIdx.x] = s;
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    const int i = threadIdx.x % KN, sub = threadIdx.x / KN;
+    double t = 0.0;
+    if (sub < SUB) {
+#pragma unroll 4
+        for (unsigned b = sub; b < gridDim.x; b += SUB) t += __ldcg(&part[(size_t)b * KN + i]);
+        sm[sub * KN + i] = t;
+    }
+    __syncthreads();
+    for (int half = SUB / 2; half > 0; half >>= 1) {  // SUB is a power of two
+        if (sub < half) sm[sub * KN + i] += sm[(sub + half) * KN + i];
+        __syncthreads();
+    }
+    if (threadIdx.x < KN) out[threadIdx.x] = sm[threadIdx.x];
+    if (threadIdx.x == 0) *counter = 0u;
+    __syncthreads();
+    return true;
+}
+
+// k_fwd on the line table (the same modes): src and its transpose srcT.
+template <int NB, int MODE>
+__global__ void __launch_bounds__(LineShape<NB>::BLOCK, LineShape<NB>::BLOCKS)
+    k_line_fwd(LineTable T, const float *__restrict__ src, const float *__restrict__ srcT, float *__restrict__ dst,
+               const float *__restrict__ m_planar, const float *__restrict__ beta_img, AdmConst C, AdmDev D,
+               const float *__restrict__ rc)
+{
+    constexpr int BLK = LineShape<NB>::BLOCK;
+    __shared__ LineSums<NB> sm;
+    const int ch = threadIdx.x % NB;
+    float nrm[2] = {0.f, 0.f};  // of channel ch
+    if (MODE == 1) {  // |grad G|^2
+        constexpr int U = 4;
+        const int64_t row = (int64_t)C.n * NB, tot = C.N * NB, gs = (int64_t)gridDim.x * BLK;
+        for (int64_t t0 = (int64_t)blockIdx.x * BLK + threadIdx.x; t0 < tot; t0 += U * gs) {
+            float gc[U], gu[U], gl[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t t = t0 + u * gs;
+                gc[u] = gu[u] = gl[u] = 0.f;
+                if (t < tot) {
+                    const int64_t pix = t / NB;
+                    const bool up = t >= row;  // not the first row
+                    const bool left = C.N <= 0xffffffffll ? (unsigned)pix % (unsigned)C.n != 0u : pix % C.n != 0;
+                    gc[u] = __ldg(src + t);
+                    gu[u] = up ? __ldg(src + t - row) : gc[u];
+                    gl[u] = left ? __ldg(src + t - NB) : gc[u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float d0 = gc[u] - gu[u], d1 = gc[u] - gl[u];
+                nrm[0] += d0 * d0 + d1 * d1;
+            }
+        }
+    }
+    const int ngb = T.ngb, ngrp = T.nv * ngb;
+    for (int gi = blockIdx.x; gi < ngrp; gi += gridDim.x) {
+        const int view = gi / ngb, gb = gi % ngb;
+        float acc[LineShape<NB>::VW];
+        line_ray_sums<NB>(T, view, gb, src, srcT, acc);
+        __syncthreads();  // the previous group's sums have been read
+        line_ray_store<NB>(sm, acc);
+        __syncthreads();
+        for (int e = threadIdx.x; e < 32 * NB; e += BLK) {
+            const int r = e / NB;
+            if (gb * 32 + r >= T.nb) break;
+            const int64_t ray = (int64_t)view * T.nb + gb * 32 + r;
+            float v = line_ray_value<NB>(sm, e, __ldg(T.len + ray));
+            if (MODE != 1) {
+                const int im = D.slot[ch];
+                if (im >= 0) v -= beta_img[ch] * m_planar[(int64_t)im * C.M + ray];
+                if (MODE >= 2) nrm[0] = fmaf(v, v, nrm[0]);
+                if (MODE == 3) {
+                    const float d = rc[ray * NB + ch] - v;
+                    nrm[1] = fmaf(d, d, nrm[1]);
+                }
+            } else {
+                nrm[1] = fmaf(v, v, nrm[1]);
+            }
+            dst[ray * NB + ch] = v;
+        }
+    }
+    if (MODE == 1) {
+        if (reduce_channels<NB, 2, BLK>(nrm, part_of<NB>(D, C_FWD), D.red + R_DD * NB, D.ctr + C_FWD))
+            adm_finish<NB>(C, D);
+    } else if (MODE == 2) {
+        float rr[1] = {nrm[0]};
+        reduce_channels<NB, 1, BLK>(rr, part_of<NB>(D, C_RES), D.red + R_RR * NB, D.ctr + C_RES);
+    } else if (MODE == 3) {
+        reduce_channels<NB, 2, BLK>(nrm, part_of<NB>(D, C_RES), D.red + R_QQ * NB, D.ctr + C_RES);
+    }
+}
+
+// r^0 = - beta m where f^0 = 0 (A f^0 = 0 needs no projection)
+template <int NB>
+__global__ void __launch_bounds__(256) k_r_zero(float *__restrict__ r, const float *__restrict__ m_planar,
+                                                const float *__restrict__ beta_img, AdmConst C, AdmDev D)
+{
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (t >= C.M * NB) return;
+    const int ch = (int)(t % NB), im = D.slot[ch];
+    r[t] = im >= 0 ? 0.f - beta_img[ch] * m_planar[(int64_t)im * C.M + t / NB] : 0.f;
+}
 
 // planar x[img][N] (times beta) -> interleaved f[N][NB]; and back (divided by beta).
 template <int NB>
@@ -1058,39 +1040,11 @@ struct Kern {
     static constexpr int GF = 32;                  // lanes per ray row
 };
 
-// A variants (autotuner candidates, one 1024-thread block per SM, a warp
-// per ray): 0 lanes gather 4 images of an entry; 1 lanes gather 8 images
-// (row_dot_w), four rounds of gathers in flight; 2 as 1 with two rounds.
-// Below 16 images only variant 0 exists (the others fall back to it).
-constexpr int kFwdVariants = DECT_FWD_VARIANTS;
-
-template <int NB, int MODE>
-void launch_fwd(const dect_plan *P, int variant, const float *src, float *dst, const float *m,
-                const float *beta, const AdmConst &C, const AdmDev &D, cudaStream_t s,
-                const float *rc = nullptr)
-{
-    constexpr int GF = Kern<NB>::GF;
-    switch (NB >= 16 ? variant : 0) {
-    case 1:
-        k_fwd<NB, GF, MODE, 8, 4, 1024><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, m, beta, C, D, rc);
-        break;
-    case 2:
-        k_fwd<NB, GF, MODE, 8, 2, 1024><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, m, beta, C, D, rc);
-        break;
-    default:
-        k_fwd<NB, GF, MODE, 4><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, m, beta, C, D, rc);
-        break;
-    }
-}
-
-template <int NB>
-void launch_residual_check(const dect_plan *P, int variant, const float *f_cur, float *q, const float *r,
-                           const float *m, const float *beta, const AdmConst &C, const AdmDev &D,
-                           cudaStream_t s)
-{
-    launch_fwd<NB, 3>(P, variant, f_cur, q, m, beta, C, D, s, r);
-    count_launches(1);
-}
+// A variants: 0-2 the CSR table, one 1024-thread block per SM, a warp per ray:
+// 0 lanes gather 4 images of an entry; 1 lanes gather 8 images (row_dot_w),
+// four rounds of gathers in flight; 2 as 1 with two rounds (below 16 images
+// 1 and 2 fall back to 0).  3 the line table (NB <= 16; otherwise 2).
+constexpr int kFwdVariants = DECT_FWD_VARIANTS, kFwdLines = 3;
 
 struct Work {
     float *f[2], *G, *lam, *z, *p, *r, *q, *beta;
@@ -1100,47 +1054,57 @@ struct Work {
     int *map;         // [NB] slot map while narrowing into this workspace
     unsigned *ctr;
     AdmDev D;
-    int win_grid;     // > 0: A^T through shared-memory windows with this grid
-    size_t win_smem;  // its dynamic shared memory
+    float *GT;        // transposed copy of G, or of an image being projected (null: no line table at this width)
     int bwd;          // A^T variant in use
     int fwd;          // A variant in use
     int tv;           // TV-step variant in use (0 k_tv, 1 k_tv_tma)
     int tv_grid;      // blocks of k_tv_tma
 };
 
-constexpr size_t kWinSmemMax = 210 * 1024;
-
-// Enable the windowed A^T for this plan and batch width when two stages of
-// its window and entries fit in shared memory.
-template <int NB>
-cudaError_t setup_window(const dect_plan *P, Work &W)
+// A of one image batch: src -> dst in the given mode of k_fwd.
+template <int NB, int MODE>
+void launch_fwd(const dect_plan *P, const Work &W, int variant, const float *src, float *dst, const AdmConst &C,
+                cudaStream_t s, const float *rc = nullptr)
 {
-    W.win_grid = 0;
-    W.win_smem = 0;
-    if (P->win_max <= 0) return cudaSuccess;
-    const size_t stage = (size_t)P->win_max * NB * sizeof(float) + (size_t)P->tile_ent_max * sizeof(Entry);
-    const size_t bytes = 2 * stage + 2 * 3 * sizeof(int) * (size_t)P->nvp;
-    if (bytes > kWinSmemMax) return cudaSuccess;
-    auto kern = k_bwd_win<NB>;
-    // the attribute is per kernel and process-wide: always the same cap, so
-    // concurrent calls on plans with different windows cannot race on it
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWinSmemMax);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kWinBlock, bytes);
-    if (e != cudaSuccess) return e;
-    if (per_sm <= 0) return cudaSuccess;
-    int grid = kSMs * per_sm;
-    if (grid > kGrid) grid = kGrid;
-    if (grid > P->win_tiles) grid = P->win_tiles;
-    W.win_grid = grid;
-    W.win_smem = bytes;
-    return cudaSuccess;
+    constexpr int GF = Kern<NB>::GF;
+    const AdmDev &D = W.D;
+    if constexpr (NB <= kLineMaxImages) {
+        if (variant == kFwdLines && W.GT) {
+            const LineTable &T = P->lines;
+            if (MODE != 1) {  // (k_bwd writes G's transpose)
+                k_line_transpose<NB><<<transpose_grid(T.n), 256, 0, s>>>(src, W.GT, T.n);
+                count_launches(1);
+            }
+            k_line_fwd<NB, MODE><<<even_grid(line_groups(T), part_blocks<NB>()), LineShape<NB>::BLOCK, 0, s>>>(
+                T, src, W.GT, dst, W.m, W.beta, C, D, rc);
+            return;
+        }
+    }
+    switch (NB >= 16 ? std::min(variant, 2) : 0) {
+    case 1:
+        k_fwd<NB, GF, MODE, 8, 4, 1024><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, W.m, W.beta, C, D, rc);
+        break;
+    case 2:
+        k_fwd<NB, GF, MODE, 8, 2, 1024><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, W.m, W.beta, C, D, rc);
+        break;
+    default:
+        k_fwd<NB, GF, MODE, 4><<<kFwdGrid, 1024, 0, s>>>(P->rowptr, P->ent, src, dst, W.m, W.beta, C, D, rc);
+        break;
+    }
+}
+
+// Exact residual of the current f (f_cur) against the carried one, for the
+// reports: QQ <- |A f - beta m|^2, GG <- |r - (A f - beta m)|^2 (q is
+// overwritten; call only where q is no longer needed).
+template <int NB>
+void launch_residual_check(const dect_plan *P, const Work &W, const float *f_cur, const AdmConst &C, cudaStream_t s)
+{
+    launch_fwd<NB, 3>(P, W, W.fwd, f_cur, W.q, C, s, W.r);
+    count_launches(1);
 }
 
 // A^T variants (autotuner candidates): 0-2 L1-cached gather with 4x4 / 8x8 /
-// 16x16 pixel tiles per 256-thread block; 3 shared-memory sinogram windows;
-// 4-5 L1-cached gather with one 1024-thread block per SM over tiles of two
+// 16x16 pixel tiles per 256-thread block; 3 none (1 takes its place); 4-5 L1-cached gather with one 1024-thread block per SM over tiles of two
 // or four block steps (8 x 8 / 16 x 8 pixels at 32 lanes per pixel, 8 x 16 /
 // 16 x 16 at 16), whose lines then stay in one L1; 6-7 lanes gather 8
 // images of an entry (row_dot_w, NB >= 16 only): 6 with the lanes and tiles
@@ -1152,35 +1116,30 @@ void launch_bwd(const dect_plan *P, const Work &W, const AdmConst &C, int varian
 {
     constexpr int GB = Kern<NB>::GB;
     constexpr int RPS1k = 1024 / GB;  // pixels per step of a 1024-thread block
+    float *GT = W.fwd == kFwdLines ? W.GT : nullptr;
     switch (variant) {
     case 0:
-        k_bwd<NB, GB, 4, 4, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+        k_bwd<NB, GB, 4, 4, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 2:
-        k_bwd<NB, GB, 16, 16, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+        k_bwd<NB, GB, 16, 16, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 4:
-        k_bwd<NB, GB, 8, RPS1k / 4, 1024><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+        k_bwd<NB, GB, 8, RPS1k / 4, 1024><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 5:
-        k_bwd<NB, GB, 16, RPS1k / 4, 1024><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+        k_bwd<NB, GB, 16, RPS1k / 4, 1024><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 6:  // 8 images per lane, the lanes and tiles of variant 4
         if constexpr (NB >= 16)
-            k_bwd<NB, GB, 8, RPS1k / 4, 1024, 8, 4><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+            k_bwd<NB, GB, 8, RPS1k / 4, 1024, 8, 4><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 7:  // 8 images per lane, 16 lanes per pixel (two pixels per warp), 8 x 8 tiles
         if constexpr (NB >= 16)
-            k_bwd<NB, 16, 8, 8, 1024, 8, 4><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+            k_bwd<NB, 16, 8, 8, 1024, 8, 4><<<kSMs, 1024, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
-    case 3: {
-        WinArgs A{P->tmaj, P->tbase, P->tpo, P->wray0, P->wcnt, P->woff, P->wtot, P->nv, P->nvp,
-                  P->win_max * NB, P->tile_ent_max};
-        k_bwd_win<NB><<<W.win_grid, kWinBlock, W.win_smem, s>>>(A, W.r, W.p, W.G, C, W.D);
-        break;
-    }
     default:
-        k_bwd<NB, GB, 8, 8, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D);
+        k_bwd<NB, GB, 8, 8, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     }
 }
@@ -1201,7 +1160,7 @@ cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     const int idx = nb_index<NB>();
     if (P->bwd_choice[idx] >= 0) {
         W.bwd = P->bwd_choice[idx];
-        if (W.bwd == 3 && W.win_grid <= 0) W.bwd = 1;
+        if (W.bwd == 3) W.bwd = 1;
         if (W.bwd >= 6 && NB < 16) W.bwd = 4;
         return cudaSuccess;
     }
@@ -1212,7 +1171,7 @@ cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     float best_us = 1e30f;
     for (int v = 0; v < kBwdVariants && e == cudaSuccess; ++v) {
         P->bwd_us[idx][v] = -1.f;
-        if (v == 3 && W.win_grid <= 0) continue;
+        if (v == 3) continue;
         if (v >= 6 && NB < 16) continue;  // wide-lane variants need 16 images
         launch_bwd<NB>(P, W, C, v, s);
         count_launches(1);
@@ -1253,6 +1212,7 @@ cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     const int idx = nb_index<NB>();
     if (P->fwd_choice[idx] >= 0) {
         W.fwd = P->fwd_choice[idx];
+        if (W.fwd == kFwdLines && !W.GT) W.fwd = NB >= 16 ? 2 : 0;
         return cudaSuccess;
     }
     cudaEvent_t a = nullptr, b = nullptr;
@@ -1262,13 +1222,13 @@ cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     float best_us = 1e30f;
     for (int v = 0; v < kFwdVariants && e == cudaSuccess; ++v) {
         P->fwd_us[idx][v] = -1.f;
-        if (v > 0 && NB < 16) continue;  // only variant 0 below 16 images
-        launch_fwd<NB, 0>(P, v, W.f[0], W.r, W.m, W.beta, C, W.D, s);
+        if (v == kFwdLines ? !W.GT : v > 0 && NB < 16) continue;  // of the others only 0 below 16 images
+        launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
         count_launches(1);
         float t[3];
         for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
             e = cudaEventRecord(a, s);
-            launch_fwd<NB, 0>(P, v, W.f[0], W.r, W.m, W.beta, C, W.D, s);
+            launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
             count_launches(1);
             if (e == cudaSuccess) e = cudaEventRecord(b, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(b);
@@ -1413,25 +1373,25 @@ void enqueue_iteration(const dect_plan *P, const Work &W, const AdmConst &C, int
                        const IterEvents *ev)
 {
     launch_tv<NB>(W, C, par, 0, s);
-    if (C.nonneg) launch_fwd<NB, 2>(P, W.fwd, W.f[1 - par], W.r, W.m, W.beta, C, W.D, s);
+    if (C.nonneg) launch_fwd<NB, 2>(P, W, W.fwd, W.f[1 - par], W.r, C, s);
     if (ev) cudaEventRecordWithFlags(ev->b0, s, cudaEventRecordExternal);
     launch_bwd<NB>(P, W, C, W.bwd, s);
     if (ev) cudaEventRecordWithFlags(ev->b1, s, cudaEventRecordExternal);
     if (ev) cudaEventRecordWithFlags(ev->f0, s, cudaEventRecordExternal);
-    launch_fwd<NB, 1>(P, W.fwd, W.G, W.q, nullptr, nullptr, C, W.D, s);
+    launch_fwd<NB, 1>(P, W, W.fwd, W.G, W.q, C, s);
     if (ev) cudaEventRecordWithFlags(ev->f1, s, cudaEventRecordExternal);
 }
 
 int kernels_per_iteration(const AdmConst &C) { return C.nonneg ? 4 : 3; }
 
 // Workspace of one batch width: one allocation, laid out once to size and
-// then for real, zeroed; the windowed A^T set up for this width.
+// then for real, zeroed.
 template <int NB>
 cudaError_t alloc_work(const dect_plan *P, Work &W, char **base_out, const float *m, cudaStream_t s)
 {
     const int64_t N = P->N, M = P->M;
     const size_t nf = (size_t)N * NB, nr = (size_t)M * NB;
-    const size_t ndbl = (size_t)R_COUNT * NB + (size_t)C_COUNT * 2 * kGrid * NB + 4 * NB;
+    const size_t ndbl = (size_t)R_COUNT * NB + (size_t)C_COUNT * 2 * part_blocks<NB>() * NB + 4 * NB;
     const size_t nint = 5 * NB + 8;
     auto layout = [&](char *b) -> size_t {
         size_t o = 0;
@@ -1442,8 +1402,9 @@ cudaError_t alloc_work(const dect_plan *P, Work &W, char **base_out, const float
         W.lam = (float *)take(2 * nf * 4);
         W.z = (float *)take(2 * nf * 4);
         W.p = (float *)take(2 * nf * 4);
-        W.r = (float *)take((nr + 2 * NB) * 4);  // windows may end one ray past M
+        W.r = (float *)take(nr * 4);
         W.q = (float *)take(nr * 4);
+        W.GT = NB <= kLineMaxImages && P->lines.ok ? (float *)take(nf * 4) : nullptr;
         W.beta = (float *)take(64 * 4);
         W.dbl = (double *)take(ndbl * 8);
         W.ints = (int *)take(nint * 4);
@@ -1460,7 +1421,7 @@ cudaError_t alloc_work(const dect_plan *P, Work &W, char **base_out, const float
     AdmDev &D = W.D;
     D.red = W.dbl;
     D.part = D.red + R_COUNT * NB;
-    D.alpha = D.part + (size_t)C_COUNT * 2 * kGrid * NB;
+    D.alpha = D.part + (size_t)C_COUNT * 2 * part_blocks<NB>() * NB;
     D.c_prev = D.alpha + NB;
     D.phi_prev = D.c_prev + NB;
     D.rel = D.phi_prev + NB;
@@ -1473,20 +1434,19 @@ cudaError_t alloc_work(const dect_plan *P, Work &W, char **base_out, const float
     D.all_done = D.k + 1;
     D.bad = D.all_done + 1;
     D.ctr = W.ctr;
-    e = cudaMemsetAsync(base, 0, bytes, s);
-    if (e == cudaSuccess) e = setup_window<NB>(P, W);
-    return e;
+    return cudaMemsetAsync(base, 0, bytes, s);
 }
 
 // Average algorithmic bytes per profiled launch, folded over batch widths.
 template <int NB>
-void add_profile_bytes(const dect_plan *P, dect_adm_profile *prof, int64_t launches_before)
+void add_profile_bytes(const dect_plan *P, const Work &W, dect_adm_profile *prof, int64_t launches_before)
 {
     if (!prof) return;
     const int64_t now = prof->fwd_launches, add = now - launches_before;
     if (now <= 0 || add <= 0) return;
     // A: table + row pointers, G read, q written
-    const double fwd = 8.0 * P->nnz + 8.0 * (P->M + 1) + 4.0 * NB * (P->N + P->M);
+    double fwd = 8.0 * P->nnz + 8.0 * (P->M + 1) + 4.0 * NB * (P->N + P->M);
+    if (W.fwd == kFwdLines) fwd = 4.0 * P->M * P->n + 4.0 * NB * (P->N + P->M);  // the line table's q
     // A^T: table + column pointers, r and the two components of p read, G written
     const double bwd = 8.0 * P->nnz + 8.0 * (P->N + 1) + 4.0 * NB * (P->M + 3 * P->N);
     prof->table_bytes_fwd = (int64_t)(((double)prof->table_bytes_fwd * launches_before + fwd * add) / now);
@@ -1629,8 +1589,8 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
                         W2.fwd = 0;
                         // time the A and A^T variants on the empty workspace, before the state arrives
                         W2.tv = 0;
-                        err = tune_bwd<NB2>(P, W2, C, cs);
-                        if (err == cudaSuccess) err = tune_fwd<NB2>(P, W2, C, cs);
+                        err = tune_fwd<NB2>(P, W2, C, cs);
+                        if (err == cudaSuccess) err = tune_bwd<NB2>(P, W2, C, cs);
                         if (err == cudaSuccess) err = tune_tv<NB2>(P, W2, C, cs);
                     }
                     if (err == cudaSuccess)
@@ -1655,7 +1615,7 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
                     // residual against A f - beta m (q and the QQ / GG slots of
                     // this workspace are free now), then write their reports
                     if (err == cudaSuccess) {
-                        launch_residual_check<NB>(P, W.fwd, W.f[par], W.q, W.r, W.m, W.beta, C, D, cs);
+                        launch_residual_check<NB>(P, W, W.f[par], C, cs);
                         err = cudaGetLastError();
                     }
                     if (err == cudaSuccess) err = cudaMemcpyAsync(hred.data(), D.red, sizeof(double) * R_COUNT * NB, cudaMemcpyDeviceToHost, cs);
@@ -1673,7 +1633,7 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
                     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, ev, 0);
                     if (err == cudaSuccess) {
                         // release this phase, then continue at NB2
-                        add_profile_bytes<NB>(P, prof, prof_before);
+                        add_profile_bytes<NB>(P, W, prof, prof_before);
                         cudaFreeAsync(base, s);
                         base = nullptr;
                         if (gx_block) cudaGraphExecDestroy(gx_block);
@@ -1709,16 +1669,16 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
     const int par = done_iters & 1;
     if (err == cudaSuccess) {
         launch_tv<NB>(W, C, par, 1, cs);
-        if (C.nonneg) launch_fwd<NB, 2>(P, W.fwd, W.f[1 - par], W.r, W.m, W.beta, C, D, cs);
+        if (C.nonneg) launch_fwd<NB, 2>(P, W, W.fwd, W.f[1 - par], W.r, C, cs);
         k_unpack<NB><<<(unsigned)((tn + 255) / 256), 256, 0, cs>>>(W.f[1 - par], x, N, D.slot, D.active, 0,
                                                                    W.beta);
         count_launches(C.nonneg ? 3 : 2);
-        launch_residual_check<NB>(P, W.fwd, W.f[1 - par], W.q, W.r, W.m, W.beta, C, D, cs);
+        launch_residual_check<NB>(P, W, W.f[1 - par], C, cs);
         err = cudaGetLastError();
     }
     if (err == cudaSuccess) err = cudaEventRecord(ev, cs);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, ev, 0);
-    add_profile_bytes<NB>(P, prof, prof_before);
+    add_profile_bytes<NB>(P, W, prof, prof_before);
 
     std::vector<double> hred(R_COUNT * NB), hrel(NB);
     std::vector<int> hit(NB), hconv(NB), hslot(NB);
@@ -1793,8 +1753,8 @@ cudaError_t pretune(const dect_plan *P, const float *m, const AdmConst &C, cudaS
         W.bwd = 1;
         W.fwd = 0;
         W.tv = 0;
-        if (e == cudaSuccess) e = tune_bwd<NB>(P, W, C, s);
         if (e == cudaSuccess) e = tune_fwd<NB>(P, W, C, s);
+        if (e == cudaSuccess) e = tune_bwd<NB>(P, W, C, s);
         if (e == cudaSuccess) e = tune_tv<NB>(P, W, C, s);
         if (base) cudaFreeAsync(base, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1847,7 +1807,10 @@ dect_status run_chunk(const dect_plan *P, const float *m, float *x, int nimg,
     // r^0 = A f^0 - beta m, with the A variant the autotuner keeps
     W.fwd = 0;
     if ((e = tune_fwd<NB>(P, W, C, s)) != cudaSuccess) return fail(e);
-    launch_fwd<NB, 0>(P, W.fwd, W.f[0], W.r, m, W.beta, C, D, s);
+    if (prm->warm_start)
+        launch_fwd<NB, 0>(P, W, W.fwd, W.f[0], W.r, C, s);
+    else
+        k_r_zero<NB><<<(unsigned)((P->M * NB + 255) / 256), 256, 0, s>>>(W.r, m, W.beta, C, D);
     count_launches(1);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
     W.bwd = 1;

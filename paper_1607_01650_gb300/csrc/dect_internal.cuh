@@ -14,10 +14,6 @@ namespace dect {
 constexpr int kSMs = 152;          // GB300: 2 dies x 76 SMs
 constexpr int kMaxBatchImages = 64; // images interleaved per ADM pass
 constexpr int kTablePad = 512;      // zero entries after the last row of each table
-// A^T with shared-memory sinogram windows: pixel tiles of kWinTH x kWinTW
-constexpr int kWinTH = 4, kWinTW = 4;
-constexpr int kWinTP = kWinTH * kWinTW;
-constexpr int kWinMaxViews = 4096;
 
 // Thread-local text of the last CUDA error (returned by dect_last_error()).
 void set_error(const char *where, cudaError_t e);
@@ -85,6 +81,25 @@ __device__ __forceinline__ bool check_index(int64_t i, int64_t bound, unsigned s
 #define DECT_IDX_OK(i, bound, site) true
 #endif
 
+// The line table of a fan-beam plan (lines.cuh): device pointers.
+struct LineTable {
+    int ok;          // built; the other fields hold only then
+    int n, nv, nb;
+    int nbp;         // row stride of q and walk, bins rounded up to 32
+    int nblk;        // blocks of 32 lines
+    int ngb;         // groups of 32 rays of a view, nbp / 32
+    float *q;        // [nv][nblk][nbp / 32][32 lines][32 rays] fraction of the ray's length in column c
+    uint2 *walk;     // [nv][nblk][nbp] columns of 32 lines of a ray
+    float2 *len;     // [nv * nb] length of the ray in a line, in two words
+    unsigned char *cls;  // [nv * nb] class of the ray
+
+    // element of q of (view, line, ray): tiles of 32 x 32, contiguous
+    __host__ __device__ int64_t at(int v, int line, int b) const
+    {
+        return ((((int64_t)v * nblk + (line >> 5)) * ngb + (b >> 5)) << 10) + ((line & 31) << 5) + (b & 31);
+    }
+};
+
 }  // namespace dect
 
 struct dect_plan {
@@ -99,25 +114,7 @@ struct dect_plan {
     dect::Entry *ent;  // [nnz]  {pixel, len}
     int64_t *colptr;   // [N + 1], pixel-major table (CSR of A^T)
     dect::Entry *tent; // [nnz]  {ray, len}, rays increasing within a pixel
-    // Per pixel tile (kWinTH x kWinTW) and view: the window of the tile's rays,
-    // [wray0, wray0 + wcnt) (even start and count), placed at woff in the
-    // tile's shared-memory window of wtot rays; tlocal = tent with the ray
-    // replaced by its index in the tile's window.  win_max = max wtot
-    // (0 when the windowed A^T is not available for this geometry).
-    int win_tiles;
-    int win_max;
-    int nvp;                   // descriptor stride per tile: nv rounded up to 4
-    int *wray0, *wcnt, *woff;  // [win_tiles * nvp]
-    int *wtot;                 // [win_tiles]
-    dect::Entry *tlocal;       // [nnz + pad]
-    // The same entries tile-major: tile t's pixels (row-major inside the tile)
-    // at tmaj[tbase[t] .. tbase[t + 1]) (even offsets, zero-padded to an even
-    // count); pixel s of tile t at tpo[t * (kWinTP + 1) + s] relative to
-    // tbase[t].  tile_ent_max = max entries of a tile.
-    dect::Entry *tmaj;
-    int64_t *tbase;            // [win_tiles + 1]
-    int *tpo;                  // [win_tiles * (kWinTP + 1)]
-    int tile_ent_max;
+    dect::LineTable lines;  // the narrow batches' form of the matrix (lines.cuh)
     // Autotuner cache: chosen A^T variant per ADM batch width (index log2(NB) - 1),
     // -1 until the first ADM call with that width has timed the candidates.
     mutable int bwd_choice[6];
@@ -145,6 +142,17 @@ cudaError_t launch_project_planar(const dect_plan *p, const float *x, float *y, 
                                   cudaStream_t s);
 cudaError_t launch_backproject_planar(const dect_plan *p, const float *y, float *x, int batch,
                                       cudaStream_t s);
+
+// Line table of a fan-beam plan (lines.cu).  lines_alloc leaves T.ok = 0 where
+// the form cannot hold or memory is short; the Siddon fill (plan.cu) then writes
+// q and the columns, and lines_finish the walk words.  *d_bad (device, zeroed by
+// the caller) becomes non-zero where the rays do not fit the form.
+struct RayPts {
+    double sx, sy, dx_, dy_;
+};
+cudaError_t lines_alloc(LineTable &T, int n, int nv, int nb, cudaStream_t s);
+cudaError_t lines_finish(LineTable &T, const short *d_col, int *d_bad, cudaStream_t s);
+void lines_free(LineTable &T);
 
 // On-the-fly projector geometry of a plan (batch.cu): built and cached on the
 // first call; synchronises `s` then.

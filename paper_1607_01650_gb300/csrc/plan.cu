@@ -27,11 +27,6 @@ namespace {
 
 __device__ constexpr double kInf = __builtin_huge_val();
 
-// Ray end points, FP64: (Sx, Sy, Dx, Dy).
-struct RayPts {
-    double sx, sy, dx_, dy_;
-};
-
 struct Grid {
     int n;
     double px;
@@ -99,8 +94,10 @@ __device__ __forceinline__ void axis_advance(AxisWalk &w, const Grid &g, double 
     }
 }
 
-// Walk one ray.  Writes entries when `out` is non-null; returns the count.
-__device__ int siddon_walk(const RayPts &r, const Grid &g, Entry *out, int *grid_aligned)
+// Walk one ray: emit(k, row, column, length in FP64) for the k-th element, in walk
+// order; returns their count.
+template <typename Emit>
+__device__ int siddon_walk(const RayPts &r, const Grid &g, Emit emit, int *grid_aligned)
 {
     const double dx = __dsub_rn(r.dx_, r.sx);
     const double dy = __dsub_rn(r.dy_, r.sy);
@@ -146,7 +143,7 @@ __device__ int siddon_walk(const RayPts &r, const Grid &g, Entry *out, int *grid
     // pixel of the previous piece (a crossing within rounding of a grid
     // corner) are added to it, in walk order, before the single FP32 rounding.
     int cnt = 0;
-    int pend_pix = -1;
+    int pend_pix = -1, pend_row = 0, pend_col = 0;
     double pend_len = 0.0;
     double cur = amin;
     // at most 2(n+1) crossings plus the exit
@@ -164,11 +161,10 @@ __device__ int siddon_walk(const RayPts &r, const Grid &g, Entry *out, int *grid
                 if (pix == pend_pix) {
                     pend_len = __dadd_rn(pend_len, seg);
                 } else {
-                    if (pend_pix >= 0) {
-                        if (out) out[cnt] = make_int2(pend_pix, __float_as_int(__double2float_rn(pend_len)));
-                        ++cnt;
-                    }
+                    if (pend_pix >= 0) emit(cnt++, pend_row, pend_col, pend_len);
                     pend_pix = pix;
+                    pend_row = row;
+                    pend_col = col;
                     pend_len = seg;
                 }
             }
@@ -178,10 +174,7 @@ __device__ int siddon_walk(const RayPts &r, const Grid &g, Entry *out, int *grid
         if (wy.next == a1) axis_advance(wy, g, r.sy, dy, amax);
         cur = a1;
     }
-    if (pend_pix >= 0) {
-        if (out) out[cnt] = make_int2(pend_pix, __float_as_int(__double2float_rn(pend_len)));
-        ++cnt;
-    }
+    if (pend_pix >= 0) emit(cnt++, pend_row, pend_col, pend_len);
     return cnt;
 }
 
@@ -191,16 +184,127 @@ __global__ void k_siddon_count(const RayPts *__restrict__ rays, int64_t M, Grid 
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= M) return;
     int al = 0;
-    counts[r] = siddon_walk(rays[r], g, nullptr, &al);
+    counts[r] = siddon_walk(rays[r], g, [](int, int, int, double) {}, &al);
     if (al) atomicAdd(aligned, 1ull);
 }
 
-__global__ void k_siddon_fill(const RayPts *__restrict__ rays, int64_t M, Grid g,
-                              const int64_t *__restrict__ rowptr, Entry *__restrict__ ent)
+// Fills a ray's row of the CSR table and, with T.ok, its lines of the line
+// table: q, and in col (laid out like q) the column c of each line, or kColOut
+// where the ray does not meet the line inside the image (then q = 1 left and
+// 0 right of it).  *bad: a line that does not fit the form.
+constexpr short kColOut = -32768;
+
+struct LineFill {
+    const LineTable &T;
+    short *col;
+    const RayPts &r;
+    double dx, dy, L, lo, px;
+    int v, b;        // view and bin
+    int cls, up;     // class; lines met in increasing order
+    int next;        // the line expected next
+    int line, k;     // line being collected, its elements so far
+    int c0;
+    double l0, l1;   // lengths in columns c0 and c0 + 1
+    bool bad;
+
+    __device__ LineFill(const LineTable &T_, short *col_, const RayPts &r_, const Grid &g, int64_t ray)
+        : T(T_), col(col_), r(r_), lo(g.lo), px(g.px), line(-1), k(0), c0(0), l0(0.0), l1(0.0), bad(false)
+    {
+        dx = __dsub_rn(r.dx_, r.sx);
+        dy = __dsub_rn(r.dy_, r.sy);
+        cls = fabs(dx) <= fabs(dy) ? 0 : 1;
+        const double d = cls ? dx : dy;
+        L = px * sqrt(dx * dx + dy * dy) / fabs(d);
+        up = d > 0.0;
+        next = up ? 0 : T.n - 1;
+        v = (int)(ray / T.nb);
+        b = (int)(ray % T.nb);
+        T.len[ray] = make_float2((float)L, (float)(L - (double)(float)L));
+        T.cls[ray] = (unsigned char)cls;
+    }
+    __device__ void put(int ln, short c, float q)
+    {
+        const int64_t o = T.at(v, ln, b);
+        T.q[o] = q;
+        col[o] = c;
+    }
+    // lines from `next` up to (not including) ln lie outside the image for this ray
+    __device__ void skip_to(int ln)
+    {
+        for (; next != ln; next += up ? 1 : -1) {
+            const double mid = lo + ((double)next + 0.5) * px;
+            const double x = cls ? r.sy + (mid - r.sx) / dx * dy : r.sx + (mid - r.sy) / dy * dx;
+            put(next, kColOut, x < 0.0 ? 1.f : 0.f);
+        }
+    }
+    __device__ void flush()
+    {
+        if (line < 0) return;
+        const double tot = l0 + l1;
+        const bool sliver = tot < 1e-10 * L, full = fabs(tot - L) < 1e-9 * L;
+        if (sliver || (up ? line < next : line > next)) return;  // (skip_to fills a sliver's line)
+        skip_to(line);
+        next += up ? 1 : -1;
+        const bool two = l1 >= 1e-10 * L, one = l0 >= 1e-10 * L;
+        if (full) {
+            if (two && one) put(line, (short)c0, (float)(l0 / tot));
+            else put(line, (short)(one ? c0 : c0 + 1), 1.f);
+        } else if (!two && c0 == 0) {  // enters or leaves through the low side in this line
+            put(line, -1, (float)(1.0 - l0 / L));
+        } else if (!(two && one) && c0 + (two ? 1 : 0) == T.n - 1) {  // through the high side
+            put(line, (short)(T.n - 1), (float)(tot / L));
+        } else {
+            put(line, kColOut, 1.f);
+            bad = true;
+        }
+    }
+    __device__ void add(int row, int column, double len)
+    {
+        const int ln = cls ? column : row, c = cls ? row : column;
+        if (ln != line) {
+            flush();
+            line = ln;
+            k = 1;
+            c0 = c;
+            l0 = len;
+            l1 = 0.0;
+            return;
+        }
+        if (c == c0 + 1) l1 += len;
+        else if (c == c0 - 1 && l1 == 0.0) {
+            l1 = l0;
+            l0 = len;
+            c0 = c;
+        } else if (len >= 1e-10 * L) bad = true;
+    }
+    __device__ void finish()
+    {
+        flush();
+        skip_to(up ? T.n : -1);
+    }
+};
+
+__global__ void k_siddon_fill(const RayPts *__restrict__ rays, int64_t M, Grid g, const int64_t *__restrict__ rowptr,
+                              Entry *__restrict__ ent, LineTable T, short *__restrict__ col, int *__restrict__ bad)
 {
     int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= M) return;
-    siddon_walk(rays[r], g, ent + rowptr[r], nullptr);
+    const RayPts ray = rays[r];
+    Entry *out = ent + rowptr[r];
+    auto entry = [&](int k, int row, int c, double len) {
+        out[k] = make_int2(row * g.n + c, __float_as_int(__double2float_rn(len)));
+    };
+    if (!T.ok) {
+        siddon_walk(ray, g, entry, nullptr);
+        return;
+    }
+    LineFill F(T, col, ray, g, r);
+    siddon_walk(ray, g, [&](int k, int row, int c, double len) {
+        entry(k, row, c, len);
+        F.add(row, c, len);
+    }, nullptr);
+    F.finish();
+    if (F.bad) atomicOr(bad, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -396,122 +500,6 @@ __global__ void k_col_sort(const int64_t *__restrict__ colptr, int64_t N,
     }
 }
 
-// Per-tile sinogram windows for the shared-memory A^T (one block per tile):
-// per view the range of bins that the tile's pixels meet, widened to an even
-// start and an even count (16-byte aligned copies for any batch of >= 2
-// images); prefix offsets; and the tile-local index of every entry.
-__global__ void k_win_build(const int64_t *__restrict__ colptr, const Entry *__restrict__ tent, int n,
-                            int nv, int nvp, int nb, int *__restrict__ wray0, int *__restrict__ wcnt,
-                            int *__restrict__ woff, int *__restrict__ wtot,
-                            Entry *__restrict__ tlocal, int *__restrict__ wmax)
-{
-    extern __shared__ int sw[];  // [2 * nv]
-    int *lo = sw, *hi = sw + nv;
-    const int tiles_x = (n + kWinTW - 1) / kWinTW;
-    const int tile = blockIdx.x, ty = tile / tiles_x, tx = tile % tiles_x;
-    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-        lo[v] = 0x7fffffff;
-        hi[v] = -1;
-    }
-    __syncthreads();
-    for (int s = 0; s < kWinTH * kWinTW; ++s) {
-        const int i = ty * kWinTH + s / kWinTW, j = tx * kWinTW + s % kWinTW;
-        if (i >= n || j >= n) continue;
-        const int64_t pix = (int64_t)i * n + j;
-        for (int64_t k = colptr[pix] + threadIdx.x; k < colptr[pix + 1]; k += blockDim.x) {
-            const int ray = tent[k].x, v = ray / nb;
-            atomicMin(&lo[v], ray);
-            atomicMax(&hi[v], ray);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int off = 0;
-        for (int v = 0; v < nv; ++v) {
-            int start = 0, cnt = 0;
-            if (hi[v] >= 0) {
-                start = lo[v] & ~1;
-                cnt = ((hi[v] + 2) & ~1) - start;
-            }
-            wray0[(int64_t)tile * nvp + v] = start;
-            wcnt[(int64_t)tile * nvp + v] = cnt;
-            woff[(int64_t)tile * nvp + v] = off;
-            lo[v] = start;
-            hi[v] = off;
-            off += cnt;
-        }
-        for (int v = nv; v < nvp; ++v) {
-            wray0[(int64_t)tile * nvp + v] = 0;
-            wcnt[(int64_t)tile * nvp + v] = 0;
-            woff[(int64_t)tile * nvp + v] = off;
-        }
-        wtot[tile] = off;
-        atomicMax(wmax, off);
-    }
-    __syncthreads();
-    for (int s = 0; s < kWinTH * kWinTW; ++s) {
-        const int i = ty * kWinTH + s / kWinTW, j = tx * kWinTW + s % kWinTW;
-        if (i >= n || j >= n) continue;
-        const int64_t pix = (int64_t)i * n + j;
-        for (int64_t k = colptr[pix] + threadIdx.x; k < colptr[pix + 1]; k += blockDim.x) {
-            const Entry t = tent[k];
-            const int v = t.x / nb;
-            tlocal[k] = make_int2(hi[v] + (t.x - lo[v]), t.y);
-        }
-    }
-}
-
-// Entries of each tile, padded to an even count.
-__global__ void k_tile_count(const int64_t *__restrict__ colptr, int n, int ntiles,
-                             int64_t *__restrict__ cnt)
-{
-    const int tile = blockIdx.x * blockDim.x + threadIdx.x;
-    if (tile >= ntiles) return;
-    const int tiles_x = (n + kWinTW - 1) / kWinTW, ty = tile / tiles_x, tx = tile % tiles_x;
-    int64_t c = 0;
-    for (int s = 0; s < kWinTP; ++s) {
-        const int i = ty * kWinTH + s / kWinTW, j = tx * kWinTW + s % kWinTW;
-        if (i < n && j < n) {
-            const int64_t pix = (int64_t)i * n + j;
-            c += colptr[pix + 1] - colptr[pix];
-        }
-    }
-    cnt[tile] = (c + 1) & ~(int64_t)1;
-}
-
-// Copy each tile's tile-local entries to their tile-major place (one block per tile).
-__global__ void k_tile_fill(const int64_t *__restrict__ colptr, const Entry *__restrict__ tlocal, int n,
-                            const int64_t *__restrict__ tbase, int *__restrict__ tpo,
-                            Entry *__restrict__ tmaj, int *__restrict__ emax)
-{
-    const int tile = blockIdx.x;
-    const int tiles_x = (n + kWinTW - 1) / kWinTW, ty = tile / tiles_x, tx = tile % tiles_x;
-    __shared__ int off[kWinTP + 1];
-    if (threadIdx.x == 0) {
-        int o = 0;
-        for (int s = 0; s < kWinTP; ++s) {
-            off[s] = o;
-            const int i = ty * kWinTH + s / kWinTW, j = tx * kWinTW + s % kWinTW;
-            if (i < n && j < n) {
-                const int64_t pix = (int64_t)i * n + j;
-                o += (int)(colptr[pix + 1] - colptr[pix]);
-            }
-        }
-        off[kWinTP] = o;
-        for (int s = 0; s <= kWinTP; ++s) tpo[(int64_t)tile * (kWinTP + 1) + s] = off[s];
-        if (o & 1) tmaj[tbase[tile] + o] = make_int2(0, 0);
-        atomicMax(emax, (int)(tbase[tile + 1] - tbase[tile]));
-    }
-    __syncthreads();
-    for (int s = 0; s < kWinTP; ++s) {
-        const int i = ty * kWinTH + s / kWinTW, j = tx * kWinTW + s % kWinTW;
-        if (i >= n || j >= n) continue;
-        const int64_t pix = (int64_t)i * n + j;
-        const int64_t b = colptr[pix], len = colptr[pix + 1] - b;
-        for (int64_t k = threadIdx.x; k < len; k += blockDim.x) tmaj[tbase[tile] + off[s] + k] = tlocal[b + k];
-    }
-}
-
 bool geometry_ok(const dect_geometry *g)
 {
     if (!g) return false;
@@ -583,14 +571,14 @@ extern "C" dect_status dect_plan_create(const dect_geometry *geom, int device, d
     int *d_ccnt = nullptr, *d_cursor = nullptr;
     int64_t *d_ccnt64 = nullptr;
     Entry *d_tmp = nullptr;
-    dect_status st = DECT_OK;
+    short *d_col = nullptr;
+    int *d_bad = nullptr;
     auto fail = [&](dect_status code) {
         cudaStreamSynchronize(s);
         cudaFree(d_rays); cudaFree(d_cnt); cudaFree(d_al); cudaFree(d_ccnt);
-        cudaFree(d_cursor); cudaFree(d_ccnt64); cudaFree(d_tmp);
+        cudaFree(d_cursor); cudaFree(d_ccnt64); cudaFree(d_tmp); cudaFree(d_col); cudaFree(d_bad);
         cudaFree(p->rowptr); cudaFree(p->ent); cudaFree(p->colptr); cudaFree(p->tent);
-        cudaFree(p->wray0); cudaFree(p->wcnt); cudaFree(p->woff); cudaFree(p->wtot); cudaFree(p->tlocal);
-        cudaFree(p->tmaj); cudaFree(p->tbase); cudaFree(p->tpo);
+        lines_free(p->lines);
         delete p;
         return code;
     };
@@ -627,7 +615,19 @@ extern "C" dect_status dect_plan_create(const dect_geometry *geom, int device, d
     size_t ne = (size_t)(nnz > 0 ? nnz : 1) + kTablePad;
     PLAN_CUDA(cudaMalloc(&p->ent, sizeof(Entry) * ne));
     PLAN_CUDA(cudaMemsetAsync(p->ent, 0, sizeof(Entry) * ne, s));
-    k_siddon_fill<<<(unsigned)((p->M + T - 1) / T), T, 0, s>>>(d_rays, p->M, g, p->rowptr, p->ent);
+    // the line table, where its form can hold and memory allows
+    if (nnz > 0) {
+        PLAN_CUDA(lines_alloc(p->lines, p->n, p->nv, p->nb, s));
+        const size_t ncol = (size_t)p->nv * p->lines.nblk * p->lines.ngb * 1024;
+        if (p->lines.ok && cudaMalloc(&d_col, sizeof(short) * ncol) != cudaSuccess) {
+            cudaGetLastError();
+            lines_free(p->lines);
+        }
+        PLAN_CUDA(cudaMalloc(&d_bad, sizeof(int)));
+        PLAN_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
+    }
+    k_siddon_fill<<<(unsigned)((p->M + T - 1) / T), T, 0, s>>>(d_rays, p->M, g, p->rowptr, p->ent, p->lines, d_col,
+                                                               d_bad);
     PLAN_CUDA(cudaGetLastError());
 
     // pixel-major transpose
@@ -655,58 +655,16 @@ extern "C" dect_status dect_plan_create(const dect_geometry *geom, int device, d
         k_col_sort<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(p->colptr, p->N, d_tmp, p->tent);
         PLAN_CUDA(cudaGetLastError());
     }
-    // shared-memory windows of the tiled A^T
-    if (p->nv <= kWinMaxViews && nnz > 0) {
-        const int tiles_x = (p->n + kWinTW - 1) / kWinTW, tiles_y = (p->n + kWinTH - 1) / kWinTH;
-        p->win_tiles = tiles_x * tiles_y;
-        p->nvp = (p->nv + 3) & ~3;
-        const size_t tv = (size_t)p->win_tiles * p->nvp;
-        PLAN_CUDA(cudaMalloc(&p->wray0, sizeof(int) * tv));
-        PLAN_CUDA(cudaMalloc(&p->wcnt, sizeof(int) * tv));
-        PLAN_CUDA(cudaMalloc(&p->woff, sizeof(int) * tv));
-        PLAN_CUDA(cudaMalloc(&p->wtot, sizeof(int) * p->win_tiles));
-        PLAN_CUDA(cudaMalloc(&p->tlocal, sizeof(Entry) * ne));
-        PLAN_CUDA(cudaMemsetAsync(p->tlocal, 0, sizeof(Entry) * ne, s));
-        int *d_wmax = d_ccnt;  // reuse a scratch int
-        PLAN_CUDA(cudaMemsetAsync(d_wmax, 0, sizeof(int), s));
-        const size_t sm = sizeof(int) * 2 * p->nv;
-        if (sm > 48 * 1024)
-            PLAN_CUDA(cudaFuncSetAttribute(k_win_build, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        k_win_build<<<p->win_tiles, 256, sm, s>>>(p->colptr, p->tent, p->n, p->nv, p->nvp, p->nb, p->wray0, p->wcnt,
-                                                   p->woff, p->wtot, p->tlocal, d_wmax);
-        PLAN_CUDA(cudaGetLastError());
-        int wmax = 0;
-        PLAN_CUDA(cudaMemcpyAsync(&wmax, d_wmax, sizeof(int), cudaMemcpyDeviceToHost, s));
-        PLAN_CUDA(cudaStreamSynchronize(s));
-        // tile-major copy of the tile-local entries
-        const int nt = p->win_tiles;
-        PLAN_CUDA(cudaMalloc(&p->tbase, sizeof(int64_t) * (nt + 1)));
-        PLAN_CUDA(cudaMalloc(&p->tpo, sizeof(int) * (size_t)nt * (kWinTP + 1)));
-        int64_t *d_tcnt = nullptr;
-        PLAN_CUDA(cudaMalloc(&d_tcnt, sizeof(int64_t) * nt));
-        k_tile_count<<<(nt + 255) / 256, 256, 0, s>>>(p->colptr, p->n, nt, d_tcnt);
-        PLAN_CUDA(cudaGetLastError());
-        PLAN_CUDA(scan_exclusive(d_tcnt, nt, p->tbase, s));
-        int64_t tot = 0;
-        PLAN_CUDA(cudaMemcpyAsync(&tot, p->tbase + nt, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-        PLAN_CUDA(cudaStreamSynchronize(s));
-        cudaFree(d_tcnt);
-        PLAN_CUDA(cudaMalloc(&p->tmaj, sizeof(Entry) * (size_t)(tot + kTablePad)));
-        PLAN_CUDA(cudaMemsetAsync(p->tmaj, 0, sizeof(Entry) * (size_t)(tot + kTablePad), s));
-        PLAN_CUDA(cudaMemsetAsync(d_wmax, 0, sizeof(int), s));
-        k_tile_fill<<<nt, 256, 0, s>>>(p->colptr, p->tlocal, p->n, p->tbase, p->tpo, p->tmaj, d_wmax);
-        PLAN_CUDA(cudaGetLastError());
-        int emax = 0;
-        PLAN_CUDA(cudaMemcpyAsync(&emax, d_wmax, sizeof(int), cudaMemcpyDeviceToHost, s));
-        PLAN_CUDA(cudaStreamSynchronize(s));
-        p->tile_ent_max = emax;
-        p->win_max = wmax;
+    int hbad = 0;
+    if (p->lines.ok) {
+        PLAN_CUDA(lines_finish(p->lines, d_col, d_bad, s));
+        PLAN_CUDA(cudaMemcpyAsync(&hbad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     }
     PLAN_CUDA(cudaStreamSynchronize(s));
+    if (hbad) lines_free(p->lines);
     cudaFree(d_rays); cudaFree(d_cnt); cudaFree(d_al); cudaFree(d_ccnt);
-    cudaFree(d_cursor); cudaFree(d_ccnt64); cudaFree(d_tmp);
+    cudaFree(d_cursor); cudaFree(d_ccnt64); cudaFree(d_tmp); cudaFree(d_col); cudaFree(d_bad);
 #undef PLAN_CUDA
-    (void)st;
     *out = p;
     return DECT_OK;
 }
@@ -900,14 +858,7 @@ extern "C" dect_status dect_plan_destroy(dect_plan *p)
     cudaFree(p->otf_inv);
     cudaFree(p->otf_view);
     cudaFree(p->otf_view2);
-    cudaFree(p->wray0);
-    cudaFree(p->wcnt);
-    cudaFree(p->woff);
-    cudaFree(p->wtot);
-    cudaFree(p->tlocal);
-    cudaFree(p->tmaj);
-    cudaFree(p->tbase);
-    cudaFree(p->tpo);
+    lines_free(p->lines);
     cudaSetDevice(cur);
     delete p;
     return DECT_OK;

@@ -1,15 +1,16 @@
 // A x and A^T y on caller-owned planar batches (Eq. (1); the A^T of G_f in
-// Eq. (9)), through the interleaved table kernels of the ADM: a batch is
-// split into passes of up to 64 images; each pass packs its images
-// pixel-major ([index][NB], zero-padded to the width NB), streams the table
-// once with every entry gathering one contiguous vector of all NB images,
-// and unpacks the result to the planar output.
+// Eq. (9)).  A batch is split into passes of up to 64 images; each pass packs its
+// images pixel-major ([index][NB], zero-padded to the width NB), streams the
+// table once with every entry gathering one contiguous vector of all NB images,
+// and unpacks the result to the planar output.  A of narrow passes streams the
+// line table instead (lines.cuh), whose kernel writes the planar result itself.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "dect_internal.cuh"
 #include "kernels.cuh"
+#include "lines.cuh"
 
 namespace dect {
 namespace {
@@ -125,11 +126,106 @@ cudaError_t run_batched(const int64_t *ptr, const Entry *ent, int64_t rows_in, i
     return e != cudaSuccess ? e : f;
 }
 
+// ---------------------------------------------------------------------------
+// A on the line table
+// ---------------------------------------------------------------------------
+// planar src [nimg][n][n] -> interleaved dst and its transpose dstT (images >= nimg are 0)
+template <int NB>
+__global__ void __launch_bounds__(256) k_line_pack(const float *__restrict__ src, float *__restrict__ dst,
+                                                   float *__restrict__ dstT, int n, int nimg)
+{
+    constexpr int VW = Batch<NB>::VW;
+    __shared__ float tile[VW][32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, j0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
+    const int64_t N = (int64_t)n * n;
+    for (int k = 0; k < NB; k += VW) {
+        for (int r = ty; r < 32; r += 8)
+            if (i0 + r < n && j0 + tx < n) {
+                const int64_t p = (int64_t)(i0 + r) * n + j0 + tx;
+                Vec<VW> v;
+#pragma unroll
+                for (int c = 0; c < VW; ++c) {
+                    v.v[c] = k + c < nimg ? src[(int64_t)(k + c) * N + p] : 0.f;
+                    tile[c][r][tx] = v.v[c];
+                }
+                st_v<VW>(dst + p * NB + k, v);
+            }
+        __syncthreads();
+        for (int r = ty; r < 32; r += 8)
+            if (j0 + r < n && i0 + tx < n) {
+                Vec<VW> v;
+#pragma unroll
+                for (int c = 0; c < VW; ++c) v.v[c] = tile[c][tx][r];
+                st_v<VW>(dstT + ((int64_t)(j0 + r) * n + i0 + tx) * NB + k, v);
+            }
+        __syncthreads();
+    }
+}
+
+// y[img][ray] = (A x)(ray): a block per group of 32 rays
+template <int NB>
+__global__ void __launch_bounds__(LineShape<NB>::BLOCK, LineShape<NB>::BLOCKS)
+    k_line_project(LineTable T, const float *__restrict__ x, const float *__restrict__ xT, float *__restrict__ y, int nimg)
+{
+    __shared__ LineSums<NB> sm;
+    const int64_t M = (int64_t)T.nv * T.nb;
+    const int v = blockIdx.x / T.ngb, gb = blockIdx.x % T.ngb;
+    float acc[LineShape<NB>::VW];
+    line_ray_sums<NB>(T, v, gb, x, xT, acc);
+    line_ray_store<NB>(sm, acc);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 32 * NB; e += LineShape<NB>::BLOCK) {
+        const int r = e & 31, k = e >> 5;
+        if (gb * 32 + r >= T.nb || k >= nimg) continue;
+        const int64_t ray = (int64_t)v * T.nb + gb * 32 + r;
+        y[(int64_t)k * M + ray] = line_ray_value<NB>(sm, r * NB + k, __ldg(T.len + ray));
+    }
+}
+
+template <int NB>
+void line_pass(const LineTable &T, const float *x, float *y, int nimg, float *buf, cudaStream_t s)
+{
+    const int64_t N = (int64_t)T.n * T.n;
+    k_line_pack<NB><<<transpose_grid(T.n), 256, 0, s>>>(x, buf, buf + N * NB, T.n, nimg);
+    k_line_project<NB><<<line_groups(T), LineShape<NB>::BLOCK, 0, s>>>(T, buf, buf + N * NB, y, nimg);
+    count_launches(2);
+}
+
+// A of up to kLineMaxImages images
+cudaError_t run_lines(const LineTable &T, const float *x, float *y, int batch, cudaStream_t s)
+{
+    int width = 2;
+    while (width < batch) width *= 2;
+    float *buf = nullptr;
+    cudaError_t e = cudaMallocAsync((void **)&buf, sizeof(float) * 2 * (size_t)T.n * T.n * width, s);
+    if (e != cudaSuccess) return e;
+    switch (width) {
+    case 2: line_pass<2>(T, x, y, batch, buf, s); break;
+    case 4: line_pass<4>(T, x, y, batch, buf, s); break;
+    case 8: line_pass<8>(T, x, y, batch, buf, s); break;
+    default: line_pass<16>(T, x, y, batch, buf, s); break;
+    }
+    e = cudaGetLastError();
+    const cudaError_t f = cudaFreeAsync(buf, s);
+    return e != cudaSuccess ? e : f;
+}
+
+// images of a batch that A takes through the line table: the last pass, where it is narrow enough
+int line_tail(const dect_plan *p, int batch)
+{
+    const int rest = batch % kMaxBatchImages;
+    return p->lines.ok && rest <= kLineMaxImages ? rest : 0;
+}
+
 }  // namespace
 
 cudaError_t launch_project_planar(const dect_plan *p, const float *x, float *y, int batch, cudaStream_t s)
 {
-    return run_batched(p->rowptr, p->ent, p->N, p->M, p->n, std::max(p->nz, 1), false, x, y, batch, s);
+    const int tail = line_tail(p, batch), head = batch - tail;
+    cudaError_t e = cudaSuccess;
+    if (head > 0) e = run_batched(p->rowptr, p->ent, p->N, p->M, p->n, std::max(p->nz, 1), false, x, y, head, s);
+    if (e == cudaSuccess && tail > 0) e = run_lines(p->lines, x + head * p->N, y + head * p->M, tail, s);
+    return e;
 }
 
 cudaError_t launch_backproject_planar(const dect_plan *p, const float *y, float *x, int batch, cudaStream_t s)
