@@ -536,13 +536,14 @@ dect_status dect_plan_set_fwd_tuning(dect_plan *plan, int images, int choice);
  *     streams the rows (f, G, the multiplier) into a ring of four
  *     shared-memory stages with 1-D bulk copies (TMA) completing on
  *     mbarriers, the other warps compute from shared memory, no block
- *     barrier per row; 4 or more channels only (otherwise 0 is used).
- * Both give the same images (the same per-pixel arithmetic); the FP32
+ *     barrier per row; 4 or more channels only (otherwise 0 is used),
+ *   2 a thread per pixel and four channels, which steps its two neighbours again.
+ * All give the same images (the same per-pixel arithmetic); the FP32
  * partial sums of the two norms are taken in a different order.  Timed
  * before the first iteration of the first ADM call with that width, where
  * the step changes nothing.  Host memory: us has DECT_TV_VARIANTS elements.
  */
-#define DECT_TV_VARIANTS 2
+#define DECT_TV_VARIANTS 3
 dect_status dect_plan_get_tv_tuning(const dect_plan *plan, int images, int *choice,
                                     float us[DECT_TV_VARIANTS]);
 

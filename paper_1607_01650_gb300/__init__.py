@@ -435,7 +435,7 @@ def fbp(plan: Plan, m, x=None, stream=None):
 BB1, CAUCHY = 0, 1
 BWD_VARIANTS = 8                        # DECT_BWD_VARIANTS in include/dect.h
 FWD_VARIANTS = 4                        # DECT_FWD_VARIANTS in include/dect.h
-TV_VARIANTS = 2                         # DECT_TV_VARIANTS in include/dect.h
+TV_VARIANTS = 3                         # DECT_TV_VARIANTS in include/dect.h
 
 
 @dataclasses.dataclass

@@ -605,6 +605,63 @@ __global__ void __launch_bounds__(TvTmaShape<NB>::THREADS) k_tv_tma(
     reduce_images<NB, 2, S::BLK>(acc, part_of<NB>(D, C_TV), D.red + R_TV * NB, D.ctr + C_TV, rsm);
 }
 
+// The same TV step, a thread per pixel vector (TV variant 2): the neighbours
+// above and to the left are read and stepped again instead of handed over.
+// For narrow batches, whose image the L2 holds and whose tiles are too few to
+// fill the SMs (96 at 512^2 and two channels, 17 rows with a block barrier each:
+// 19 to 25 us; this one 10 us at 128^2, 19 at 512^2).  Same arithmetic per pixel,
+// so the same images.
+template <int NB, bool JOINT>
+__global__ void __launch_bounds__(kBlock) k_tv_px(const float *__restrict__ f_in, float *__restrict__ f_out,
+                                                  const float *__restrict__ G, float *__restrict__ lam,
+                                                  float *__restrict__ z, float *__restrict__ p, float *__restrict__ r,
+                                                  const float *__restrict__ q, AdmConst C, AdmDev D, int final_pass)
+{
+    constexpr int VW = Batch<NB>::VW, CPB = Batch<NB>::CPB;
+    __shared__ double smem[reduce_smem_doubles<NB, kBlock>(2)];
+    const int k = *D.k, vl = threadIdx.x % CPB;
+    const float inv_rho = 1.0f / C.rho;
+    const bool clamp = C.nonneg && k > 0;
+    Vec<VW> a, acc[2];
+#pragma unroll
+    for (int c = 0; c < VW; ++c) a.v[c] = (float)D.alpha[vl * VW + c];
+    acc[0].zero();
+    acc[1].zero();
+    const int64_t sN = C.N * NB, row = (int64_t)C.n * NB, tot = C.N * CPB;
+    const float *lsrc = C.xi_is_rho ? p : lam;
+    const int64_t first = (int64_t)blockIdx.x * kBlock + threadIdx.x, stride = (int64_t)gridDim.x * kBlock;
+    for (int64_t t = first; t < tot; t += stride) {
+        const int64_t pix = t / CPB, o = pix * NB + vl * VW;
+        const int i = (int)((unsigned)pix / (unsigned)C.n), j = (int)((unsigned)pix % (unsigned)C.n);
+        auto step = [&](int64_t at, const Vec<VW> &g) {
+            Vec<VW> f = ld_v<VW>(f_in + at);
+#pragma unroll
+            for (int c = 0; c < VW; ++c) f.v[c] = nonneg_step(f.v[c], a.v[c], g.v[c], clamp);
+            return f;
+        };
+        const Vec<VW> gc = ld_v<VW>(G + o), fc = step(o, gc);
+        Vec<VW> gu = gc, fu = fc, gl = gc, fl = fc, l0, l1;
+        if (i > 0) {
+            gu = ld_v<VW>(G + o - row);
+            fu = step(o - row, gu);
+        }
+        if (j > 0) {
+            gl = ld_v<VW>(G + o - NB);
+            fl = step(o - NB, gl);
+        }
+        l0.zero();
+        l1.zero();
+        if (!final_pass) {
+            l0 = ld_v<VW>(lsrc + o);
+            l1 = ld_v<VW>(lsrc + sN + o);
+        }
+        st_v<VW>(f_out + o, fc);
+        tv_pixel<NB, JOINT>(fc, gc, fu, gu, fl, gl, l0, l1, i, j, o, sN, a, k, inv_rho, C, final_pass, lam, z, p, acc[0]);
+    }
+    r_step<VW>(r, q, C.nonneg ? 0 : C.M * CPB, first, stride, a, acc[1]);
+    reduce_images<NB, 2, kBlock>(acc, part_of<NB>(D, C_TV), D.red + R_TV * NB, D.ctr + C_TV, smem);
+}
+
 // G = mu A^T r + grad^T p over the pixel-major table.  A block of BLK
 // threads takes TW x TH pixel tiles (BLK / G_ pixels at a time), so the
 // sinogram lines its pixels gather are shared in L1.
@@ -1254,8 +1311,8 @@ cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
 
 // TV-step variants (autotuner candidates): 0 k_tv (tiles claimed from a
 // counter, rows exchanged through shared memory, one barrier per row); 1
-// k_tv_tma (rows streamed by bulk copies into a ring of stages, NB >= 4).
-// Both give the same images.
+// k_tv_tma (rows streamed by bulk copies into a ring of stages, NB >= 4); 2
+// k_tv_px (a thread per pixel vector).  All give the same images.
 constexpr int kTvVariants = DECT_TV_VARIANTS;
 
 // Prepare k_tv_tma for this width: its shared memory, and the grid (blocks
@@ -1295,7 +1352,7 @@ cudaError_t tune_tv(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t
     const int idx = nb_index<NB>();
     const bool tma_ok = NB >= 4 && W.tv_grid > 0;
     if (P->tv_choice[idx] >= 0) {
-        W.tv = (P->tv_choice[idx] == 1 && tma_ok) ? 1 : 0;
+        W.tv = P->tv_choice[idx] == 1 && !tma_ok ? 0 : P->tv_choice[idx];
         return cudaSuccess;
     }
     cudaEvent_t a = nullptr, b = nullptr;
@@ -1350,6 +1407,16 @@ void launch_tv(const Work &W, const AdmConst &C, int par, int final_pass, cudaSt
                                                                            W.p, W.r, W.q, C, W.D, final_pass);
             return;
         }
+    }
+    if (W.tv == 2) {
+        const int grid = (int)std::min<int64_t>((C.N * Batch<NB>::CPB + kBlock - 1) / kBlock, kGrid);
+        if (C.joint)
+            k_tv_px<NB, true><<<grid, kBlock, 0, s>>>(W.f[par], W.f[1 - par], W.G, W.lam, W.z, W.p, W.r, W.q, C, W.D,
+                                                      final_pass);
+        else
+            k_tv_px<NB, false><<<grid, kBlock, 0, s>>>(W.f[par], W.f[1 - par], W.G, W.lam, W.z, W.p, W.r, W.q, C, W.D,
+                                                       final_pass);
+        return;
     }
     using S = TvShape<NB>;
     const int ntiles = ((C.n + S::W - 1) / S::W) * ((C.n + S::H - 1) / S::H);

@@ -147,10 +147,13 @@ __host__ __device__ constexpr int red_slots()
     return (BLOCK / 32) % 8 == 0 ? 8 : BLOCK / 32;
 }
 
+// threads that share an image's grid total: one thread adding the partials of
+// a thousand blocks would be most of a narrow batch's launch
 template <int NB, int BLOCK>
 __host__ __device__ constexpr int red_split()
 {
-    return BLOCK / NB < 8 ? BLOCK / NB : 8;
+    constexpr int most = 256 / NB < 8 ? 8 : 256 / NB;
+    return BLOCK / NB < most ? BLOCK / NB : most;
 }
 
 template <int NB, int BLOCK = 256>
@@ -166,7 +169,7 @@ __device__ __forceinline__ bool reduce_images(Vec<Batch<NB>::VW> (&v)[K], double
 {
     constexpr int VW = Batch<NB>::VW, CPB = Batch<NB>::CPB;
     constexpr int NW = BLOCK / 32, SL = red_slots<BLOCK>(), SPLIT = red_split<NB, BLOCK>();
-    static_assert(NW % SL == 0 && BLOCK % NB == 0, "reduce_images: block shape");
+    static_assert(NW % SL == 0 && BLOCK % NB == 0 && (SPLIT & (SPLIT - 1)) == 0, "reduce_images: block shape");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t pstride = (size_t)gridDim.x * NB;
 #pragma unroll
@@ -201,7 +204,7 @@ __device__ __forceinline__ bool reduce_images(Vec<Batch<NB>::VW> (&v)[K], double
     if (!last) return false;
     __threadfence();
     // grid total: SPLIT threads per image each sum a fixed stride of the block
-    // partials, then one thread per image adds the SPLIT sub-sums in order
+    // partials, then the SPLIT sub-sums are added pairwise, halving
     const int img = threadIdx.x % NB, sub = threadIdx.x / NB;
     double sv[K];
 #pragma unroll
@@ -217,12 +220,16 @@ __device__ __forceinline__ bool reduce_images(Vec<Batch<NB>::VW> (&v)[K], double
 #pragma unroll
         for (int q = 0; q < K; ++q) smem[(q * SPLIT + sub) * NB + img] = sv[q];
     __syncthreads();
-    if (threadIdx.x < K * NB) {
-        const int q = threadIdx.x / NB, im = threadIdx.x % NB;
-        double t = 0.0;
-        for (int u = 0; u < SPLIT; ++u) t += smem[(q * SPLIT + u) * NB + im];
-        out[q * NB + im] = t;
+#pragma unroll 1
+    for (int half = SPLIT / 2; half > 0; half >>= 1) {
+        if (sub < half)
+#pragma unroll
+            for (int q = 0; q < K; ++q) smem[(q * SPLIT + sub) * NB + img] += smem[(q * SPLIT + sub + half) * NB + img];
+        __syncthreads();
     }
+    if (sub == 0)
+#pragma unroll
+        for (int q = 0; q < K; ++q) out[q * NB + img] = smem[q * SPLIT * NB + img];
     if (threadIdx.x == 0) *counter = 0u;
     __syncthreads();
     return true;
