@@ -1093,8 +1093,12 @@ __global__ void k_repack_scalars(AdmDev D, AdmDev D2, const int *__restrict__ ma
 // ---------------------------------------------------------------------------
 template <int NB>
 struct Kern {
-    static constexpr int GB = NB >= 32 ? 32 : 16;  // lanes per pixel row
-    static constexpr int GF = 32;                  // lanes per ray row
+    // lanes per pixel row: eight on narrow batches, so that a warp's four
+    // adjacent pixels gather from the same cache lines (A^T at two channels, 512^2
+    // / 60 views: 72 us, with 16 lanes 80); at 16 channels sixteen (128^2: 25 us,
+    // with eight 29 to 34)
+    static constexpr int GB = NB >= 32 ? 32 : NB == 16 ? 16 : 8;
+    static constexpr int GF = 32;  // lanes per ray row (eight: 126 against 110 us at 8 channels)
 };
 
 // A variants: 0-2 the CSR table, one 1024-thread block per SM, a warp per ray:
@@ -1160,10 +1164,11 @@ void launch_residual_check(const dect_plan *P, const Work &W, const float *f_cur
     count_launches(1);
 }
 
-// A^T variants (autotuner candidates): 0-2 L1-cached gather with 4x4 / 8x8 /
-// 16x16 pixel tiles per 256-thread block; 3 none (1 takes its place); 4-5 L1-cached gather with one 1024-thread block per SM over tiles of two
-// or four block steps (8 x 8 / 16 x 8 pixels at 32 lanes per pixel, 8 x 16 /
-// 16 x 16 at 16), whose lines then stay in one L1; 6-7 lanes gather 8
+// A^T variants (autotuner candidates): 0-2 L1-cached gather with 4x4 (4x8 up to
+// 8 channels) / 8x8 / 16x16 pixel tiles per 256-thread block; 3 none (1 takes
+// its place); 4-5 L1-cached gather with one 1024-thread block per SM over tiles
+// of two or four block steps (8 x 8 / 16 x 8 pixels at 32 lanes per pixel, 8 x 16
+// / 16 x 16 at 16, 8 x 32 / 16 x 32 at 8), whose lines then stay in one L1; 6-7 lanes gather 8
 // images of an entry (row_dot_w, NB >= 16 only): 6 with the lanes and tiles
 // of 4; 7 with 16 lanes per pixel (two pixels per warp) over 8 x 8 tiles.
 constexpr int kBwdVariants = DECT_BWD_VARIANTS;
@@ -1176,7 +1181,8 @@ void launch_bwd(const dect_plan *P, const Work &W, const AdmConst &C, int varian
     float *GT = W.fwd == kFwdLines ? W.GT : nullptr;
     switch (variant) {
     case 0:
-        k_bwd<NB, GB, 4, 4, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
+        k_bwd<NB, GB, 4, (kBlock / GB > 16 ? kBlock / GB / 4 : 4), kBlock>
+            <<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);
         break;
     case 2:
         k_bwd<NB, GB, 16, 16, kBlock><<<kGrid, kBlock, 0, s>>>(P->colptr, P->tent, W.r, W.p, W.G, C, W.D, GT);

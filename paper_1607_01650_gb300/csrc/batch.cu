@@ -22,8 +22,8 @@
 // view parameters are computed in FP64 and stored in FP32.
 //
 // The multi-slice ADM also runs on the plans' stored tables instead
-// (dect_adm_tv_batch_ex with DECT_PROJ_TABLE): a warp per ray of the
-// ray-major table for A, a warp per pixel of the pixel-major table for A^T
+// (dect_adm_tv_batch_ex with DECT_PROJ_TABLE): eight lanes per ray of the
+// ray-major table for A, eight per pixel of the pixel-major table for A^T
 // (the row kernels of the single-plan ADM at two channels).
 //
 // Multi-slice ADM.  Each slice (both energies interleaved, [pixel][2])
@@ -285,10 +285,12 @@ cudaError_t otf_operator(const dect_plan *P, const float *src, float *dst, int b
 // Multi-slice ADM
 // ---------------------------------------------------------------------------
 enum { PH_TV = 0, PH_BWD = 1, PH_FWD = 2, PH_COUNT = 3 };
-// stored-table projector: a warp per ray of the ray-major table (A) and per
-// pixel of the pixel-major table (A^T, the warps of a block taking turns
-// over the block's 16 x 16 tile, whose pixels share sinogram lines in L1)
-constexpr int kTabRaysPerBlock = kOtfBlock / 32;
+// stored-table projector: eight lanes per ray of the ray-major table (A) and per
+// pixel of the pixel-major table (A^T, the lanes of a block taking turns over
+// the block's 16 x 16 tile, whose pixels share sinogram lines in L1); a warp's
+// four adjacent rows gather from the same cache lines
+constexpr int kTabLanes = 8;
+constexpr int kTabRaysPerBlock = kOtfBlock / kTabLanes;
 enum { Q_TV = 0, Q_RR = 1, Q_DD = 2, Q_QQ = 3, Q_GG = 4, Q_COUNT = 5 };
 
 struct SliceDesc {
@@ -519,7 +521,7 @@ __device__ __forceinline__ void bwd_finish(const SliceDesc &d, const BatchConst 
 }
 
 // G = mu A^T r + grad^T p per pixel of the block's 16 x 16 tile; |G|^2 per
-// channel.  TABLE: A^T r from the pixel-major table (a warp per pixel, the
+// channel.  TABLE: A^T r from the pixel-major table (eight lanes per pixel, the
 // block's warps taking the tile's pixels in turn); otherwise on the fly (a
 // thread per pixel).
 template <bool TABLE>
@@ -531,10 +533,10 @@ __global__ void __launch_bounds__(kOtfBlock) k_bwd_m(const SliceDesc *__restrict
     const int n = d.G.g.n, lb = blockIdx.x - d.blk0[PH_BWD];
     float acc[1][2] = {{0.f, 0.f}};
     if constexpr (TABLE) {
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int lr = threadIdx.x % kTabLanes;
         const int tx = (n + kOtfTile - 1) / kOtfTile;
         const int i0 = (lb / tx) * kOtfTile, j0 = (lb % tx) * kOtfTile;
-        for (int k = warp; k < kOtfTile * kOtfTile; k += kOtfBlock / 32) {
+        for (int k = threadIdx.x / kTabLanes; k < kOtfTile * kOtfTile; k += kTabRaysPerBlock) {
             const int i = i0 + k / kOtfTile, j = j0 + k % kOtfTile;
             const bool ok = i < n && j < n;
             int64_t b = 0, e = 0;
@@ -542,9 +544,9 @@ __global__ void __launch_bounds__(kOtfBlock) k_bwd_m(const SliceDesc *__restrict
                 b = d.colptr[(int64_t)i * n + j];
                 e = d.colptr[(int64_t)i * n + j + 1];
             }
-            const Vec<2> a = row_dot<2, 32, true>(d.tent, b, e, reinterpret_cast<const float *>(d.r), d.M, lane,
-                                                 CHK_GATHER_AT);
-            if (ok && lane == 0) bwd_finish(d, C, i, j, make_float2(a.v[0], a.v[1]), acc);
+            const Vec<2> a = row_dot<2, kTabLanes, true>(d.tent, b, e, reinterpret_cast<const float *>(d.r), d.M, lr,
+                                                         CHK_GATHER_AT);
+            if (ok && lr == 0) bwd_finish(d, C, i, j, make_float2(a.v[0], a.v[1]), acc);
         }
     } else {
         int i, j;
@@ -612,7 +614,7 @@ __device__ void slice_finish(int s, const BatchConst &C, const BatchDev &B)
 // slice's step.  MODE 0: r = A f - beta m.  MODE 2: the same and |r|^2
 // (projected f-step).  MODE 3: |A f - beta m|^2 and |r - (A f - beta m)|^2
 // (check of the carried residual, into QQ and GG).
-// TABLE: q (or A f) from the ray-major table, a warp per ray; otherwise on
+// TABLE: q (or A f) from the ray-major table, eight lanes per ray; otherwise on
 // the fly, a thread per ray.
 template <int MODE, bool TABLE>
 __global__ void __launch_bounds__(kOtfBlock) k_fwd_m(const SliceDesc *__restrict__ SD, const int *__restrict__ bmap,
@@ -636,16 +638,16 @@ __global__ void __launch_bounds__(kOtfBlock) k_fwd_m(const SliceDesc *__restrict
     float2 v = make_float2(0.f, 0.f);
     bool mine;  // this thread holds the ray's sum
     if constexpr (TABLE) {
-        ray = (int64_t)lb * kTabRaysPerBlock + (threadIdx.x >> 5);
+        ray = (int64_t)lb * kTabRaysPerBlock + threadIdx.x / kTabLanes;
         int64_t b = 0, e = 0;
         if (ray < d.M) {
             b = d.rowptr[ray];
             e = d.rowptr[ray + 1];
         }
-        const Vec<2> a = row_dot<2, 32, true>(d.ent, b, e, reinterpret_cast<const float *>(src), d.N,
-                                             threadIdx.x & 31, CHK_GATHER_A);
+        const Vec<2> a = row_dot<2, kTabLanes, true>(d.ent, b, e, reinterpret_cast<const float *>(src), d.N,
+                                                     threadIdx.x % kTabLanes, CHK_GATHER_A);
         v = make_float2(a.v[0], a.v[1]);
-        mine = ray < d.M && (threadIdx.x & 31) == 0;
+        mine = ray < d.M && threadIdx.x % kTabLanes == 0;
     } else {
         ray = (int64_t)lb * kOtfBlock + threadIdx.x;
         mine = ray < d.M;
@@ -779,7 +781,7 @@ int tiles_of(int n) { return ((n + kOtfTile - 1) / kOtfTile) * ((n + kOtfTile - 
 
 // Block maps of the three phases for the slices with `on[s]`; writes each
 // slice's first block and block count into its descriptor.  table: the
-// forward phase takes a warp per ray.
+// forward phase takes eight lanes per ray.
 void build_maps(std::vector<SliceDesc> &desc, const std::vector<char> &on, std::vector<int> (&map)[PH_COUNT],
                 bool table)
 {

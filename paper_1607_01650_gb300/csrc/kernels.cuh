@@ -298,6 +298,12 @@ __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_g(const Entry *__restrict_
             // gathers in flight, then their multiply-adds
             constexpr int NR = G / EG, R = NR < 8 ? NR : 8;
             static_assert(NR <= 8 || NR % 8 == 0, "rounds must split into groups of 8");
+            // a lane of a short split sums many entries: the step's are summed by
+            // themselves first, so that the running sum is rounded once a step
+            // (error of A and A^T no larger than with a warp per row)
+            constexpr bool PART = G <= 8;
+            const Vec<VW> run = acc;
+            if constexpr (PART) acc.zero();
 #pragma unroll
             for (int u = 0; u < U; ++u) {
 #pragma unroll
@@ -319,6 +325,9 @@ __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_g(const Entry *__restrict_
                         for (int c = 0; c < VW; ++c) acc.v[c] = fmaf(w[j], xv[j].v[c], acc.v[c]);
                 }
             }
+            if constexpr (PART)
+#pragma unroll
+                for (int c = 0; c < VW; ++c) acc.v[c] += run.v[c];
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) cur[u] = nxt[u];

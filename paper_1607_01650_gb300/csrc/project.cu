@@ -16,7 +16,15 @@ namespace dect {
 namespace {
 
 constexpr int kOpBlock = 1024;  // one block per SM
-constexpr int kTile = 8;        // A^T: 8 x 8 pixel tiles, so a tile's sinogram lines stay in one L1
+// Lanes per row (ray or pixel).  Narrow passes are bound by the cache lines that
+// a warp's gathers touch: with 8 lanes a warp takes four adjacent rows, whose
+// entries meet the same lines (A^T of two images at 512^2 / 60 views: 117 -> 65
+// us against a warp per row; 4 lanes 64 us, but 20 % slower on small images;
+// cone-beam 256^2 x 64, 60 views of 64 x 368, one volume: A 1275 -> 971 us, A^T
+// 1821 -> 974; 16 volumes 3485 -> 3382 and 3864 -> 2759).
+template <int NB>
+constexpr int kLanes = NB <= 16 ? 8 : 32;
+constexpr int kTileW = 8;  // A^T: tiles of 8 columns, so a tile's sinogram lines stay in one L1
 
 // planar src [nimg][rows] -> interleaved dst [rows][NB] (images >= nimg are 0)
 template <int NB>
@@ -40,22 +48,23 @@ __global__ void k_from_il(const float *__restrict__ src, float *__restrict__ dst
     if (img < nimg) dst[(int64_t)img * rows + row] = src[t];
 }
 
-// dst[row][NB] = sum over the row's entries of len * src[index][NB].  A warp
-// per row (G = 32 lanes).  TILED (pixel-major table of an n x n image): the
-// block's consecutive rows walk 8 x 8 pixel tiles, so that pixels sharing
-// rays share an L1; otherwise rows are taken in order (adjacent rays of a
-// view share pixels).  Lanes gather 8 images of an entry at 16 or more
-// images (row_dot_w), 4 below (row_dot_g).
+// dst[row][NB] = sum over the row's entries of len * src[index][NB], kLanes
+// lanes per row.  TILED (pixel-major table of an n x n image): the block's
+// consecutive rows walk pixel tiles of 8 columns, so that pixels sharing rays
+// share an L1; otherwise rows are taken in order (adjacent rays of a view share
+// pixels).  Lanes gather 8 images of an entry above 16 images (row_dot_w), 4
+// below (row_dot_g).
 template <int NB, bool TILED>
 __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict__ ptr, const Entry *__restrict__ ent,
                                                       int64_t rows, int n, int nz, const float *__restrict__ src,
                                                       int64_t src_rows, float *__restrict__ dst)
 {
-    constexpr int G = 32, VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
+    constexpr int G = kLanes<NB>, VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
+    constexpr int TW = kTileW, TH = kOpBlock / G > 64 ? kOpBlock / G / TW : 8;
     const int lr = threadIdx.x % G, grp = lr / LPE, vl = lr % LPE;
     const int64_t rpb = kOpBlock / G;
-    const int tiles_x = (n + kTile - 1) / kTile;
-    const int64_t per_slice = (int64_t)tiles_x * tiles_x * kTile * kTile;
+    const int tiles_x = (n + TW - 1) / TW, tiles_y = (n + TH - 1) / TH;
+    const int64_t per_slice = (int64_t)tiles_x * tiles_y * TW * TH;
     const int64_t vrows = TILED ? per_slice * nz : rows;
     const unsigned long long pol = l2_evict_last_policy();
     for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
@@ -64,9 +73,9 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
         bool ok = v < vrows;
         if (TILED && ok) {  // slice k, tile of the slice, pixel of the tile
             const int64_t k = v / per_slice, vs = v % per_slice;
-            const int64_t tile = vs / (kTile * kTile);
-            const int w = (int)(vs % (kTile * kTile));
-            const int i = (int)(tile / tiles_x) * kTile + w / kTile, j = (int)(tile % tiles_x) * kTile + w % kTile;
+            const int64_t tile = vs / (TW * TH);
+            const int w = (int)(vs % (TW * TH));
+            const int i = (int)(tile / tiles_x) * TH + w / TW, j = (int)(tile % tiles_x) * TW + w % TW;
             ok = i < n && j < n;
             row = (k * n + i) * n + j;
         }
@@ -76,7 +85,7 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
             e = ptr[row + 1];
         }
         Vec<VW> acc;
-        if constexpr (NB >= 16)
+        if constexpr (NB > 16)
             acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
         else
             acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, TILED ? CHK_GATHER_AT : CHK_GATHER_A);

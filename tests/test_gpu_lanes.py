@@ -1,0 +1,33 @@
+"""Rows of eight lanes (cone-beam A and A^T of narrow batches) against the oracle (GPU).
+
+Sizes around the 8 x 16 pixel tiles of A^T and the rows of one block, at every
+batch width the kernels are built for.  Tolerance 1e-5 relative L2, that of the
+projector tests.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1607_01650_gb300 as dect  # noqa: E402
+
+
+@pytest.mark.parametrize("n,nz,nr,nc", [(7, 2, 3, 11), (16, 1, 1, 33), (17, 3, 4, 29)])
+@pytest.mark.parametrize("batch", [1, 2, 4, 5, 8, 15, 16, 17])
+def test_cone_operators_match_oracle(n, nz, nr, nc, batch):
+    g = synth.ConeGeometry(n=n, nz=nz, px=1.0, pz=1.3, nv=9, nr=nr, nc=nc, pu=1.3, pv=1.7, sod=60.0,
+                           sdd=130.0, start=0.2, off_u=0.15)
+    plan, t = dect.ConePlan(g), oracle.table3(g)
+    rng = np.random.default_rng(batch)
+    x = rng.standard_normal((batch, nz, n, n)).astype(np.float32)
+    y = rng.standard_normal((batch, g.nv, nr, nc)).astype(np.float32)
+    p = dect.project_cone(plan, torch.tensor(x, device="cuda")).cpu().numpy()
+    b = dect.backproject_cone(plan, torch.tensor(y, device="cuda")).cpu().numpy()
+    for k in range(batch):
+        for got, want in ((p[k], oracle.project3(t, x[k].astype(np.float64))),
+                          (b[k], oracle.backproject3(t, y[k].astype(np.float64)))):
+            assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
