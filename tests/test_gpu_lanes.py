@@ -2,7 +2,10 @@
 
 Sizes around the 8 x 16 pixel tiles of A^T and the rows of one block, at every
 batch width the kernels are built for.  Tolerance 1e-5 relative L2, that of the
-projector tests.
+projector tests.  The sums of A and A^T of narrow fan-beam batches carry their
+rounding errors along: what remains is the rounding of the result (2^-23 / sqrt(12)
+of its power of two, at most 3.5e-8) and of the 200 to 400 entries' lengths and
+partial sums, less than as much again: 5e-8 together, rms.
 """
 import numpy as np
 import pytest
@@ -31,3 +34,33 @@ def test_cone_operators_match_oracle(n, nz, nr, nc, batch):
         for got, want in ((p[k], oracle.project3(t, x[k].astype(np.float64))),
                           (b[k], oracle.backproject3(t, y[k].astype(np.float64)))):
             assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("batch", [1, 7, 14])
+def test_narrow_sums_carry_their_rounding(batch):
+    g = synth.tiny_geometry(n=256, nv=120, nb=370, px=1.0, sod=700.0, sdd=1400.0)
+    plan, t = dect.Plan(g), oracle.table(g)
+    rng = np.random.default_rng(batch)
+    x = rng.uniform(0.5, 1.5, (batch, g.n, g.n)).astype(np.float32)
+    y = rng.uniform(0.5, 1.5, (batch, g.nv, g.nb)).astype(np.float32)
+    p = dect.project(plan, torch.tensor(x, device="cuda")).cpu().numpy()
+    b = dect.backproject(plan, torch.tensor(y, device="cuda")).cpu().numpy()
+    for k in range(0, batch, 3):
+        for got, want in ((p[k], oracle.project(t, x[k].astype(np.float64))),
+                          (b[k], oracle.backproject(t, y[k].astype(np.float64)))):
+            assert np.linalg.norm(got - want) <= 5e-8 * np.linalg.norm(want)
+
+
+def test_infinite_pixel_keeps_its_sign():
+    g = synth.tiny_geometry(n=48, nv=20, nb=70, px=1.0, sod=100.0, sdd=200.0)
+    plan = dect.Plan(g)
+    x = torch.ones((1, 48, 48), device="cuda")
+    clean = dect.project(plan, x)
+    x[0, 20, 27] = float("-inf")
+    y = dect.project(plan, x)
+    hit = y != clean
+    assert hit.any() and bool((y[hit] == float("-inf")).all())
+    r = clean.clone()
+    r[0, 3, 35] = float("inf")
+    b = dect.backproject(plan, r)
+    assert not torch.isnan(b).any() and bool((b == float("inf")).any())
