@@ -967,26 +967,43 @@ __global__ void __launch_bounds__(kWgThreads, 1)
 
 // dW (flat [Cout][Cin_real][3][3]) = sum over blocks k of part[k][g][row][co]
 // (fixed order), row = (slot % 4) * 32 + channel, slot = tap * ncb + ci / 32.
-__global__ void k_wgrad_tc_reduce(const float *part, int nparts, int ngroups, int N, int ncb, int Cin_real,
-                                  float *dW)
+// As in k_wgrad_reduce, a block takes 32 elements and 8 slices of the partials: a
+// thread per element (48 blocks for 32 -> 32 channels) walked its 152 partials
+// one load after the other, 28 us; now 7.  The sums take two FP32 words: in FP64,
+// at 1/64 of the rate, 10 us, and 27 instead of 11 for 192 -> 64 channels.
+__global__ void __launch_bounds__(256) k_wgrad_tc_reduce(const float *part, int nparts, int ngroups, int N, int ncb,
+                                                         int Cin_real, float *dW)
 {
-    const int64_t n = (int64_t)ngroups * 128 * N;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int co = (int)(e % N);
-        const int64_t rr = e / N;
-        const int row = (int)(rr % 128), g = (int)(rr / 128);
-        const int sidx = g * 4 + row / 32, ci = (sidx % ncb) * 32 + row % 32, tap = sidx / ncb;
-        if (sidx >= 9 * ncb || ci >= Cin_real) continue;
-        double acc = 0.0;
-        for (int k = 0; k < nparts; ++k) acc += part[(int64_t)k * n + e];
-        dW[((int64_t)co * Cin_real + ci) * 9 + tap] = (float)acc;
+    __shared__ float2 red[8][32];
+    const int64_t n = (int64_t)ngroups * 128 * N;  // a multiple of 32
+    const int64_t e = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    const int j = threadIdx.x >> 5;
+    float acc = 0.f, lost = 0.f;
+#pragma unroll 4
+    for (int k = j; k < nparts; k += 8) comp_pair(acc, lost, part[(int64_t)k * n + e]);
+    red[j][threadIdx.x & 31] = make_float2(acc, lost);
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int co = (int)(e % N);
+    const int64_t rr = e / N;
+    const int row = (int)(rr % 128), g = (int)(rr / 128);
+    const int sidx = g * 4 + row / 32, ci = (sidx % ncb) * 32 + row % 32, tap = sidx / ncb;
+    if (sidx >= 9 * ncb || ci >= Cin_real) return;
+    for (int jj = 1; jj < 8; ++jj) {
+        lost += red[jj][threadIdx.x].y;
+        comp_pair(acc, lost, red[jj][threadIdx.x].x);
     }
+    dW[((int64_t)co * Cin_real + ci) * 9 + tap] = comp_value(acc, lost);
 }
 
 // Per-channel sums of a [P][ld] BF16 tensor over pixels: one block per range
 // of pps pixels; thread t sums channels 8 (t % (C/8)) .. +7 over the pixels
 // p0 + t / (C/8), + 256 / (C/8), ...; then a fixed-order reduction in shared
-// memory.  part[block][C].
+// memory.  part[block][C].  kSumBlocks blocks at most, eight per SM: with one per
+// 4096 pixels the quarter-size layers ran on 16 blocks (70 us, the full-size ones 22).
+constexpr int kSumBlocks = kSMs * 8;
+inline int sum_pixels(int P) { return std::max(64, (P + kSumBlocks - 1) / kSumBlocks); }
+
 __global__ void k_chansum(const bf16 *Y, int ld, int C, int P, int pps, float *part)
 {
     __shared__ float red[256][8];
@@ -995,6 +1012,7 @@ __global__ void k_chansum(const bf16 *Y, int ld, int C, int P, int pps, float *p
     const int p0 = blockIdx.x * pps, p1 = min(P, p0 + pps);
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (pr < lanes)
+#pragma unroll 4
         for (int p = p0 + pr; p < p1; p += lanes) {
             const B8 v = ld8(Y + (int64_t)p * ld + cg * 8);
 #pragma unroll
@@ -1032,13 +1050,17 @@ __global__ void __launch_bounds__(256) k_sum_cols(const float *part, int nblk, i
 // Elementwise pieces
 // ---------------------------------------------------------------------------
 // network input: channel 0 = x / s, channels 1 .. 31 zero (the first layer's
-// padded input); grid-stride, as its grid is capped (grid_for)
+// padded input); grid-stride, as its grid is capped (grid_for).  16 bytes a thread: one
+// channel a thread took 53 us at 2^20 pixels (67 MB written), this 13.
 __global__ void k_in_prep(const float *x, int P, float inv_s, bf16 *xin)
 {
-    const int64_t n = (int64_t)P * 32;
+    const int64_t n = (int64_t)P * 4;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int p = (int)(i / 32), c = (int)(i % 32);
-        xin[i] = __float2bfloat16(c == 0 ? x[p] * inv_s : 0.f);
+        B8 v;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v.v[k] = 0.f;
+        if ((i & 3) == 0) v.v[0] = x[i >> 2] * inv_s;
+        st8(xin + i * 8, v);
     }
 }
 
@@ -1108,73 +1130,87 @@ __global__ void k_pool_back_mask(const bf16 *dskip, int lds, const bf16 *dp, int
     }
 }
 
-// out = x + s (Wh . d1 + bh); per-block partial sums of (out - t)^2 when t given
-__global__ void k_head(const bf16 *d1, const float *Wh, const float *bh, const float *x, float s, int P,
-                       float *out, const float *t, float *lpart)
+// Head, out = x + s (Wh . d1 + bh): four lanes share a pixel, 8 channels each, so
+// that a warp reads 512 contiguous bytes (a thread per pixel read its 64 bytes in
+// four strided pieces).  The sum passes from lane to lane in the order of the channels:
+// the value does not depend on the split.
+__device__ __forceinline__ float head_value(const B8 &v, const float (&wh)[8], float bh, float x, float s)
 {
-    __shared__ float red[256];
-    float l = 0.f;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        float h = *bh;
-        const bf16 *row = d1 + (int64_t)p * 32;
+    float h = bh;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const B8 v = ld8(row + 8 * g);
+    for (int g = 0; g < 4; ++g) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) h = fmaf(Wh[8 * g + c], v.v[c], h);
-        }
-        const float o = x[p] + s * h;
-        if (out) out[p] = o;
-        if (t) {
-            const float e = o - t[p];
-            l += e * e;
-        }
+        for (int k = 0; k < 8; ++k) h = fmaf(wh[k], v.v[k], h);
+        h = __shfl_sync(0xffffffffu, h, (threadIdx.x & 28) + g);
     }
-    if (!lpart) return;
-    red[threadIdx.x] = l;
-    __syncthreads();
-    for (int k = blockDim.x / 2; k > 0; k >>= 1) {
-        if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) lpart[blockIdx.x] = red[0];
+    return x + s * h;
 }
 
-// Head backward: dh = s * 2 (out - t) / P; dd1 = dh Wh * (d1 > 0);
-// partials of dWh[c] = sum dh d1[c] and dbh = sum dh per block.
-__global__ void k_head_back(const bf16 *d1, const float *Wh, const float *out, const float *t, float s, int P,
-                            bf16 *dd1, float *part /*[blocks][33]*/)
+constexpr int kHeadBlocks = kSMs * 8;
+inline int head_grid(int P) { return std::min((P + 63) / 64, kHeadBlocks); }
+
+__global__ void __launch_bounds__(256) k_head(const bf16 *__restrict__ d1, const float *__restrict__ Wh,
+                                              const float *__restrict__ bh, const float *__restrict__ x, float s, int P,
+                                              float *__restrict__ out)
 {
-    __shared__ float red[33][256];
-    float acc[33];
+    const int cg = threadIdx.x & 3;
+    float wh[8];
 #pragma unroll
-    for (int c = 0; c < 33; ++c) acc[c] = 0.f;
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        const float dh = s * 2.f * (out[p] - t[p]) / (float)P;
-        const bf16 *row = d1 + (int64_t)p * 32;
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const B8 v = ld8(row + 8 * g);
-            B8 o;
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                acc[8 * g + c] = fmaf(dh, v.v[c], acc[8 * g + c]);
-                o.v[c] = v.v[c] > 0.f ? dh * Wh[8 * g + c] : 0.f;
-            }
-            st8(dd1 + (int64_t)p * 32 + 8 * g, o);
-        }
-        acc[32] += dh;
-    }
-#pragma unroll
-    for (int c = 0; c < 33; ++c) red[c][threadIdx.x] = acc[c];
-    __syncthreads();
-    if (threadIdx.x < 33) {
-        float sum = 0.f;
-        for (int k = 0; k < (int)blockDim.x; ++k) sum += red[threadIdx.x][k];
-        part[blockIdx.x * 33 + threadIdx.x] = sum;
+    for (int k = 0; k < 8; ++k) wh[k] = Wh[cg * 8 + k];
+    const float b = *bh;
+    for (int p0 = blockIdx.x * 64; p0 < P; p0 += gridDim.x * 64) {
+        const int p = p0 + (threadIdx.x >> 2), q = min(p, P - 1);
+        const float o = head_value(ld8(d1 + (int64_t)q * 32 + cg * 8), wh, b, x[q], s);
+        if (p < P && cg == 0) out[p] = o;
     }
 }
 
+// Head of a training step, forward and backward in one pass over d1 (two passes
+// took 24 + 65 us at 2^20 pixels, one takes 30): e = out - t, dh = 2 s e / P,
+// dd1 = dh Wh (d1 > 0); part[block][34]: sums of dh d1[c], of dh and of e^2.
+__global__ void __launch_bounds__(256) k_head_train(const bf16 *__restrict__ d1, const float *__restrict__ Wh,
+                                                    const float *__restrict__ bh, const float *__restrict__ x,
+                                                    const float *__restrict__ t, float s, int P, bf16 *__restrict__ dd1,
+                                                    float *__restrict__ part)
+{
+    __shared__ float red[8][4][10];
+    const int cg = threadIdx.x & 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float wh[8], acc[10];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) wh[k] = Wh[cg * 8 + k];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) acc[k] = 0.f;
+    const float b = *bh;
+    for (int p0 = blockIdx.x * 64; p0 < P; p0 += gridDim.x * 64) {
+        const int p = p0 + (threadIdx.x >> 2), q = min(p, P - 1);
+        const B8 v = ld8(d1 + (int64_t)q * 32 + cg * 8);
+        const float e = head_value(v, wh, b, x[q], s) - t[q];
+        if (p >= P) continue;
+        const float dh = s * 2.f * e / (float)P;
+        B8 o;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            acc[k] = fmaf(dh, v.v[k], acc[k]);
+            o.v[k] = v.v[k] > 0.f ? dh * wh[k] : 0.f;
+        }
+        st8(dd1 + (int64_t)p * 32 + cg * 8, o);
+        acc[8] += dh;
+        acc[9] += e * e;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        for (int off = 4; off < 32; off <<= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
+        if (lane < 4) red[warp][cg][k] = acc[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 34) {
+        const int c = threadIdx.x, g = c < 32 ? c / 8 : 0, k = c < 32 ? c % 8 : c - 24;
+        double sum = 0.0;
+        for (int w = 0; w < 8; ++w) sum += red[w][g][k];
+        part[(int64_t)blockIdx.x * 34 + c] = (float)sum;
+    }
+}
 
 // FP32 flat layer weights -> BF16 [Cout][9][Cin_pad] (forward) and
 // [Cin][9][Cout] flipped (input gradient).
@@ -1213,7 +1249,7 @@ using namespace dect;
 struct dect_cnn {
     int device;
     int max_p;  // max batch * H * W
-    float *prm, *grad, *m, *v;  // FP32 [num_params]
+    float *prm, *grad, *m, *v;  // FP32 [num_params]; the sum of squared errors behind grad
     int64_t np;
     int64_t off_w[kLayers], off_b[kLayers], off_h;
     bf16 *wf[kLayers], *wt[kLayers];
@@ -1225,7 +1261,7 @@ struct dect_cnn {
     bf16 *p2, *a5, *bt;
     // gradients
     bf16 *g_full_a, *g_full_b, *g_c1, *g_half_a, *g_half_b, *g_c2, *g_q_a, *g_q_b;
-    float *out, *wpart, *cpart, *hpart;
+    float *wpart, *cpart;
     size_t wpart_elems;
     int steps;  // Adam step count
     int conv_path;  // DECT_CNN_CONV_TCGEN05 or DECT_CNN_CONV_MMA_SYNC
@@ -1444,8 +1480,8 @@ dect_status wgrad_tc(dect_cnn *n, int l, const bf16 *dY, int ldd, const bf16 *X,
     }
     DECT_CUDA(cudaFuncSetAttribute(k_wgrad_tc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     k_wgrad_tc<N><<<dim3(gy, gx), kWgThreads, smem, s>>>(tx, td, a, G, nstage, n->wpart, n->err);
-    k_wgrad_tc_reduce<<<grid_for((int64_t)a.ngroups * 128 * N), 256, 0, s>>>(n->wpart, gx, a.ngroups, N, a.ncb,
-                                                                            kCin[l], n->grad + n->off_w[l]);
+    k_wgrad_tc_reduce<<<(unsigned)(a.ngroups * 4 * N), 256, 0, s>>>(n->wpart, gx, a.ngroups, N, a.ncb, kCin[l],
+                                                                 n->grad + n->off_w[l]);
     count_launches(2);
     return DECT_OK;
 }
@@ -1463,7 +1499,7 @@ dect_status wgrad(dect_cnn *n, int l, const bf16 *dY, int ldd, const bf16 *X, in
         default: set_error_text("k_wgrad_tc: unsupported output channel count");
         }
         if (st != DECT_OK) return st;
-        const int cpps = 4096, csplits = (P + cpps - 1) / cpps;
+        const int cpps = sum_pixels(P), csplits = (P + cpps - 1) / cpps;
         k_chansum<<<csplits, 256, 0, s>>>(dY, ldd, Cout, P, cpps, n->cpart);
         k_sum_cols<<<Cout, 256, 0, s>>>(n->cpart, csplits, Cout, n->grad + n->off_b[l]);
         count_launches(2);
@@ -1480,7 +1516,7 @@ dect_status wgrad(dect_cnn *n, int l, const bf16 *dY, int ldd, const bf16 *X, in
     k_wgrad<<<g, 128, 0, s>>>(a);
     k_wgrad_reduce<<<(unsigned)(((int64_t)Cout * 9 * Cinp + 31) / 32), 256, 0, s>>>(n->wpart, splits, Cout, Cinp, kCin[l],
                                                                         n->grad + n->off_w[l]);
-    const int cpps = 4096, csplits = (P + cpps - 1) / cpps;
+    const int cpps = sum_pixels(P), csplits = (P + cpps - 1) / cpps;
     k_chansum<<<csplits, 256, 0, s>>>(dY, ldd, Cout, P, cpps, n->cpart);
     k_sum_cols<<<Cout, 256, 0, s>>>(n->cpart, csplits, Cout, n->grad + n->off_b[l]);
     count_launches(4);
@@ -1497,7 +1533,7 @@ dect_status forward(dect_cnn *n, const float *x, int B, int H, int W, float scal
             n->prm + n->off_w[l], kCout[l], kCin[l], cin_pad(l), n->wf[l], n->wt[l]);
         count_launches(1);
     }
-    k_in_prep<<<grid_for((int64_t)P * 32), 256, 0, s>>>(x, P, 1.f / scale, n->xin);
+    k_in_prep<<<grid_for((int64_t)P * 4), 256, 0, s>>>(x, P, 1.f / scale, n->xin);
     count_launches(1);
     const float *b = n->prm;
     dect_status st;
@@ -1554,7 +1590,7 @@ extern "C" dect_status dect_cnn_create(int device, int max_pixels, dect_cnn **ou
     }
     n->off_h = o;
     const size_t P = (size_t)max_pixels, P2 = P / 4 + 1, P4 = P / 16 + 1;
-    bool ok = alloc((void **)&n->prm, 4 * n->np) && alloc((void **)&n->grad, 4 * n->np) &&
+    bool ok = alloc((void **)&n->prm, 4 * n->np) && alloc((void **)&n->grad, 4 * (n->np + 1)) &&
               alloc((void **)&n->m, 4 * n->np) && alloc((void **)&n->v, 4 * n->np);
     for (int l = 0; l < kLayers && ok; ++l) {
         ok = alloc((void **)&n->wf[l], 2 * (size_t)kCout[l] * 9 * cin_pad(l)) &&
@@ -1568,8 +1604,9 @@ extern "C" dect_status dect_cnn_create(int device, int max_pixels, dect_cnn **ou
     A(&n->g_half_a, P2 * 64); A(&n->g_half_b, P2 * 64); A(&n->g_c2, P2 * 192);
     A(&n->g_q_a, P4 * 128); A(&n->g_q_b, P4 * 128);
     n->wpart_elems = (size_t)64 << 20;  // 256 MB of FP32 split-K partials at most
-    if (ok) ok = alloc((void **)&n->out, 4 * P) && alloc((void **)&n->wpart, 4 * n->wpart_elems) &&
-                 alloc((void **)&n->cpart, 4 * ((P / 4096 + 2) * 192)) && alloc((void **)&n->hpart, 4 * 4096 * 33);
+    // partials of the sums over pixels: kSumBlocks of 128 channels, kHeadBlocks of 34
+    static_assert(kSumBlocks * 128 >= kHeadBlocks * 34, "size of cpart");
+    if (ok) ok = alloc((void **)&n->wpart, 4 * n->wpart_elems) && alloc((void **)&n->cpart, 4 * (size_t)kSumBlocks * 128);
     if (ok) ok = alloc((void **)&n->err, sizeof(unsigned));
     if (ok) ok = cudaMemset(n->m, 0, 4 * n->np) == cudaSuccess && cudaMemset(n->v, 0, 4 * n->np) == cudaSuccess &&
                  cudaMemset(n->prm, 0, 4 * n->np) == cudaSuccess && cudaMemset(n->err, 0, sizeof(unsigned)) == cudaSuccess;
@@ -1588,7 +1625,7 @@ extern "C" dect_status dect_cnn_destroy(dect_cnn *n)
     cudaDeviceSynchronize();
     void *ptrs[] = {n->prm, n->grad, n->m, n->v, n->xin, n->a1, n->e1, n->c1, n->a9, n->d1, n->p1, n->a3,
                     n->c2, n->a7, n->d2, n->p2, n->a5, n->bt, n->g_full_a, n->g_full_b, n->g_c1, n->g_half_a,
-                    n->g_half_b, n->g_c2, n->g_q_a, n->g_q_b, n->out, n->wpart, n->cpart, n->hpart, n->err};
+                    n->g_half_b, n->g_c2, n->g_q_a, n->g_q_b, n->wpart, n->cpart, n->err};
     for (void *p : ptrs) cudaFree(p);
     for (int l = 0; l < kLayers; ++l) {
         cudaFree(n->wf[l]);
@@ -1626,8 +1663,7 @@ extern "C" dect_status dect_cnn_forward(dect_cnn *n, const float *x, float *out,
     dect_status st = forward(n, x, batch, h, w, scale, s);
     if (st != DECT_OK) return st;
     const int P = batch * h * w;
-    k_head<<<grid_for(P), 256, 0, s>>>(n->d1, n->prm + n->off_h, n->prm + n->off_h + 32, x, scale, P, out,
-                                      nullptr, nullptr);
+    k_head<<<head_grid(P), 256, 0, s>>>(n->d1, n->prm + n->off_h, n->prm + n->off_h + 32, x, scale, P, out);
     count_launches(1);
     DECT_LAUNCH_CHECK();
     return DECT_OK;
@@ -1643,16 +1679,12 @@ extern "C" dect_status dect_cnn_loss_grad(dect_cnn *n, const float *x, const flo
     if (st != DECT_OK) return st;
     const int B = batch, H = h, W = w, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
     const int P = B * H * W, P2 = B * H2 * W2, P4 = B * H4 * W4;
-    const int hb = (int)std::min<int64_t>((P + 255) / 256, 4096);
-    k_head<<<hb, 256, 0, s>>>(n->d1, n->prm + n->off_h, n->prm + n->off_h + 32, x, scale, P, n->out, target,
-                              n->hpart);
-    k_sum_cols<<<1, 256, 0, s>>>(n->hpart, hb, 1, n->cpart);  // loss * P in cpart[0]
-    float lsum = 0.f;
-    DECT_CUDA(cudaMemcpyAsync(&lsum, n->cpart, 4, cudaMemcpyDeviceToHost, s));
-    // head backward
-    k_head_back<<<hb, 256, 0, s>>>(n->d1, n->prm + n->off_h, n->out, target, scale, P, n->g_full_a, n->hpart);
-    k_sum_cols<<<33, 256, 0, s>>>(n->hpart, hb, 33, n->grad + n->off_h);
-    count_launches(4);
+    // the head, forward and backward: its gradients, and behind them the sum of squared errors
+    const int hb = head_grid(P);
+    k_head_train<<<hb, 256, 0, s>>>(n->d1, n->prm + n->off_h, n->prm + n->off_h + 32, x, target, scale, P, n->g_full_a,
+                                    n->cpart);
+    k_sum_cols<<<34, 256, 0, s>>>(n->cpart, hb, 34, n->grad + n->off_h);
+    count_launches(2);
     // conv10: input a9, output grad g_full_a (dd1, masked)
     if ((st = wgrad(n, 9, n->g_full_a, 32, n->a9, 32, B, H, W, s)) != DECT_OK) return st;
     if ((st = conv(n, n->g_full_a, 32, 32, n->wt[9], nullptr, n->g_full_b, 32, 32, n->a9, 32, false, B, H, W, s)) != DECT_OK) return st;  // da9
@@ -1679,7 +1711,9 @@ extern "C" dect_status dect_cnn_loss_grad(dect_cnn *n, const float *x, const flo
     if ((st = wgrad(n, 1, n->g_full_a, 32, n->a1, 32, B, H, W, s)) != DECT_OK) return st;
     if ((st = conv(n, n->g_full_a, 32, 32, n->wt[1], nullptr, n->g_full_b, 32, 32, n->a1, 32, false, B, H, W, s)) != DECT_OK) return st;  // da1
     if ((st = wgrad(n, 0, n->g_full_b, 32, n->xin, 32, B, H, W, s)) != DECT_OK) return st;
-    count_launches(3);
+    count_launches(4);
+    float lsum = 0.f;
+    DECT_CUDA(cudaMemcpyAsync(&lsum, n->grad + n->np, 4, cudaMemcpyDeviceToHost, s));
     DECT_LAUNCH_CHECK();
     DECT_CUDA(cudaStreamSynchronize(s));
     if ((st = dect_cnn_check(n)) != DECT_OK) return st;
