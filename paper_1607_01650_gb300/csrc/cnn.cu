@@ -782,32 +782,38 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float *part, int spl
 // ---------------------------------------------------------------------------
 // Weight gradient on the tensor cores (tcgen05):
 //   dW[co][tap][ci] = sum over pixels p of X[p + off(tap)][ci] * dY[p][co]
-// as D[m][n] = sum over k of A[m][k] B[n][k] with k = pixel, n = co and m a
-// row of a "slot" (tap, 32 input channels): an MMA of M = 128 covers a
-// group of four slots.  Both operands are read in their NHWC layout, i.e.
-// MN-major (the 32 channels of a pixel contiguous): TMA copies, per tile of
-// 8 x 16 pixels, one box {32 channels, 16, 8} of X shifted by each slot's
-// tap (zero outside the image) and the Cout / 32 boxes of dY; in the 64-byte
-// swizzle an atom is 32 channels x 8 pixels, atoms along M (or N) are one
-// box apart (LBO) and groups of 8 pixels 512 bytes apart (SBO); a K = 16
-// step is one image row of the tile (+1 KB).  A persistent block keeps its
-// groups' accumulators (FP32, G x Cout columns) in tensor memory over all
+// as D[m][n] = sum over k of A[m][k] B[n][k] with k = pixel, n = co and m = (row
+// of the 3 x 3 window, input channel of a block of 32): an MMA of M = 128 covers
+// a group, the three taps of one column offset dx.  Both operands are read in
+// their NHWC layout, i.e. MN-major (the 32 channels of a pixel contiguous): TMA
+// copies, per tile of 8 x 16 pixels, three boxes {32 channels, 16, 10} of X, one
+// per dx (zero outside the image), and the Cout / 32 boxes {32, 16, 8} of dY.  In
+// the 64-byte swizzle an atom is 32 channels x 8 pixels; groups of 8 pixels lie
+// 512 bytes apart (SBO), a K = 16 step is one image row of the tile (+1 KB), and so
+// is the next tap of the group: the atoms along M are 1 KB apart (LBO), and the
+// box serves all three taps.  The fourth atom of M = 128 reads the row below
+// (at the tile's last row 1 KB past the box, which is the next box): its 32 rows
+// of D are dropped.  (A box per tap, nine of 8 KB, was bound by the copies: with
+// 32 -> 32 channels at 2^20 pixels 95 us, 96 -> 32 339 us; now 46 and 126.)
+//   A block takes the 32 input channels of blockIdx.x.  A persistent block keeps its
+// three accumulators (FP32, 3 x Cout columns) in tensor memory over all
 // its tiles and writes them once as a partial; the partials are then added
 // in block order (k_wgrad_tc_reduce).  Roles and bounded waits as in
 // k_conv_tc: warp 0 TMA, warp 1 MMA, warps 2-5 read the accumulators.
 // ---------------------------------------------------------------------------
 constexpr int kWgR = 8;                               // image rows per tile (K = 128 pixels)
-constexpr int kWgBox = kWgR * kTcTW * kTcBK * 2;      // one box {32 channels, 16, 8}: 8 KB
+constexpr int kWgRow = kTcTW * kTcBK * 2;             // 16 pixels of 32 channels: 1 KB
+constexpr int kWgBox = kWgR * kWgRow;                 // a box of dY {32 channels, 16, 8}: 8 KB
+constexpr int kWgBoxX = (kWgR + 2) * kWgRow;          // a box of X {32 channels, 16, 10}: 10 KB
 constexpr int kWgMaxStages = 4;
 constexpr int kWgThreads = 192;
 
 struct WgTcArgs {
     int Cin, Cout, B, H, W;
-    int ncb;      // Cin / 32: slots per tap
-    int ngroups;  // ceil(9 ncb / 4)
+    int ncb;  // Cin / 32
 };
 
-__host__ __device__ constexpr int wg_stage_bytes(int G, int N) { return (4 * G + N / 32) * kWgBox; }
+__host__ __device__ constexpr int wg_stage_bytes(int N) { return 3 * kWgBoxX + N / 32 * kWgBox; }
 
 // MN-major operand in the 64-byte swizzle: atoms of 32 elements x 8 rows,
 // `lbo` bytes between atoms along M (or N), 512 bytes between 8-row groups
@@ -824,14 +830,14 @@ __host__ __device__ constexpr uint32_t tc_idesc_mn(int m, int n) { return tc_ide
 template <int N>
 __global__ void __launch_bounds__(kWgThreads, 1)
     k_wgrad_tc(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD, WgTcArgs a,
-               int G, int nstage, float *part, unsigned *err)
+               int nstage, float *part, unsigned *err)
 {
     static_assert(N == 32 || N == 64 || N == 128, "Cout of a forward layer");
     constexpr uint32_t idesc = tc_idesc_mn(128, N);
     extern __shared__ unsigned char smraw[];
     unsigned char *sm =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
-    const int STAGE = wg_stage_bytes(G, N);
+    constexpr int STAGE = wg_stage_bytes(N);
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + nstage * STAGE);
     uint64_t *full = bars, *empty = bars + kWgMaxStages, *done = bars + 2 * kWgMaxStages;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
@@ -840,13 +846,11 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tiles_x = (a.W + kTcTW - 1) / kTcTW, tiles_y = (a.H + kWgR - 1) / kWgR;
     const int per_img = tiles_x * tiles_y, ntiles = a.B * per_img;
-    // blockIdx.x: the group set (the blocks sharing a tile are launched side
+    // blockIdx.x: the 32 input channels (the blocks sharing a tile are launched side
     // by side, so that they read its pixels from L2 at about the same time);
     // blockIdx.y: the block's share of the tiles
-    const int g0 = blockIdx.x * G, gn = min(G, a.ngroups - g0);
-    const int nslot = 9 * a.ncb;
-    uint32_t tm_cols = 32;
-    while (tm_cols < (uint32_t)(G * N)) tm_cols *= 2;
+    const int cb = blockIdx.x;
+    constexpr uint32_t tm_cols = N == 32 ? 128 : N == 64 ? 256 : 512;  // three accumulators
 
     if (threadIdx.x == 0) {
         for (int q = 0; q < nstage; ++q) {
@@ -866,10 +870,6 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     int issued = 0;
     if (warp == 0) {
         if (lane == 0) {
-            // boxes per tile: the valid slots of the block's groups, then dY
-            int nvalid = 0;
-            for (int k = 0; k < 4 * gn; ++k) nvalid += (g0 * 4 + k) < nslot;
-            const unsigned bytes = (unsigned)((nvalid + N / 32) * kWgBox);
             int n = 0, st = 0, u = 0;
             for (int t = blockIdx.y; t < ntiles && !s_fail; t += gridDim.y, ++n) {
                 if (u > 0 && !tc_wait(empty + st, (u - 1) & 1, &s_fail)) {
@@ -879,16 +879,13 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 const int b = t / per_img, r = t % per_img;
                 const int y0 = (r / tiles_x) * kWgR, x0 = (r % tiles_x) * kTcTW;
                 unsigned char *dst = sm + st * STAGE;
-                mbar_arrive_expect_tx(full + st, bytes);
-                for (int k = 0; k < 4 * gn; ++k) {
-                    const int sidx = g0 * 4 + k;
-                    if (sidx >= nslot) break;
-                    const int tap = sidx / a.ncb, cb = sidx % a.ncb;
-                    tma_load_4d(dst + k * kWgBox, &tmX, cb * kTcBK, x0 + tap % 3 - 1, y0 + tap / 3 - 1, b, full + st);
-                }
+                mbar_arrive_expect_tx(full + st, (unsigned)STAGE);
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+                    tma_load_4d(dst + dx * kWgBoxX, &tmX, cb * kTcBK, x0 + dx - 1, y0 - 1, b, full + st);
 #pragma unroll
                 for (int j = 0; j < N / 32; ++j)
-                    tma_load_4d(dst + (4 * G + j) * kWgBox, &tmD, j * kTcBK, x0, y0, b, full + st);
+                    tma_load_4d(dst + 3 * kWgBoxX + j * kWgBox, &tmD, j * kTcBK, x0, y0, b, full + st);
                 issued = n + 1;
                 if (++st == nstage) {
                     st = 0;
@@ -907,9 +904,10 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 }
                 tc_fence_after();
                 const unsigned char *base = sm + st * STAGE;
-                const uint64_t bd0 = sw64_mn_desc(base + 4 * G * kWgBox, kWgBox);
-                for (int gi = 0; gi < gn; ++gi) {
-                    const uint64_t ad0 = sw64_mn_desc(base + gi * 4 * kWgBox, kWgBox);
+                const uint64_t bd0 = sw64_mn_desc(base + 3 * kWgBoxX, kWgBox);
+#pragma unroll
+                for (int gi = 0; gi < 3; ++gi) {
+                    const uint64_t ad0 = sw64_mn_desc(base + gi * kWgBoxX, kWgRow);
 #pragma unroll
                     for (int i = 0; i < kWgR; ++i)  // one image row (16 pixels) per K step: +1 KB
                         tc_mma(tmem + (uint32_t)(gi * N), ad0 + (uint64_t)(i * 64), bd0 + (uint64_t)(i * 64), idesc,
@@ -926,13 +924,13 @@ __global__ void __launch_bounds__(kWgThreads, 1)
             tc_commit(done);
         }
     } else {
-        // accumulators -> partial: part[block y][group][row][co], row = slot-in-group * 32 + channel
+        // accumulators -> partial: part[block y][cb][dx][dy * 32 + channel][co]; the fourth quarter is dropped
         const int q = warp & 3;
         const bool ok = tc_wait(done, 0, &s_fail);
         if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            for (int gi = 0; gi < gn; ++gi) {
-                float *dst = part + (((int64_t)blockIdx.y * a.ngroups + g0 + gi) * 128 + q * 32 + lane) * N;
+            for (int gi = 0; gi < (q < 3 ? 3 : 0); ++gi) {
+                float *dst = part + ((((int64_t)blockIdx.y * a.ncb + cb) * 3 + gi) * 96 + q * 32 + lane) * N;
 #pragma unroll 1
                 for (int c0 = 0; c0 < N; c0 += 16) {
                     uint32_t v[16];
@@ -965,17 +963,16 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     if (warp == 0) tc_dealloc(tmem, tm_cols);
 }
 
-// dW (flat [Cout][Cin_real][3][3]) = sum over blocks k of part[k][g][row][co]
-// (fixed order), row = (slot % 4) * 32 + channel, slot = tap * ncb + ci / 32.
+// dW (flat [Cout][Cin_real][3][3]) = sum over blocks k of part[k][cb][dx][dy * 32 + channel][co] (fixed order).
 // As in k_wgrad_reduce, a block takes 32 elements and 8 slices of the partials: a
 // thread per element (48 blocks for 32 -> 32 channels) walked its 152 partials
 // one load after the other, 28 us; now 7.  The sums take two FP32 words: in FP64,
 // at 1/64 of the rate, 10 us, and 27 instead of 11 for 192 -> 64 channels.
-__global__ void __launch_bounds__(256) k_wgrad_tc_reduce(const float *part, int nparts, int ngroups, int N, int ncb,
-                                                         int Cin_real, float *dW)
+__global__ void __launch_bounds__(256) k_wgrad_tc_reduce(const float *part, int nparts, int N, int ncb, int Cin_real,
+                                                         float *dW)
 {
     __shared__ float2 red[8][32];
-    const int64_t n = (int64_t)ngroups * 128 * N;  // a multiple of 32
+    const int64_t n = (int64_t)ncb * 288 * N;  // a multiple of 32
     const int64_t e = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
     const int j = threadIdx.x >> 5;
     float acc = 0.f, lost = 0.f;
@@ -986,9 +983,9 @@ __global__ void __launch_bounds__(256) k_wgrad_tc_reduce(const float *part, int 
     if (threadIdx.x >= 32) return;
     const int co = (int)(e % N);
     const int64_t rr = e / N;
-    const int row = (int)(rr % 128), g = (int)(rr / 128);
-    const int sidx = g * 4 + row / 32, ci = (sidx % ncb) * 32 + row % 32, tap = sidx / ncb;
-    if (sidx >= 9 * ncb || ci >= Cin_real) return;
+    const int row = (int)(rr % 96), g = (int)(rr / 96);
+    const int ci = g / 3 * 32 + row % 32, tap = row / 32 * 3 + g % 3;
+    if (ci >= Cin_real) return;
     for (int jj = 1; jj < 8; ++jj) {
         lost += red[jj][threadIdx.x].y;
         comp_pair(acc, lost, red[jj][threadIdx.x].x);
@@ -1452,10 +1449,8 @@ dect_status wgrad_tc(dect_cnn *n, int l, const bf16 *dY, int ldd, const bf16 *X,
         return DECT_ERR_CUDA;
     }
     const int Cinp = cin_pad(l);
-    WgTcArgs a{Cinp, N, B, H, W, Cinp / kTcBK, (9 * (Cinp / kTcBK) + 3) / 4};
-    // groups of four slots per block: as many as two stages of the ring allow
-    const int G = std::min(N == 32 ? 3 : 2, a.ngroups);
-    const int stage = wg_stage_bytes(G, N);
+    WgTcArgs a{Cinp, N, B, H, W, Cinp / kTcBK};
+    constexpr int stage = wg_stage_bytes(N);
     const int nstage = std::min(kWgMaxStages, (kTcSmemMax - 1024 - 256 - kWgBox) / stage);
     if (nstage < 2) {
         set_error_text("k_wgrad_tc: no ring of two stages fits");
@@ -1465,23 +1460,23 @@ dect_status wgrad_tc(dect_cnn *n, int l, const bf16 *dY, int ldd, const bf16 *X,
     // either stride of its descriptor, can leave the block's shared memory)
     const int smem = 1024 + nstage * stage + 256 + kWgBox;
     CUtensorMap tx, td;
-    CUresult r = encode_nhwc(enc, &tx, X, Cinp, ldx, B, H, W, kWgR);
+    CUresult r = encode_nhwc(enc, &tx, X, Cinp, ldx, B, H, W, kWgR + 2);
     if (r == CUDA_SUCCESS) r = encode_nhwc(enc, &td, dY, N, ldd, B, H, W, kWgR);
     if (r != CUDA_SUCCESS) {
         set_error_text("k_wgrad_tc: cuTensorMapEncodeTiled failed with CUresult " + std::to_string((int)r));
         return DECT_ERR_CUDA;
     }
-    const int gy = (a.ngroups + G - 1) / G;
+    const int gy = a.ncb;
     const int ntiles = B * ((W + kTcTW - 1) / kTcTW) * ((H + kWgR - 1) / kWgR);
     const int gx = std::max(1, std::min(ntiles, kSMs / gy));
-    if ((int64_t)gx * a.ngroups * 128 * N > (int64_t)n->wpart_elems) {
+    if ((int64_t)gx * a.ncb * 288 * N > (int64_t)n->wpart_elems) {
         set_error_text("k_wgrad_tc: partials exceed the scratch buffer");
         return DECT_ERR_INVALID_ARG;
     }
     DECT_CUDA(cudaFuncSetAttribute(k_wgrad_tc<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_wgrad_tc<N><<<dim3(gy, gx), kWgThreads, smem, s>>>(tx, td, a, G, nstage, n->wpart, n->err);
-    k_wgrad_tc_reduce<<<(unsigned)(a.ngroups * 4 * N), 256, 0, s>>>(n->wpart, gx, a.ngroups, N, a.ncb, kCin[l],
-                                                                 n->grad + n->off_w[l]);
+    k_wgrad_tc<N><<<dim3(gy, gx), kWgThreads, smem, s>>>(tx, td, a, nstage, n->wpart, n->err);
+    k_wgrad_tc_reduce<<<(unsigned)(a.ncb * 9 * N), 256, 0, s>>>(n->wpart, gx, N, a.ncb, kCin[l],
+                                                             n->grad + n->off_w[l]);
     count_launches(2);
     return DECT_OK;
 }
