@@ -478,7 +478,8 @@ dect_status dect_adm_tv_ex(const dect_plan *plan, const float *m, float *x, int 
  * c channels uses the next of these widths >= min(c, 64)), and the measured
  * median time of each variant in microseconds (-1 = not available):
  *   0-2 L1-cached gather with 4x4 / 8x8 / 16x16 pixel tiles per 256-thread block,
- *   3   none (falls back to 1),
+ *   3   at 16 channels eight lanes per pixel, one 1024-thread block per SM over
+ *       8x32 tiles; otherwise none (falls back to 1),
  *   4-5 L1-cached gather, one 1024-thread block per SM, tiles of two / four
  *       block steps (8x8 / 16x8 pixels at 32 and 64 channels, 8x16 / 16x16 below),
  *   6-7 (16, 32 or 64 channels; otherwise 4 is used) each lane gathers 8

@@ -64,3 +64,17 @@ def test_infinite_pixel_keeps_its_sign():
     r[0, 3, 35] = float("inf")
     b = dect.backproject(plan, r)
     assert not torch.isnan(b).any() and bool((b == float("inf")).any())
+
+
+@pytest.mark.parametrize("n,ns", [(33, 7), (52, 8)])
+def test_eight_lane_backprojector_of_sixteen_channels(n, ns):
+    g = synth.tiny_geometry(n=n, nv=24, nb=80, px=1.0, sod=130.0, sdd=260.0)
+    m = np.stack([synth.make_slice(g, seed=400 + i, i0=1e5).m for i in range(ns)]).astype(np.float32)
+    plan, t = dect.Plan(g), oracle.table(g)
+    plan.set_tuning(16, 3)
+    x, _ = dect.adm_tv(plan, torch.tensor(m, device="cuda"), dect.AdmParams(mu=4.0, rho=256.0, max_iter=12))
+    for i in (0, ns - 1):
+        op = oracle.AdmParams(mu=4.0, rho=256.0, max_iter=12, step_rule=oracle.CAUCHY)
+        xo, _ = oracle.adm_dual(t, m[i].astype(np.float64), op)
+        for e in range(2):  # the bound of the other variants' test
+            assert np.linalg.norm(x[i, e].cpu().numpy() - xo[e]) <= 1e-4 * np.linalg.norm(xo[e])
