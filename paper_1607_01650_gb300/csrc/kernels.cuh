@@ -368,12 +368,12 @@ __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_g(const Entry *__restrict_
             }
 #pragma unroll
         for (int c = 0; c < VW; ++c) acc.v[c] = comp_value(acc.v[c], lost.v[c]);
-        return acc;
+    } else {
+#pragma unroll
+        for (int off = LPE; off < G; off <<= 1)
+#pragma unroll
+            for (int c = 0; c < VW; ++c) acc.v[c] += __shfl_xor_sync(0xffffffffu, acc.v[c], off);
     }
-#pragma unroll
-    for (int off = LPE; off < G; off <<= 1)
-#pragma unroll
-        for (int c = 0; c < VW; ++c) acc.v[c] += __shfl_xor_sync(0xffffffffu, acc.v[c], off);
     return acc;
 }
 

