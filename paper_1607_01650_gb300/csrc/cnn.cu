@@ -782,19 +782,22 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce(const float *part, int spl
 // ---------------------------------------------------------------------------
 // Weight gradient on the tensor cores (tcgen05):
 //   dW[co][tap][ci] = sum over pixels p of X[p + off(tap)][ci] * dY[p][co]
-// as D[m][n] = sum over k of A[m][k] B[n][k] with k = pixel, n = co and m = (row
-// of the 3 x 3 window, input channel of a block of 32): an MMA of M = 128 covers
-// a group, the three taps of one column offset dx.  Both operands are read in
-// their NHWC layout, i.e. MN-major (the 32 channels of a pixel contiguous): TMA
-// copies, per tile of 8 x 16 pixels, three boxes {32 channels, 16, 10} of X, one
-// per dx (zero outside the image), and the Cout / 32 boxes {32, 16, 8} of dY.  In
-// the 64-byte swizzle an atom is 32 channels x 8 pixels; groups of 8 pixels lie
-// 512 bytes apart (SBO), a K = 16 step is one image row of the tile (+1 KB), and so
-// is the next tap of the group: the atoms along M are 1 KB apart (LBO), and the
-// box serves all three taps.  The fourth atom of M = 128 reads the row below
-// (at the tile's last row 1 KB past the box, which is the next box): its 32 rows
-// of D are dropped.  (A box per tap, nine of 8 KB, was bound by the copies: with
-// 32 -> 32 channels at 2^20 pixels 95 us, 96 -> 32 339 us; now 46 and 126.)
+// as D[m][n] = sum over k of A[m][k] B[n][k] with k = pixel, m = (row offset dy of
+// the tap, input channel of a block of 32) and n = (column offset dx, co): the
+// row offset moves X, the column offset moves dY the other way (wg_move_d), so
+// that one MMA of M = 128 and N = 3 Cout takes all nine taps.  An MMA costs about
+// 55 cycles at any N <= 64: with X moved by dx and an MMA of N = Cout per dx, as for
+// 128 output channels (3 Cout > 256), 32 -> 32 channels at 2^20 pixels took 46 us
+// and 96 -> 32 126; now 30 and 79.  Both operands are read in their NHWC layout,
+// i.e. MN-major (the 32 channels of a pixel contiguous): TMA copies, per tile of
+// 8 x 16 pixels, boxes {32 channels, 16, 10} of X and {32, 16, 8} of dY, zero
+// outside the image.  In the 64-byte swizzle an atom is 32 channels x 8 pixels;
+// groups of 8 pixels lie 512 bytes apart (SBO), a K = 16 step is one image row of
+// the tile (+1 KB), and so is the next dy: the atoms of A along M are 1 KB apart
+// (LBO), and a box of X serves three taps.  The fourth atom of M = 128 reads the
+// row below (at the tile's last row 1 KB past the box, which is the next box):
+// its 32 rows of D are dropped.  (A box per tap, nine of 8 KB, was bound by
+// the copies: 95 and 339 us.)
 //   A block takes the 32 input channels of blockIdx.x.  A persistent block keeps its
 // three accumulators (FP32, 3 x Cout columns) in tensor memory over all
 // its tiles and writes them once as a partial; the partials are then added
@@ -813,7 +816,11 @@ struct WgTcArgs {
     int ncb;  // Cin / 32
 };
 
-__host__ __device__ constexpr int wg_stage_bytes(int N) { return 3 * kWgBoxX + N / 32 * kWgBox; }
+__host__ __device__ constexpr bool wg_move_d(int N) { return 3 * N <= 256; }  // the column offset moves dY (else X)
+__host__ __device__ constexpr int wg_stage_bytes(int N)
+{
+    return (wg_move_d(N) ? 1 : 3) * kWgBoxX + (wg_move_d(N) ? 3 : 1) * (N / 32) * kWgBox;
+}
 
 // MN-major operand in the 64-byte swizzle: atoms of 32 elements x 8 rows,
 // `lbo` bytes between atoms along M (or N), 512 bytes between 8-row groups
@@ -833,7 +840,9 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                int nstage, float *part, unsigned *err)
 {
     static_assert(N == 32 || N == 64 || N == 128, "Cout of a forward layer");
-    constexpr uint32_t idesc = tc_idesc_mn(128, N);
+    constexpr bool MOVE_D = wg_move_d(N);
+    constexpr int NX = MOVE_D ? 1 : 3, ND = MOVE_D ? 3 : 1;  // moved copies of X and of dY
+    constexpr uint32_t idesc = tc_idesc_mn(128, ND * N);
     extern __shared__ unsigned char smraw[];
     unsigned char *sm =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
@@ -881,11 +890,14 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 unsigned char *dst = sm + st * STAGE;
                 mbar_arrive_expect_tx(full + st, (unsigned)STAGE);
 #pragma unroll
-                for (int dx = 0; dx < 3; ++dx)
-                    tma_load_4d(dst + dx * kWgBoxX, &tmX, cb * kTcBK, x0 + dx - 1, y0 - 1, b, full + st);
+                for (int k = 0; k < NX; ++k)
+                    tma_load_4d(dst + k * kWgBoxX, &tmX, cb * kTcBK, MOVE_D ? x0 : x0 + k - 1, y0 - 1, b, full + st);
 #pragma unroll
-                for (int j = 0; j < N / 32; ++j)
-                    tma_load_4d(dst + 3 * kWgBoxX + j * kWgBox, &tmD, j * kTcBK, x0, y0, b, full + st);
+                for (int k = 0; k < ND; ++k)
+#pragma unroll
+                    for (int j = 0; j < N / 32; ++j)
+                        tma_load_4d(dst + NX * kWgBoxX + (k * (N / 32) + j) * kWgBox, &tmD, j * kTcBK,
+                                    MOVE_D ? x0 + 1 - k : x0, y0, b, full + st);
                 issued = n + 1;
                 if (++st == nstage) {
                     st = 0;
@@ -904,9 +916,9 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                 }
                 tc_fence_after();
                 const unsigned char *base = sm + st * STAGE;
-                const uint64_t bd0 = sw64_mn_desc(base + 3 * kWgBoxX, kWgBox);
+                const uint64_t bd0 = sw64_mn_desc(base + NX * kWgBoxX, kWgBox);
 #pragma unroll
-                for (int gi = 0; gi < 3; ++gi) {
+                for (int gi = 0; gi < NX; ++gi) {
                     const uint64_t ad0 = sw64_mn_desc(base + gi * kWgBoxX, kWgRow);
 #pragma unroll
                     for (int i = 0; i < kWgR; ++i)  // one image row (16 pixels) per K step: +1 KB
