@@ -1222,16 +1222,26 @@ __global__ void __launch_bounds__(256) k_head_train(const bf16 *__restrict__ d1,
 }
 
 // FP32 flat layer weights -> BF16 [Cout][9][Cin_pad] (forward) and
-// [Cin][9][Cout] flipped (input gradient).
-__global__ void k_wprep(const float *w, int Cout, int Cin, int Cin_pad, bf16 *wf, bf16 *wt)
+// [Cin][9][Cout] flipped (input gradient), layer blockIdx.y of all ten: a launch per
+// layer took 3 to 5 us each, 37 together, and was a third of a forward pass's launches
+// (training step at 16 images of 256^2: 1857 us, with one launch 1832).
+struct WprepArgs {
+    const float *w[kLayers];
+    bf16 *wf[kLayers], *wt[kLayers];
+    int cout[kLayers], cin[kLayers], cin_pad[kLayers];
+};
+__global__ void __launch_bounds__(256) k_wprep(const __grid_constant__ WprepArgs a)
 {
-    const int64_t n = (int64_t)Cout * Cin_pad * 9;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int co = (int)(i / (9 * Cin_pad)), r = (int)(i % (9 * Cin_pad));
+    const int l = blockIdx.y, Cout = a.cout[l], Cin = a.cin[l], Cin_pad = a.cin_pad[l];
+    const float *w = a.w[l];
+    bf16 *wf = a.wf[l], *wt = a.wt[l];
+    const int n = Cout * Cin_pad * 9;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
+        const int co = i / (9 * Cin_pad), r = i % (9 * Cin_pad);
         const int tap = r / Cin_pad, ci = r % Cin_pad;
-        const float v = ci < Cin ? w[((int64_t)co * Cin + ci) * 9 + tap] : 0.f;
+        const float v = ci < Cin ? w[(co * Cin + ci) * 9 + tap] : 0.f;
         wf[i] = __float2bfloat16(v);
-        if (wt && ci < Cin) wt[((int64_t)ci * 9 + (8 - tap)) * Cout + co] = __float2bfloat16(v);
+        if (ci < Cin) wt[(ci * 9 + (8 - tap)) * Cout + co] = __float2bfloat16(v);
     }
 }
 
@@ -1535,11 +1545,17 @@ dect_status forward(dect_cnn *n, const float *x, int B, int H, int W, float scal
 {
     const int P = B * H * W, H2 = H / 2, W2 = W / 2, H4 = H / 4, W4 = W / 4;
     const int P2 = B * H2 * W2, P4 = B * H4 * W4;
+    WprepArgs wa;
     for (int l = 0; l < kLayers; ++l) {
-        k_wprep<<<grid_for((int64_t)kCout[l] * cin_pad(l) * 9), 256, 0, s>>>(
-            n->prm + n->off_w[l], kCout[l], kCin[l], cin_pad(l), n->wf[l], n->wt[l]);
-        count_launches(1);
+        wa.w[l] = n->prm + n->off_w[l];
+        wa.wf[l] = n->wf[l];
+        wa.wt[l] = n->wt[l];
+        wa.cout[l] = kCout[l];
+        wa.cin[l] = kCin[l];
+        wa.cin_pad[l] = cin_pad(l);
     }
+    k_wprep<<<dim3(kSMs, kLayers), 256, 0, s>>>(wa);
+    count_launches(1);
     k_in_prep<<<grid_for((int64_t)P * 4), 256, 0, s>>>(x, P, 1.f / scale, n->xin);
     count_launches(1);
     const float *b = n->prm;
