@@ -18,14 +18,21 @@
 // Filter.  The taps cancel the projections' large mean, so the sums need more
 // than FP32.  FP64 runs at 1/64 of the FP32 rate (direct FP64 sums: 4.9 ms for
 // 64 images of 60 x 736), so the convolution runs on the tensor cores with
-// exact integer arithmetic: the odd taps couple bins of one parity to bins of
-// the other, a product with a Toeplitz matrix T(|d|) = 1 / d^2, d odd.  Each
-// row of q is scaled by a power of two and rounded to 38 bits, T likewise;
-// both are cut into five signed 8-bit digits, which BF16 holds exactly, and
-// the 15 digit products of weight above 2^-40 are summed by mma.sync in FP32,
-// one accumulator per weight: the sums are integers below 2^24, so nothing is
-// rounded.  The accumulators, the cosine weight and the h(0) term are then
-// joined in two FP32 words and rounded once.
+// integer arithmetic: the odd taps couple bins of one parity to bins of
+// the other, a product with a Toeplitz matrix T(|d|) = 1 / d^2, d odd.  A
+// row of q (below 2^e) is rounded to 2^(e-46), T to 2^-46;
+// both are cut into six signed 8-bit digits, which BF16 holds exactly, and
+// the 21 digit products of weight 2^(e-52) and above are summed by mma.sync in
+// FP32, one accumulator per weight: the sums are integers below 2^24, so these
+// sums are not rounded.  What is dropped leaves an error of the row's
+// magnitude, about sqrt(n_bins) 2^(e-47) rms (736 bins: 1.6e-13 of 2^e, at most
+// 7e-13 in 17664 sums), whatever the size of the output.  The
+// accumulators, the cosine weight and the h(0) term are then joined in two FP32
+// words and rounded once; an output so small that the error could show beside
+// that rounding (below 2^27 of the rms, 3e-5 of 2^e at 736 bins: about one in
+// 150 of a CT row, more than half of a row with one bin 100 times the others) is
+// summed again in FP64.  (Five digits and no second sum were 8.7e-9 off
+// before the rounding on CT rows, and 2.5e-7 beside such a bin.)
 //
 // Back-projection.  The bin coordinate t reaches n_bins - 1 and its rounding
 // moves the interpolation weights, so the per-pixel geometry is formed in two
@@ -82,15 +89,6 @@ struct ViewGeo {
     FF ex, ey, cx, cy;
 };
 
-__global__ void k_fbp_views(dect_geometry g, ViewGeo *vg)
-{
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= g.n_views) return;
-    const double th = g.start_rad + (double)v * (g.arc_rad / (double)g.n_views);
-    const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
-    vg[v] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
-}
-
 // cosine weight of bin b
 __device__ __forceinline__ double cos_weight(const dect_geometry &g, int b)
 {
@@ -98,10 +96,29 @@ __device__ __forceinline__ double cos_weight(const dect_geometry &g, int b)
     const double sb = u * (g.sod_mm / g.sdd_mm);
     return g.sod_mm / sqrt(g.sod_mm * g.sod_mm + sb * sb);
 }
+// tap h(k), k odd
+__device__ __forceinline__ double odd_tap(double k, double ds)
+{
+    const double pi = 3.14159265358979323846;
+    return -1.0 / (pi * pi * k * k * ds * ds);
+}
+
+// The views' directions, and for k_fbp_filter_tc the cosine weights [n_bins] and the
+// taps at odd distances 2 j + 1 [n_bins / 2 + 1].
+__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap)
+{
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v < g.n_bins) cwd[v] = cos_weight(g, v);
+    if (v <= g.n_bins / 2) tap[v] = odd_tap(2.0 * v + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
+    if (v >= g.n_views) return;
+    const double th = g.start_rad + (double)v * (g.arc_rad / (double)g.n_views);
+    const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
+    vg[v] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
+}
 
 // ---------------------------------------------------------------------------
 // FP64 filter: one block per (view, image); shared memory q[nb] and the odd
-// taps.  For detectors too wide for the digits of k_fbp_filter_tc.
+// taps.  For detectors of more than kTcMaxBins bins.
 // ---------------------------------------------------------------------------
 constexpr int kFbpBlock = 256;
 
@@ -115,11 +132,7 @@ __global__ void __launch_bounds__(kFbpBlock) k_fbp_filter(const float *__restric
     const int64_t row = ((int64_t)img * g.n_views + v) * nb;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) q[b] = (double)m[row + b] * cos_weight(g, b);
     const int nodd = nb / 2 + 1;
-    const double pi = 3.14159265358979323846;
-    for (int j = threadIdx.x; j < nodd; j += blockDim.x) {
-        const double k = 2.0 * j + 1.0;
-        hodd[j] = -1.0 / (pi * pi * k * k * ds * ds);
-    }
+    for (int j = threadIdx.x; j < nodd; j += blockDim.x) hodd[j] = odd_tap(2.0 * j + 1.0, ds);
     __syncthreads();
     const double h0 = 1.0 / (4.0 * ds * ds);
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
@@ -140,21 +153,25 @@ __global__ void __launch_bounds__(kFbpBlock) k_fbp_filter(const float *__restric
 
 // ---------------------------------------------------------------------------
 // Tensor-core filter (see the file header).  A block takes 16 rows (row R =
-// view R / nimg, image R % nimg) and all bins: the digits of both parities
-// stay in shared memory (160 bytes per bin), 16 warps share the 8-bin output
+// view R / nimg, image R % nimg) and all bins: the digits of one parity at a time
+// stay in shared memory (96 bytes per bin), 16 warps share the 8-bin output
 // tiles.  B fragments come from a table of T's digits by n - k (Toeplitz), two
 // neighbouring taps per 32-bit word.  T's first digit is zero from d = 13 on
 // and its second from d = 183 on (1 / d^2 below half a unit of it), so tiles
-// farther from the diagonal leave out the products with it.  Per block 32 k MMAs at
-// 736 bins; two blocks' worth per SM at 64 images of 60 views.
+// farther from the diagonal leave out the products with it.  Up to 44 k MMAs per
+// block at 736 bins; two blocks' worth per SM at 64 images of 60 views.
+//   The sum of one weight's products is at most the sum of |T digit| over both
+// sides' taps times 128: 0.92 2^24 at 1152 bins, below 2^24 up to 1270.
 // ---------------------------------------------------------------------------
-constexpr int kTcRows = 16, kTcWarps = 16, kTcThreads = 32 * kTcWarps, kDig = 5, kTcTiles = 3;
+constexpr int kTcRows = 16, kTcWarps = 16, kTcThreads = 32 * kTcWarps, kDig = 6, kTcTiles = 3;
+constexpr int kTcMaxBins = 1270;
 
 struct FilterShape {
     int half[2];  // bins of each parity
     int kpad;     // padded to a multiple of 16, for both
     int ld;       // row stride of a digit plane (BF16), 16 bytes off a multiple of 32
     int tn;       // words of one digit of the tap table
+    int nw;       // words of a row's bits
     size_t smem;
 };
 __host__ __device__ inline FilterShape filter_shape(int nb)
@@ -165,10 +182,12 @@ __host__ __device__ inline FilterShape filter_shape(int nb)
     f.kpad = (f.half[0] + 15) & ~15;
     f.ld = f.kpad + 8;
     f.tn = 2 * f.kpad + 32;
-    f.smem = (size_t)2 * kDig * kTcRows * f.ld * 2 + (size_t)kDig * f.tn * 4 + (size_t)nb * sizeof(FF);
+    f.nw = (nb + 31) / 32;
+    f.smem = (size_t)kDig * kTcRows * f.ld * 2 + (size_t)kDig * f.tn * 4 + (size_t)nb * sizeof(FF) +
+             (size_t)kTcRows * f.nw * 4;
     return f;
 }
-constexpr size_t kTcSmemMax = 220 * 1024;
+constexpr size_t kTcSmemMax = 176 * 1024;  // kTcMaxBins: 169 KB
 
 __device__ __forceinline__ void ldsm_a(unsigned (&r)[4], const void *p)
 {
@@ -185,7 +204,7 @@ __device__ __forceinline__ void mma_exact(float (&d)[4], const unsigned (&a)[4],
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// the five signed 8-bit digits of |Q| <= 2^38, most significant first, as BF16
+// the six signed 8-bit digits of |Q| <= 2^46, most significant first, as BF16
 __device__ __forceinline__ void digits(long long Q, __nv_bfloat16 (&d)[kDig])
 {
 #pragma unroll
@@ -197,44 +216,47 @@ __device__ __forceinline__ void digits(long long Q, __nv_bfloat16 (&d)[kDig])
 }
 
 __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__restrict__ m, float *__restrict__ qf,
-                                                              dect_geometry g, int nimg, int width)
+                                                              const double *__restrict__ cwd,
+                                                              const double *__restrict__ tap, dect_geometry g, int nimg,
+                                                              int width)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ float sscale[kTcRows];  // 2^(e - 12) of the row; 0: a row left to FP64
-    __shared__ int any_bad;
+    __shared__ float sscale[kTcRows];  // 2^(e - 12) of the row
+    __shared__ float slim[kTcRows];    // smaller outputs (times ds) are left to FP64; NaN: all of them
     const int nb = g.n_bins, nv = g.n_views;
     const FilterShape F = filter_shape(nb);
-    __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16 *>(dyn);  // [parity][digit][row][ld]
-    unsigned *T = reinterpret_cast<unsigned *>(A + (size_t)2 * kDig * kTcRows * F.ld);  // [digit][tn]
+    __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16 *>(dyn);  // [digit][row][ld], the inputs of one parity
+    unsigned *T = reinterpret_cast<unsigned *>(A + (size_t)kDig * kTcRows * F.ld);  // [digit][tn]
     FF *cw = reinterpret_cast<FF *>(T + (size_t)kDig * F.tn);
+    unsigned *todo = reinterpret_cast<unsigned *>(cw + nb);  // [row][nw] a bit per bin left to FP64
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t R0 = (int64_t)blockIdx.x * kTcRows, rows = (int64_t)nv * nimg;
     const double ds = g.pitch_mm * (g.sod_mm / g.sdd_mm);
-    if (threadIdx.x == 0) any_bad = 0;
-    for (int b = threadIdx.x; b < nb; b += kTcThreads) cw[b] = ff_of(cos_weight(g, b));
+    for (int b = threadIdx.x; b < nb; b += kTcThreads) cw[b] = ff_of(cwd[b]);
+    for (int b = threadIdx.x; b < kTcRows * F.nw; b += kTcThreads) todo[b] = 0u;
     // tap table: word w holds (T(w - kpad - 16), T(w - kpad - 17)) of the even outputs,
     // T(x) = 1 / (2 j + 1)^2, j = x - 1 for x > 0 and -x otherwise
     for (int w = threadIdx.x; w < F.tn; w += kTcThreads) {
         __nv_bfloat16 d0[kDig], d1[kDig];
         const int x = w - F.kpad - 16, j0 = x > 0 ? x - 1 : -x, j1 = x - 1 > 0 ? x - 2 : 1 - x;
         const double k0 = 2.0 * j0 + 1.0, k1 = 2.0 * j1 + 1.0;
-        digits(__double2ll_rn(0x1p38 / (k0 * k0)), d0);
-        digits(__double2ll_rn(0x1p38 / (k1 * k1)), d1);
+        digits(__double2ll_rn(0x1p46 / (k0 * k0)), d0);
+        digits(__double2ll_rn(0x1p46 / (k1 * k1)), d1);
 #pragma unroll
         for (int k = 0; k < kDig; ++k)
             T[k * F.tn + w] = (unsigned)__bfloat16_as_ushort(d0[k]) | ((unsigned)__bfloat16_as_ushort(d1[k]) << 16);
     }
     __syncthreads();
-    // q's digits, a warp per row
+    // a warp per row: its scale, later its digits
+    const bool on = R0 + warp < rows;
+    const int vw = on ? (int)((R0 + warp) / nimg) : 0, iw = on ? (int)((R0 + warp) % nimg) : 0;
+    const float *mine = m + ((int64_t)iw * nv + vw) * nb;
+    float sc;
     {
-        const int64_t R = R0 + warp;
-        const bool on = R < rows;
-        const int v = on ? (int)(R / nimg) : 0, img = on ? (int)(R % nimg) : 0;
-        const float *src = m + ((int64_t)img * nv + v) * nb;
         float mx = 0.f;
         bool finite = true;
         for (int b = lane; b < nb && on; b += 32) {
-            const float q = fabsf(src[b] * cw[b].h);
+            const float q = fabsf(mine[b] * cw[b].h);
             finite &= isfinite(q);
             mx = fmaxf(mx, q);
         }
@@ -246,30 +268,30 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
         frexpf(mx, &e);
         e += 1;  // the rounded product above may lie a rounding below q
         const bool bad = !finite || (mx > 0.f && (mx < 0x1p-60f || mx > 0x1p60f));
-        const float sc = mx > 0.f && !bad ? ldexpf(1.f, 38 - e) : 0.f;
+        sc = mx > 0.f && !bad ? ldexpf(1.f, 46 - e) : 0.f;
         if (lane == 0) {
-            sscale[warp] = bad ? 0.f : ldexpf(1.f, mx > 0.f ? e - 12 : 0);
-            if (bad) any_bad = 1;
+            sscale[warp] = ldexpf(1.f, sc > 0.f ? e - 12 : 0);
+            slim[warp] = bad ? NAN : mx > 0.f ? ldexpf(sqrtf((float)nb), e - 23) : 0.f;
         }
-        for (int b = lane; b < 2 * F.kpad; b += 32) {
+    }
+    const FF ipi2 = ff_of(1.0 / (3.14159265358979323846 * 3.14159265358979323846)), ids = ff_of(1.0 / ds);
+    const int gid = lane >> 2, t4 = lane & 3;
+    for (int par = 0; par < 2; ++par) {  // outputs of parity par from inputs of the other
+        __syncthreads();  // the scales are written; the other parity's digits have been read
+        for (int i = lane; i < F.kpad; i += 32) {
             __nv_bfloat16 d[kDig];
+            const int b = 2 * i + 1 - par;
             long long Q = 0;
             if (on && b < nb && sc > 0.f) {
-                const FF q = ff_mul(FF{src[b], 0.f}, cw[b]);
+                const FF q = ff_mul(FF{mine[b], 0.f}, cw[b]);
                 Q = __float2ll_rn(q.h * sc) + __float2ll_rn(q.l * sc);
             }
             digits(Q, d);
 #pragma unroll
-            for (int k = 0; k < kDig; ++k)
-                A[(((size_t)(b & 1) * kDig + k) * kTcRows + warp) * F.ld + (b >> 1)] = d[k];
+            for (int k = 0; k < kDig; ++k) A[((size_t)k * kTcRows + warp) * F.ld + i] = d[k];
         }
-    }
-    __syncthreads();
-    const FF ipi2 = ff_of(1.0 / (3.14159265358979323846 * 3.14159265358979323846)), ids = ff_of(1.0 / ds);
-    const int gid = lane >> 2, t4 = lane & 3;
-    for (int par = 0; par < 2; ++par) {  // outputs of parity par from inputs of the other
+        __syncthreads();
         const int nt = (F.half[par] + 7) / 8, per = (nt + kTcWarps - 1) / kTcWarps;
-        const __nv_bfloat16 *Ap = A + (size_t)(1 - par) * kDig * kTcRows * F.ld;
         const int ksteps = (F.half[1 - par] + 15) / 16;
         for (int base = 0; base < per; base += kTcTiles) {
             float acc[kTcTiles][kDig][4];
@@ -284,7 +306,7 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
                 unsigned af[kDig][4];
 #pragma unroll
                 for (int k = 0; k < kDig; ++k)
-                    ldsm_a(af[k], Ap + ((size_t)k * kTcRows + (lane & 15)) * F.ld + ks * 16 + (lane >> 4) * 8);
+                    ldsm_a(af[k], A + ((size_t)k * kTcRows + (lane & 15)) * F.ld + ks * 16 + (lane >> 4) * 8);
 #pragma unroll
                 for (int t = 0; t < kTcTiles; ++t) {
                     if (t >= ntl) break;
@@ -312,36 +334,44 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
                     const int b = 2 * n + par, v = (int)(R / nimg), img = (int)(R % nimg);
                     const FF s1 = two_sum(acc[t][0][c], acc[t][1][c] * 0x1p-8f);
                     const FF s2 = two_sum(s1.h, acc[t][2][c] * 0x1p-16f);
-                    const float sc = sscale[row];
-                    const FF sum = two_sum(s2.h, __fadd_rn(__fadd_rn(s1.l, s2.l),
-                                                           fmaf(acc[t][4][c], 0x1p-32f, acc[t][3][c] * 0x1p-24f)));
-                    const FF far = ff_mul(FF{sum.h * sc, sum.l * sc}, ipi2);
+                    const FF s3 = two_sum(s2.h, acc[t][3][c] * 0x1p-24f);
+                    const float scale = sscale[row];
+                    const FF sum = two_sum(s3.h, __fadd_rn(__fadd_rn(s1.l, __fadd_rn(s2.l, s3.l)),
+                                                           fmaf(acc[t][5][c], 0x1p-40f, acc[t][4][c] * 0x1p-32f)));
+                    const FF far = ff_mul(FF{sum.h * scale, sum.l * scale}, ipi2);
                     const FF q = ff_mul(FF{m[((int64_t)img * nv + v) * nb + b], 0.f}, cw[b]);
-                    const FF o = ff_mul(ff_add(FF{0.25f * q.h, 0.25f * q.l}, FF{-far.h, -far.l}), ids);
-                    qf[((int64_t)v * nb + b) * width + img] = __fadd_rn(o.h, o.l);
+                    const FF d = ff_add(FF{0.25f * q.h, 0.25f * q.l}, FF{-far.h, -far.l});
+                    if (fabsf(d.h) >= slim[row]) {
+                        const FF o = ff_mul(d, ids);
+                        qf[((int64_t)v * nb + b) * width + img] = __fadd_rn(o.h, o.l);
+                    } else {
+                        atomicOr(&todo[row * F.nw + (b >> 5)], 1u << (b & 31));
+                    }
                 }
         }
     }
+    // what is left to FP64: the row's q over the digits, a warp per output, its lanes over the taps
     __syncthreads();
-    if (!any_bad) return;
-    // rows with non-finite, very small or very large values: FP64 sums, taps in the order of k_fbp_filter
+    double *q = reinterpret_cast<double *>(dyn);
+    const double h0 = 1.0 / (4.0 * ds * ds);
     for (int row = 0; row < kTcRows; ++row) {
-        if (sscale[row] != 0.f || R0 + row >= rows) continue;
+        unsigned *bits = todo + row * F.nw;
+        if (!__syncthreads_or(threadIdx.x < F.nw && bits[threadIdx.x] != 0u)) continue;
         const int v = (int)((R0 + row) / nimg), img = (int)((R0 + row) % nimg);
         const float *src = m + ((int64_t)img * nv + v) * nb;
-        auto q = [&](int b) { return (double)src[b] * ((double)cw[b].h + (double)cw[b].l); };
-        for (int b = threadIdx.x; b < nb; b += kTcThreads) {
-            double acc = 0.0;
-            for (int j = max(b, nb - 1 - b) / 2; j >= 0; --j) {
-                const int d = 2 * j + 1;
-                double pair = 0.0;
-                if (b - d >= 0) pair += q(b - d);
-                if (b + d < nb) pair += q(b + d);
-                acc = fma(-1.0 / (9.869604401089358 * (double)d * (double)d * ds * ds), pair, acc);
+        for (int b = threadIdx.x; b < nb; b += kTcThreads) q[b] = (double)src[b] * cwd[b];
+        __syncthreads();
+        for (int w = warp; w < F.nw; w += kTcWarps)
+            for (unsigned left = bits[w]; left != 0u; left &= left - 1u) {
+                const int b = w * 32 + __ffs(left) - 1;
+                double acc = 0.0;
+#pragma unroll 4
+                for (int i = 1 - (b & 1) + 2 * lane; i < nb; i += 64) acc = fma(tap[abs(i - b) >> 1], q[i], acc);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+                if (lane == 0)
+                    qf[((int64_t)v * nb + b) * width + img] = (float)(ds * fma(h0, q[b], acc));
             }
-            acc = fma(1.0 / (4.0 * ds * ds), q(b), acc);
-            qf[((int64_t)v * nb + b) * width + img] = (float)(ds * acc);
-        }
     }
 }
 
@@ -497,18 +527,21 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
     int width = 1;  // images per pass: the next power of two >= min(batch, 64)
     while (width < std::min(batch, kMaxBatchImages)) width *= 2;
     const size_t nr = (size_t)g.n_views * g.n_bins, qbytes = (sizeof(float) * nr * width + 255) & ~(size_t)255;
+    const int nodd = g.n_bins / 2 + 1;
     char *base = nullptr;
-    DECT_CUDA(cudaMallocAsync((void **)&base, qbytes + sizeof(ViewGeo) * g.n_views, s));
+    DECT_CUDA(cudaMallocAsync((void **)&base,
+                              qbytes + sizeof(ViewGeo) * g.n_views + sizeof(double) * (size_t)(g.n_bins + nodd), s));
     float *qf = (float *)base;
     ViewGeo *vg = (ViewGeo *)(base + qbytes);
+    double *cwd = (double *)(vg + g.n_views), *tap = cwd + g.n_bins;
     const FilterShape F = filter_shape(g.n_bins);
-    const bool tc = F.smem <= kTcSmemMax;  // up to about 1170 bins
+    const bool tc = g.n_bins <= kTcMaxBins;
     cudaError_t e = cudaFuncSetAttribute(k_fbp_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fbp_filter_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
     const FF t0 = ff_of(-0.5 * (double)(g.n_bins - 1) + g.det_offset_mm / g.pitch_mm);
     if (e == cudaSuccess) {
-        k_fbp_views<<<(g.n_views + 255) / 256, 256, 0, s>>>(g, vg);
+        k_fbp_tables<<<(std::max(g.n_views, g.n_bins) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap);
         count_launches(1);
     }
     for (int done = 0; done < batch && e == cudaSuccess; done += kMaxBatchImages) {
@@ -519,7 +552,7 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
         while (w < k) w *= 2;
         if (tc)
             k_fbp_filter_tc<<<(unsigned)(((int64_t)g.n_views * k + kTcRows - 1) / kTcRows), kTcThreads, F.smem, s>>>(
-                mk, qf, g, k, w);
+                mk, qf, cwd, tap, g, k, w);
         else
             k_fbp_filter<<<dim3(g.n_views, k), kFbpBlock, smem, s>>>(mk, qf, g, w);
         switch (w) {
