@@ -35,9 +35,10 @@
 // before the rounding on CT rows, and 2.5e-7 beside such a bin.)
 //
 // Back-projection.  The bin coordinate t reaches n_bins - 1 and its rounding
-// moves the interpolation weights, so the per-pixel geometry is formed in two
-// FP32 words (about 2^-44 of t), once per pixel and view for all images (it
-// was FP64, once per four images: 10.4 ms of the above case).
+// moves the interpolation weights, so the per-pixel geometry (t and the weight
+// (SOD / L)^2 dtheta / 2) is formed in two FP32 words (about 2^-44 of t) and rounded
+// once, once per pixel and view for all images (it was FP64, once per four
+// images: 10.4 ms of the above case).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict_
     const FF px = ff_of(((double)j + 0.5 - 0.5 * (double)n) * g.pixel_mm);
     const FF py = ff_of(((double)i + 0.5 - 0.5 * (double)n) * g.pixel_mm);
     const FF sod = ff_of(g.sod_mm);
-    const float half_dth = (float)(0.5 * g.arc_rad / (double)nv), sodf = (float)g.sod_mm;
+    const FF half_dth = ff_of(0.5 * g.arc_rad / (double)nv);
     const float tmax = (float)(nb - 1);
     float acc[S::IPL];
 #pragma unroll
@@ -442,7 +443,12 @@ __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict_
                     b0 -= 1.f;
                     w = 1.f;
                 }
-                const float r = sodf * rc, wt = half_dth * r * r;
+                // weight half_dth (sod / L)^2, rounded once
+                FF r;
+                r.h = __fmul_rn(sod.h, rc);
+                r.l = __fmul_rn(rc, __fadd_rn(fmaf(-r.h, L.h, sod.h), fmaf(-r.h, L.l, sod.l)));
+                const FF wt2 = ff_mul(half_dth, ff_mul(r, r));
+                const float wt = __fadd_rn(wt2.h, wt2.l);
                 int bi = (int)b0;
                 if (!DECT_IDX_OK(bi, nb - 1, CHK_FBP_BIN)) bi = 0;
                 ray[e] = v * nb + bi;

@@ -68,3 +68,18 @@ def test_rows_share_a_block_with_rows_of_other_ranges():
     for k in range(len(m)):
         one = dect.fbp(plan, torch.tensor(m[k][None, None], device="cuda"))[0]
         assert torch.equal(torch.nan_to_num(x[k]), torch.nan_to_num(one)), k
+
+
+@pytest.mark.parametrize("n,batch", [(33, 1), (301, 2), (64 * 4 + 1, 9)])
+def test_pixel_weights_are_rounded_once(n, batch):
+    """The row of pixels through the isocentre sees one bin, with interpolation weight 1, at every distance from
+    the source.  That bin holds a power of two: the result is (SOD / L)^2 dtheta / 2 rounded to FP32, half a unit
+    in the last place off (and 2^-20 of that for the two words)."""
+    g = synth.tiny_geometry(n=n, nv=1, nb=17, px=0.7, pitch=2.0, sod=333.3, sdd=666.6)
+    m = np.zeros((batch, 1, 17), np.float32)
+    m[:, 0, 8] = 2.0 ** np.arange(batch)
+    x = dect.fbp(dect.Plan(g), torch.tensor(m, device="cuda")).cpu().numpy().astype(np.float64)
+    r = g.sod / (g.sod - (np.arange(n) + 0.5 - 0.5 * n) * g.px)
+    for k in range(batch):
+        want = np.pi * r * r * 2.0 ** k / 4
+        assert (np.abs(x[k, n // 2] - want) <= 2.0 ** -24 * (1 + 2.0 ** -20) * want).all()
