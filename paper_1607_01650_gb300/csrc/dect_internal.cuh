@@ -88,7 +88,7 @@ struct LineTable {
     int nbp;         // row stride of q and walk, bins rounded up to 32
     int nblk;        // blocks of 32 lines
     int ngb;         // groups of 32 rays of a view, nbp / 32
-    float *q;        // [nv][nblk][nbp / 32][32 lines][32 rays] fraction of the ray's length in column c
+    float *q;        // [nv][nblk][nbp / 32][32 lines][32 rays] fractions of the ray's length in columns c and c + 1 (lines.cuh)
     uint2 *walk;     // [nv][nblk][nbp] columns of 32 lines of a ray
     float2 *len;     // [nv * nb] length of the ray in a line, in two words
     unsigned char *cls;  // [nv * nb] class of the ray

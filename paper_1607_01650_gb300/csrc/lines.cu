@@ -14,7 +14,7 @@ constexpr short kColOut = -32768;  // as in plan.cu
 constexpr int kMaxN = 4096;
 
 // One thread per (view, block of 32 lines, bin).  A line outside the image
-// counts as column -1 (q = 1) or n - 1 (q = 0), neither of which adds anything.
+// counts as column -1 (q = 1: -0) or n - 1 (q = 0), neither of which adds anything.
 __global__ void __launch_bounds__(256) k_line_walk(LineTable T, const short *__restrict__ col, int *__restrict__ bad)
 {
     const int b = blockIdx.x * 256 + threadIdx.x, blk = blockIdx.y, v = blockIdx.z;
@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(256) k_line_walk(LineTable T, const short *__r
     const int ns = min(32, T.n - blk * 32);
     auto column = [&](int k) {
         const short c = col[at + k * 32];
-        return c != kColOut ? (int)c : T.q[at + k * 32] == 1.f ? -1 : T.n - 1;
+        return c != kColOut ? (int)c : __float_as_int(T.q[at + k * 32]) < 0 ? -1 : T.n - 1;
     };
     int prev = column(0), sign = 0;
     const unsigned first = (unsigned)(prev + 1);

@@ -4,9 +4,11 @@
 // A ray with |dx| <= |dy| ("class 0") crosses the image line by line along the
 // rows: in row i it meets at most two pixels, (i, c) and (i, c + 1), and its
 // length inside the row is the same in every row.  The table holds, per view,
-// line and ray, the fraction q of that length that lies in pixel c (the rest
-// lies in c + 1), 4 bytes per ray and line, and per ray the length L (two words):
-//   y = L sum over the lines of q x[c] + (1 - q) x[c + 1].
+// line and ray, which fraction of that length lies in pixel c and which in
+// c + 1, 4 bytes per ray and line, and per ray the length L (two words):
+//   y = L sum over the lines of q x[c] + p x[c + 1],  q + p = 1.
+// Stored is the smaller fraction, with a minus sign if that is p, so that a piece of
+// any size keeps its 24 bits (q itself, with p = 1 - q, held small p to 2^-25 of L).
 // Rays with |dx| > |dy| ("class 1") are stored the same way with rows and columns
 // exchanged, and gather from a transposed copy of the image.  Columns outside
 // the image stand for the part of a line that a ray spends outside it.
@@ -67,10 +69,20 @@ __device__ __forceinline__ void l2_prefetch(const void *p, unsigned bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
+// The fractions (q, p) of an entry of the table, and the entry of given fractions.
+__device__ __forceinline__ void line_weights(float v, float &q, float &p)
+{
+    const float small = fabsf(v), large = 1.f - small;
+    const bool neg = __float_as_int(v) < 0;
+    q = neg ? large : small;
+    p = neg ? small : large;
+}
+__device__ __forceinline__ float line_entry(double q, double p) { return q <= p ? (float)q : -(float)p; }
+
 inline int line_groups(const LineTable &T) { return T.nv * T.ngb; }
 
 // The 32 lines of a block, none of whose columns lies outside the image: sum of
-// q x[c] + (1 - q) x[c + 1].  q: the ray's entry of the tile's first line.
+// q x[c] + p x[c + 1].  qt: the ray's entry of the tile's first line.
 template <int NB>
 __device__ __forceinline__ void line_block(const float *__restrict__ x, const float *__restrict__ qt, int n, int s0,
                                            const uint2 &w, float (&acc)[LineShape<NB>::VW])
@@ -103,9 +115,10 @@ __device__ __forceinline__ void line_block(const float *__restrict__ x, const fl
         for (int t = 0; t < VW; ++t) sum[t] = 0.f;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const float p = 1.f - q[u];
+            float a, b;
+            line_weights(q[u], a, b);
 #pragma unroll
-            for (int t = 0; t < VW; ++t) sum[t] = fmaf(q[u], lo[u].v[t], fmaf(p, hi[u].v[t], sum[t]));
+            for (int t = 0; t < VW; ++t) sum[t] = fmaf(a, lo[u].v[t], fmaf(b, hi[u].v[t], sum[t]));
         }
 #pragma unroll
         for (int t = 0; t < VW; ++t) acc[t] += sum[t];
@@ -130,9 +143,9 @@ __device__ __forceinline__ void line_block_edge(const float *__restrict__ x, con
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const bool on = k0 + u < ns;
-            q[u] = on ? __ldg(qt + (k0 + u) * 32) : 0.f;
-            p[u] = on && c + 1 < n ? 1.f - q[u] : 0.f;
-            q[u] = c >= 0 ? q[u] : 0.f;
+            line_weights(on ? __ldg(qt + (k0 + u) * 32) : 0.f, q[u], p[u]);
+            if (!on || c + 1 >= n) p[u] = 0.f;
+            if (c < 0) q[u] = 0.f;
             const int c0 = max(c, 0), c1 = min(c + 1, n - 1);
             lo[u] = ld_il<VW>(row + (int64_t)c0 * NB);
             hi[u] = ld_il<VW>(row + (int64_t)c1 * NB);
@@ -161,7 +174,8 @@ __device__ __noinline__ void line_block_careful(const float *x, const float *qt,
     int c = (int)(w.x & 0xffffu) - 1;
     const int dir = (w.x & kWalkFalls) ? -1 : 1, ns = min(32, n - s0);
     for (int k = 0; k < ns; ++k) {
-        const float q = __ldg(qt + k * 32), p = 1.f - q;
+        float q, p;
+        line_weights(__ldg(qt + k * 32), q, p);
         const float *row = x + (int64_t)(s0 + k) * n * NB;
         if (c >= 0 && c < n && q != 0.f) {
             const Vec<VW> v = ld_il<VW>(row + (int64_t)c * NB);

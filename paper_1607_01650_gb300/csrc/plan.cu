@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "dect_internal.cuh"
+#include "lines.cuh"
 
 namespace dect {
 namespace {
@@ -191,7 +192,8 @@ __global__ void k_siddon_count(const RayPts *__restrict__ rays, int64_t M, Grid 
 // Fills a ray's row of the CSR table and, with T.ok, its lines of the line
 // table: q, and in col (laid out like q) the column c of each line, or kColOut
 // where the ray does not meet the line inside the image (then q = 1 left and
-// 0 right of it).  *bad: a line that does not fit the form.
+// 0 right of it).  Pieces shorter than 1e-10 of L, which rounding of the walk may
+// make or swallow, are left out.  *bad: a line that does not fit the form.
 constexpr short kColOut = -32768;
 
 struct LineFill {
@@ -222,10 +224,11 @@ struct LineFill {
         T.len[ray] = make_float2((float)L, (float)(L - (double)(float)L));
         T.cls[ray] = (unsigned char)cls;
     }
-    __device__ void put(int ln, short c, float q)
+    // fractions qf in column c and pf in c + 1
+    __device__ void put(int ln, short c, double qf, double pf)
     {
         const int64_t o = T.at(v, ln, b);
-        T.q[o] = q;
+        T.q[o] = line_entry(qf, pf);
         col[o] = c;
     }
     // lines from `next` up to (not including) ln lie outside the image for this ray
@@ -234,7 +237,7 @@ struct LineFill {
         for (; next != ln; next += up ? 1 : -1) {
             const double mid = lo + ((double)next + 0.5) * px;
             const double x = cls ? r.sy + (mid - r.sx) / dx * dy : r.sx + (mid - r.sy) / dy * dx;
-            put(next, kColOut, x < 0.0 ? 1.f : 0.f);
+            put(next, kColOut, x < 0.0 ? 1.0 : 0.0, x < 0.0 ? 0.0 : 1.0);
         }
     }
     __device__ void flush()
@@ -247,14 +250,14 @@ struct LineFill {
         next += up ? 1 : -1;
         const bool two = l1 >= 1e-10 * L, one = l0 >= 1e-10 * L;
         if (full) {
-            if (two && one) put(line, (short)c0, (float)(l0 / tot));
-            else put(line, (short)(one ? c0 : c0 + 1), 1.f);
+            if (two && one) put(line, (short)c0, l0 / tot, l1 / tot);
+            else put(line, (short)(one ? c0 : c0 + 1), 1.0, 0.0);
         } else if (!two && c0 == 0) {  // enters or leaves through the low side in this line
-            put(line, -1, (float)(1.0 - l0 / L));
+            put(line, -1, 1.0 - l0 / L, l0 / L);
         } else if (!(two && one) && c0 + (two ? 1 : 0) == T.n - 1) {  // through the high side
-            put(line, (short)(T.n - 1), (float)(tot / L));
+            put(line, (short)(T.n - 1), tot / L, 1.0 - tot / L);
         } else {
-            put(line, kColOut, 1.f);
+            put(line, kColOut, 1.0, 0.0);
             bad = true;
         }
     }
