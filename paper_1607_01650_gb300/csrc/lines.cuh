@@ -238,12 +238,16 @@ __device__ __forceinline__ void line_ray_sums(const LineTable &T, int v, int gb,
         fine = fine && isfinite(acc[k]);
     }
     if (fine) return;
+    float sum[VW];
 #pragma unroll
-    for (int k = 0; k < VW; ++k) acc[k] = 0.f;
+    for (int k = 0; k < VW; ++k) sum[k] = 0.f;
     for (int blk = part; blk < T.nblk; blk += PARTS) {
         const uint2 now = __ldg(walk + (int64_t)blk * T.nbp);
-        line_block_careful<NB>(((now.x & kWalkCls1) ? srcT : src) + img, q + blk * tile, n, blk * 32, now, acc);
+        line_block_careful<NB>(((now.x & kWalkCls1) ? srcT : src) + img, q + blk * tile, n, blk * 32, now, sum);
     }
+#pragma unroll
+    for (int k = 0; k < VW; ++k)  // images that are finite keep their sums
+        if (!isfinite(acc[k])) acc[k] = sum[k];
 }
 
 // The block's sums of all 32 rays, [part][ray][NB].

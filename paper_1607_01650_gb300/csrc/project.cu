@@ -103,6 +103,9 @@ __global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict_
 // share an L1; otherwise rows are taken in order (adjacent rays of a view share
 // pixels).  Lanes gather 8 images of an entry above 16 images (row_dot_w), 4
 // below (row_dot_g).
+//   row_dot pads a row with entries of weight 0 at index 0, whose product with a
+// value there that is not finite is not 0: a block with a sum that is not finite
+// goes over its rows once more, without padding.
 template <int NB, bool TILED>
 __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict__ ptr, const Entry *__restrict__ ent,
                                                       int64_t rows, int n, int nz, const float *__restrict__ src,
@@ -110,15 +113,16 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
 {
     constexpr int G = kLanes<NB>, VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
     constexpr int TW = kTileW, TH = kOpBlock / G > 64 ? kOpBlock / G / TW : 8;
+    constexpr unsigned SITE = TILED ? CHK_GATHER_AT : CHK_GATHER_A;
     const int lr = threadIdx.x % G, grp = lr / LPE, vl = lr % LPE;
     const int64_t rpb = kOpBlock / G;
     const int tiles_x = (n + TW - 1) / TW, tiles_y = (n + TH - 1) / TH;
     const int64_t per_slice = (int64_t)tiles_x * tiles_y * TW * TH;
     const int64_t vrows = TILED ? per_slice * nz : rows;
     const unsigned long long pol = l2_evict_last_policy();
-    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
-        const int64_t v = v0 + threadIdx.x / G;
-        int64_t row = v;
+    // row v of the block's walk: its index (false: none) and its entries [b, e)
+    auto locate = [&](int64_t v, int64_t &row, int64_t &b, int64_t &e) {
+        row = v;
         bool ok = v < vrows;
         if (TILED && ok) {  // slice k, tile of the slice, pixel of the tile
             const int64_t k = v / per_slice, vs = v % per_slice;
@@ -128,17 +132,50 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
             ok = i < n && j < n;
             row = (k * n + i) * n + j;
         }
-        int64_t b = 0, e = 0;
+        b = e = 0;
         if (ok) {
             b = ptr[row];
             e = ptr[row + 1];
         }
+        return ok;
+    };
+    float zero = 0.f;  // stays 0 while every sum is finite
+    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
+        int64_t row, b, e;
+        const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
         Vec<VW> acc;
         if constexpr (NB > 16)
-            acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
+            acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, SITE);
         else
-            acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
+            acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, SITE);
+#pragma unroll
+        for (int c = 0; c < VW; ++c) zero = fmaf(acc.v[c], 0.f, zero);
         if (ok && grp == 0) st_v<VW>(dst + row * NB + vl * VW, acc);
+    }
+    if (__syncthreads_and(zero == 0.f)) return;
+    const GatherIL<NB> gather{src, src_rows, SITE};
+    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
+        int64_t row, b, e;
+        const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
+        Vec<VW> acc;
+        acc.zero();
+        for (int64_t k = b + grp; k < e; k += G / LPE) {
+            const Entry en = ld_entry(ent + k);
+            const Vec<VW> xv = gather(en.x, vl);
+#pragma unroll
+            for (int c = 0; c < VW; ++c) acc.v[c] = fmaf(__int_as_float(en.y), xv.v[c], acc.v[c]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int off = LPE; off < G; off <<= 1)
+#pragma unroll
+            for (int c = 0; c < VW; ++c) acc.v[c] += __shfl_xor_sync(0xffffffffu, acc.v[c], off);
+        if (ok && grp == 0) {
+            float *o = dst + row * NB + vl * VW;  // written by this thread
+#pragma unroll
+            for (int c = 0; c < VW; ++c)
+                if (!isfinite(o[c])) o[c] = acc.v[c];
+        }
     }
 }
 
