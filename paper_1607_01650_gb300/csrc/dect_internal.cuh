@@ -147,10 +147,7 @@ cudaError_t launch_backproject_planar(const dect_plan *p, const float *y, float 
 // the form cannot hold or memory is short; the Siddon fill (plan.cu) then writes
 // q and the columns, and lines_finish the walk words.  *d_bad (device, zeroed by
 // the caller) becomes non-zero where the rays do not fit the form.
-struct RayPts {
-    double sx, sy, dx_, dy_;
-};
-cudaError_t lines_alloc(LineTable &T, int n, int nv, int nb, cudaStream_t s);
+cudaError_t lines_alloc(LineTable &T, int n, int nv, int nb);
 cudaError_t lines_finish(LineTable &T, const short *d_col, int *d_bad, cudaStream_t s);
 void lines_free(LineTable &T);
 

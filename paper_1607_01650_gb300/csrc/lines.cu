@@ -58,7 +58,7 @@ void lines_free(LineTable &T)
     T = LineTable{};
 }
 
-cudaError_t lines_alloc(LineTable &T, int n, int nv, int nb, cudaStream_t s)
+cudaError_t lines_alloc(LineTable &T, int n, int nv, int nb)
 {
     T = LineTable{};
     if (n < 4 || n > kMaxN || nv > 65535) return cudaSuccess;

@@ -28,6 +28,11 @@ namespace {
 
 __device__ constexpr double kInf = __builtin_huge_val();
 
+// Ray end points, FP64: (Sx, Sy, Dx, Dy).
+struct RayPts {
+    double sx, sy, dx_, dy_;
+};
+
 struct Grid {
     int n;
     double px;
@@ -618,28 +623,33 @@ extern "C" dect_status dect_plan_create(const dect_geometry *geom, int device, d
     size_t ne = (size_t)(nnz > 0 ? nnz : 1) + kTablePad;
     PLAN_CUDA(cudaMalloc(&p->ent, sizeof(Entry) * ne));
     PLAN_CUDA(cudaMemsetAsync(p->ent, 0, sizeof(Entry) * ne, s));
-    // the line table, where its form can hold and memory allows
-    if (nnz > 0) {
-        PLAN_CUDA(lines_alloc(p->lines, p->n, p->nv, p->nb, s));
-        const size_t ncol = (size_t)p->nv * p->lines.nblk * p->lines.ngb * 1024;
-        if (p->lines.ok && cudaMalloc(&d_col, sizeof(short) * ncol) != cudaSuccess) {
-            cudaGetLastError();
-            lines_free(p->lines);
-        }
-        PLAN_CUDA(cudaMalloc(&d_bad, sizeof(int)));
-        PLAN_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
-    }
-    k_siddon_fill<<<(unsigned)((p->M + T - 1) / T), T, 0, s>>>(d_rays, p->M, g, p->rowptr, p->ent, p->lines, d_col,
-                                                               d_bad);
-    PLAN_CUDA(cudaGetLastError());
-
-    // pixel-major transpose
     PLAN_CUDA(cudaMalloc(&d_ccnt, sizeof(int) * p->N));
     PLAN_CUDA(cudaMalloc(&d_cursor, sizeof(int) * p->N));
     PLAN_CUDA(cudaMalloc(&d_ccnt64, sizeof(int64_t) * p->N));
     PLAN_CUDA(cudaMalloc(&p->colptr, sizeof(int64_t) * (p->N + 1)));
     PLAN_CUDA(cudaMalloc(&d_tmp, sizeof(Entry) * ne));
     PLAN_CUDA(cudaMalloc(&p->tent, sizeof(Entry) * ne));
+    PLAN_CUDA(cudaMalloc(&d_bad, sizeof(int)));
+    PLAN_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
+    // the line table, where its form can hold: after all that the plan cannot do
+    // without, and given back where memory runs short all the same
+    auto drop_lines = [&]() {
+        cudaStreamSynchronize(s);
+        cudaGetLastError();
+        cudaFree(d_col);
+        d_col = nullptr;
+        lines_free(p->lines);
+    };
+    if (nnz > 0) {
+        PLAN_CUDA(lines_alloc(p->lines, p->n, p->nv, p->nb));
+        const size_t ncol = (size_t)p->nv * p->lines.nblk * p->lines.ngb * 1024;
+        if (p->lines.ok && cudaMalloc(&d_col, sizeof(short) * ncol) != cudaSuccess) drop_lines();
+    }
+    k_siddon_fill<<<(unsigned)((p->M + T - 1) / T), T, 0, s>>>(d_rays, p->M, g, p->rowptr, p->ent, p->lines, d_col,
+                                                               d_bad);
+    PLAN_CUDA(cudaGetLastError());
+
+    // pixel-major transpose
     PLAN_CUDA(cudaMemsetAsync(p->tent, 0, sizeof(Entry) * ne, s));
     PLAN_CUDA(cudaMemsetAsync(d_ccnt, 0, sizeof(int) * p->N, s));
     PLAN_CUDA(cudaMemsetAsync(d_cursor, 0, sizeof(int) * p->N, s));
@@ -649,7 +659,12 @@ extern "C" dect_status dect_plan_create(const dect_geometry *geom, int device, d
     }
     k_int_to_i64<<<(unsigned)((p->N + 255) / 256), 256, 0, s>>>(d_ccnt, p->N, d_ccnt64);
     PLAN_CUDA(cudaGetLastError());
-    PLAN_CUDA(scan_exclusive(d_ccnt64, p->N, p->colptr, s));
+    cudaError_t se = scan_exclusive(d_ccnt64, p->N, p->colptr, s);
+    if (se == cudaErrorMemoryAllocation && p->lines.ok) {
+        drop_lines();
+        se = scan_exclusive(d_ccnt64, p->N, p->colptr, s);
+    }
+    PLAN_CUDA(se);
     if (nnz > 0) {
         k_col_scatter<<<(unsigned)((p->M + T - 1) / T), T, 0, s>>>(p->rowptr, p->ent, p->M, p->colptr,
                                                                    d_cursor, d_tmp);
