@@ -476,7 +476,8 @@ dect_status dect_adm_tv_ex(const dect_plan *plan, const float *m, float *x, int 
  * Autotuner record of a plan: the A^T variant that dect_adm_tv chose for a
  * batch of `images` interleaved channels (2, 4, 8, 16, 32 or 64; a call with
  * c channels uses the next of these widths >= min(c, 64)), and the measured
- * median time of each variant in microseconds (-1 = not available):
+ * time of each variant in microseconds (the median of three launches, or the
+ * smaller of two where both are behind the fastest so far; -1 = not available):
  *   0-2 L1-cached gather with 4x4 / 8x8 / 16x16 pixel tiles per 256-thread block,
  *   3   at 16 channels eight lanes per pixel, one 1024-thread block per SM over
  *       8x32 tiles; otherwise none (falls back to 1),

@@ -52,6 +52,7 @@
 #include "dect_internal.cuh"
 #include "kernels.cuh"
 #include "lines.cuh"
+#include "tune.h"
 
 namespace dect {
 namespace {
@@ -1105,7 +1106,7 @@ struct Kern {
 // 0 lanes gather 4 images of an entry; 1 lanes gather 8 images (row_dot_w),
 // four rounds of gathers in flight; 2 as 1 with two rounds (below 16 images
 // 1 and 2 fall back to 0).  3 the line table (NB <= 16; otherwise 2).
-constexpr int kFwdVariants = DECT_FWD_VARIANTS, kFwdLines = 3;
+constexpr int kFwdLines = 3;
 
 struct Work {
     float *f[2], *G, *lam, *z, *p, *r, *q, *beta;
@@ -1175,7 +1176,6 @@ void launch_residual_check(const dect_plan *P, const Work &W, const float *f_cur
 // / 16 x 16 at 16, 8 x 32 / 16 x 32 at 8), whose lines then stay in one L1; 6-7 lanes gather 8
 // images of an entry (row_dot_w, NB >= 16 only): 6 with the lanes and tiles
 // of 4; 7 with 16 lanes per pixel (two pixels per warp) over 8 x 8 tiles.
-constexpr int kBwdVariants = DECT_BWD_VARIANTS;
 
 template <int NB>
 void launch_bwd(const dect_plan *P, const Work &W, const AdmConst &C, int variant, cudaStream_t s)
@@ -1223,110 +1223,83 @@ constexpr int nb_index()
     return NB == 2 ? 0 : NB == 4 ? 1 : NB == 8 ? 2 : NB == 16 ? 3 : NB == 32 ? 4 : 5;
 }
 
-// A variant whose first timed launch takes this many times the best is out without two more
-constexpr float kTuneClear = 1.15f;
-
-// Time every available A^T variant on this workspace (CUDA events, median of
-// three launches after one warm-up) and keep the fastest in the plan.  The
-// kernels only write G and reduction slots, which the first iteration
-// rewrites, so timing them here changes no result.
-template <int NB>
-cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t s)
+// Time the variants v with avail(v) (CUDA events; each launched once before it is
+// timed) and put their times into us (-1: not available) and the fastest into choice.
+template <int COUNT, typename Avail, typename Launch>
+cudaError_t tune_variants(cudaStream_t s, float (&us)[COUNT], int &choice, Avail avail, Launch launch)
 {
-    const int idx = nb_index<NB>();
-    if (P->bwd_choice[idx] >= 0) {
-        W.bwd = P->bwd_choice[idx];
-        if (W.bwd == 3 && NB != 16) W.bwd = 1;
-        if (W.bwd >= 6 && NB < 16) W.bwd = 4;
-        return cudaSuccess;
-    }
     cudaEvent_t a = nullptr, b = nullptr;
     cudaError_t e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
-    int best = 1;
-    float best_us = 1e30f;
-    for (int v = 0; v < kBwdVariants && e == cudaSuccess; ++v) {
-        P->bwd_us[idx][v] = -1.f;
-        if (v == 3 && NB != 16) continue;
-        if (v >= 6 && NB < 16) continue;  // wide-lane variants need 16 images
-        launch_bwd<NB>(P, W, C, v, s);
+    auto sample = [&](int v, float &t) {
+        e = cudaEventRecord(a, s);
+        launch(v);
         count_launches(1);
-        float t[3];
-        for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-            e = cudaEventRecord(a, s);
-            launch_bwd<NB>(P, W, C, v, s);
-            count_launches(1);
-            if (e == cudaSuccess) e = cudaEventRecord(b, s);
-            if (e == cudaSuccess) e = cudaEventSynchronize(b);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], a, b);
-            if (k == 0 && t[0] * 1e3f > kTuneClear * best_us) t[1] = t[2] = t[0], k = 3;
-        }
-        if (e != cudaSuccess) break;
-        std::sort(t, t + 3);
-        const float us = t[1] * 1e3f;
-        P->bwd_us[idx][v] = us;
-        if (us < best_us) {
-            best_us = us;
+        if (e == cudaSuccess) e = cudaEventRecord(b, s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(b);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&t, a, b);
+        t *= 1e3f;
+        return e == cudaSuccess;
+    };
+    int best = -1;
+    float best_us = 1e30f;
+    for (int v = 0; v < COUNT && e == cudaSuccess; ++v) {
+        us[v] = -1.f;
+        if (!avail(v)) continue;
+        launch(v);
+        count_launches(1);
+        float t = 0.f;
+        if (!median_time(best_us, [&](float &x) { return sample(v, x); }, t)) break;
+        us[v] = t;
+        if (t < best_us) {
+            best_us = t;
             best = v;
         }
     }
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    P->bwd_choice[idx] = best;
-    W.bwd = best;
+    if (e == cudaSuccess) choice = best;
+    return e;
+}
+
+// Time every available A^T variant on this workspace and keep the fastest in
+// the plan.  The kernels only write G and reduction slots, which the first
+// iteration rewrites, so timing them here changes no result.
+template <int NB>
+cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t s)
+{
+    const int idx = nb_index<NB>();
+    if (P->bwd_choice[idx] < 0) {
+        // 3 needs 16 images, 6 and 7 at least 16
+        const cudaError_t e = tune_variants(
+            s, P->bwd_us[idx], P->bwd_choice[idx], [](int v) { return v == 3 ? NB == 16 : v < 6 || NB >= 16; },
+            [&](int v) { launch_bwd<NB>(P, W, C, v, s); });
+        if (e != cudaSuccess) return e;
+    }
+    W.bwd = P->bwd_choice[idx];
+    if (W.bwd == 3 && NB != 16) W.bwd = 1;
+    if (W.bwd >= 6 && NB < 16) W.bwd = 4;
     return cudaSuccess;
 }
 
-// Time every A variant on the set-up projection r = A f - beta m (CUDA
-// events, median of three launches after one warm-up) and keep the fastest
-// in the plan.  The caller runs the set-up projection again afterwards with
+// Time every A variant on the set-up projection r = A f - beta m and keep the
+// fastest in the plan.  The caller runs the set-up projection again afterwards with
 // the chosen variant (the variants sum in different orders).
 template <int NB>
 cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t s)
 {
     const int idx = nb_index<NB>();
-    if (P->fwd_choice[idx] >= 0) {
-        W.fwd = P->fwd_choice[idx];
-        if (W.fwd == kFwdLines && !W.GT) W.fwd = NB >= 16 ? 2 : 0;
-        return cudaSuccess;
+    if (P->fwd_choice[idx] < 0) {
+        // of 0-2 only 0 below 16 images
+        const cudaError_t e = tune_variants(
+            s, P->fwd_us[idx], P->fwd_choice[idx],
+            [&](int v) { return v == kFwdLines ? W.GT != nullptr : v == 0 || NB >= 16; },
+            [&](int v) { launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s); });
+        if (e != cudaSuccess) return e;
     }
-    cudaEvent_t a = nullptr, b = nullptr;
-    cudaError_t e = cudaEventCreate(&a);
-    if (e == cudaSuccess) e = cudaEventCreate(&b);
-    int best = 0;
-    float best_us = 1e30f;
-    for (int v = 0; v < kFwdVariants && e == cudaSuccess; ++v) {
-        P->fwd_us[idx][v] = -1.f;
-        if (v == kFwdLines ? !W.GT : v > 0 && NB < 16) continue;  // of the others only 0 below 16 images
-        launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
-        count_launches(1);
-        float t[3];
-        for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-            e = cudaEventRecord(a, s);
-            launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
-            count_launches(1);
-            if (e == cudaSuccess) e = cudaEventRecord(b, s);
-            if (e == cudaSuccess) e = cudaEventSynchronize(b);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], a, b);
-            if (k == 0 && t[0] * 1e3f > kTuneClear * best_us) t[1] = t[2] = t[0], k = 3;
-        }
-        if (e != cudaSuccess) break;
-        std::sort(t, t + 3);
-        const float us = t[1] * 1e3f;
-        P->fwd_us[idx][v] = us;
-        if (us < best_us) {
-            best_us = us;
-            best = v;
-        }
-    }
-    if (a) cudaEventDestroy(a);
-    if (b) cudaEventDestroy(b);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    P->fwd_choice[idx] = best;
-    W.fwd = best;
+    W.fwd = P->fwd_choice[idx];
+    if (W.fwd == kFwdLines && !W.GT) W.fwd = NB >= 16 ? 2 : 0;
     return cudaSuccess;
 }
 
@@ -1334,7 +1307,6 @@ cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
 // counter, rows exchanged through shared memory, one barrier per row); 1
 // k_tv_tma (rows streamed by bulk copies into a ring of stages, NB >= 4); 2
 // k_tv_px (a thread per pixel vector).  All give the same images.
-constexpr int kTvVariants = DECT_TV_VARIANTS;
 
 // Prepare k_tv_tma for this width: its shared memory, and the grid (blocks
 // that fit on an SM x SMs, at most kGrid, whose partials the reduction holds).
@@ -1360,10 +1332,9 @@ cudaError_t setup_tv_tma(Work &W)
 template <int NB>
 void launch_tv(const Work &W, const AdmConst &C, int par, int final_pass, cudaStream_t s);
 
-// Time the TV-step variants (CUDA events, median of three launches after
-// one warm-up) and keep the faster in the plan.  Called before the first
-// iteration (k = 0, alpha = 0), where the step is idempotent: f[1] = f[0],
-// r is unchanged and p (lambda, z) and the two norms are those the first
+// Time the TV-step variants and keep the fastest in the plan.  Called before
+// the first iteration (k = 0, alpha = 0), where the step is idempotent: f[1] =
+// f[0], r is unchanged and p (lambda, z) and the two norms are those the first
 // iteration computes again, so timing changes no result.
 template <int NB>
 cudaError_t tune_tv(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t s)
@@ -1372,45 +1343,15 @@ cudaError_t tune_tv(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t
     if (e != cudaSuccess) return e;
     const int idx = nb_index<NB>();
     const bool tma_ok = NB >= 4 && W.tv_grid > 0;
-    if (P->tv_choice[idx] >= 0) {
-        W.tv = P->tv_choice[idx] == 1 && !tma_ok ? 0 : P->tv_choice[idx];
-        return cudaSuccess;
+    if (P->tv_choice[idx] < 0) {
+        e = tune_variants(s, P->tv_us[idx], P->tv_choice[idx], [&](int v) { return v != 1 || tma_ok; },
+                          [&](int v) {
+                              W.tv = v;
+                              launch_tv<NB>(W, C, 0, 0, s);
+                          });
+        if (e != cudaSuccess) return e;
     }
-    cudaEvent_t a = nullptr, b = nullptr;
-    e = cudaEventCreate(&a);
-    if (e == cudaSuccess) e = cudaEventCreate(&b);
-    int best = 0;
-    float best_us = 1e30f;
-    for (int v = 0; v < kTvVariants && e == cudaSuccess; ++v) {
-        P->tv_us[idx][v] = -1.f;
-        if (v == 1 && !tma_ok) continue;
-        W.tv = v;
-        launch_tv<NB>(W, C, 0, 0, s);
-        count_launches(1);
-        float t[3];
-        for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-            e = cudaEventRecord(a, s);
-            launch_tv<NB>(W, C, 0, 0, s);
-            count_launches(1);
-            if (e == cudaSuccess) e = cudaEventRecord(b, s);
-            if (e == cudaSuccess) e = cudaEventSynchronize(b);
-            if (e == cudaSuccess) e = cudaEventElapsedTime(&t[k], a, b);
-        }
-        if (e != cudaSuccess) break;
-        std::sort(t, t + 3);
-        const float us = t[1] * 1e3f;
-        P->tv_us[idx][v] = us;
-        if (us < best_us) {
-            best_us = us;
-            best = v;
-        }
-    }
-    if (a) cudaEventDestroy(a);
-    if (b) cudaEventDestroy(b);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    P->tv_choice[idx] = best;
-    W.tv = best;
+    W.tv = P->tv_choice[idx] == 1 && !tma_ok ? 0 : P->tv_choice[idx];
     return cudaSuccess;
 }
 
