@@ -1133,10 +1133,8 @@ void launch_fwd(const dect_plan *P, const Work &W, int variant, const float *src
     if constexpr (NB <= kLineMaxImages) {
         if (variant == kFwdLines && W.GT) {
             const LineTable &T = P->lines;
-            if (MODE != 1) {  // (k_bwd writes G's transpose)
+            if (MODE != 1)  // (k_bwd writes G's transpose)
                 k_line_transpose<NB><<<transpose_grid(T.n), 256, 0, s>>>(src, W.GT, T.n);
-                count_launches(1);
-            }
             k_line_fwd<NB, MODE><<<even_grid(line_groups(T), part_blocks<NB>()), LineShape<NB>::BLOCK, 0, s>>>(
                 T, src, W.GT, dst, W.m, W.beta, C, D, rc);
             return;
@@ -1155,6 +1153,12 @@ void launch_fwd(const dect_plan *P, const Work &W, int variant, const float *src
     }
 }
 
+// Kernels that launch_fwd launches.
+int fwd_kernels(const Work &W, int variant, int mode)
+{
+    return variant == kFwdLines && W.GT && mode != 1 ? 2 : 1;
+}
+
 // Exact residual of the current f (f_cur) against the carried one, for the
 // reports: QQ <- |A f - beta m|^2, GG <- |r - (A f - beta m)|^2 (q is
 // overwritten; call only where q is no longer needed).
@@ -1162,7 +1166,7 @@ template <int NB>
 void launch_residual_check(const dect_plan *P, const Work &W, const float *f_cur, const AdmConst &C, cudaStream_t s)
 {
     launch_fwd<NB, 3>(P, W, W.fwd, f_cur, W.q, C, s, W.r);
-    count_launches(1);
+    count_launches(fwd_kernels(W, W.fwd, 3));
 }
 
 // A^T variants (autotuner candidates): 0-2 L1-cached gather with 4x4 (4x8 up to
@@ -1295,7 +1299,10 @@ cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
         const cudaError_t e = tune_variants(
             s, P->fwd_us[idx], P->fwd_choice[idx],
             [&](int v) { return v == kFwdLines ? W.GT != nullptr : v == 0 || NB >= 16; },
-            [&](int v) { launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s); });
+            [&](int v) {
+                launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
+                count_launches(fwd_kernels(W, v, 0) - 1);
+            });
         if (e != cudaSuccess) return e;
     }
     W.fwd = P->fwd_choice[idx];
@@ -1411,7 +1418,10 @@ void enqueue_iteration(const dect_plan *P, const Work &W, const AdmConst &C, int
     if (ev) cudaEventRecordWithFlags(ev->f1, s, cudaEventRecordExternal);
 }
 
-int kernels_per_iteration(const AdmConst &C) { return C.nonneg ? 4 : 3; }
+int kernels_per_iteration(const Work &W, const AdmConst &C)
+{
+    return 3 + (C.nonneg ? fwd_kernels(W, W.fwd, 2) : 0);
+}
 
 // Workspace of one batch width: one allocation, laid out once to size and
 // then for real, zeroed.
@@ -1584,7 +1594,7 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
     if (h_flags) h_flags[0] = 0;
     while (err == cudaSuccess && done_iters + block <= K) {
         err = cudaGraphLaunch(gx_block, cs);
-        count_launches((int64_t)kernels_per_iteration(C) * block);
+        count_launches((int64_t)kernels_per_iteration(W, C) * block);
         done_iters += block;
         if (err == cudaSuccess) err = collect(block, 0);
         if (err == cudaSuccess && use_tol) {
@@ -1690,7 +1700,7 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
     while (err == cudaSuccess && !finished && done_iters < K) {
         const int par = done_iters & 1;
         err = cudaGraphLaunch(gx_one[par], cs);
-        count_launches(kernels_per_iteration(C));
+        count_launches(kernels_per_iteration(W, C));
         ++done_iters;
         if (err == cudaSuccess) err = collect(1, block + par);
     }
@@ -1701,7 +1711,7 @@ dect_status iterate(const dect_plan *P, const AdmConst &C, Work W, char *base, f
         if (C.nonneg) launch_fwd<NB, 2>(P, W, W.fwd, W.f[1 - par], W.r, C, cs);
         k_unpack<NB><<<(unsigned)((tn + 255) / 256), 256, 0, cs>>>(W.f[1 - par], x, N, D.slot, D.active, 0,
                                                                    W.beta);
-        count_launches(C.nonneg ? 3 : 2);
+        count_launches(2 + (C.nonneg ? fwd_kernels(W, W.fwd, 2) : 0));
         launch_residual_check<NB>(P, W, W.f[1 - par], C, cs);
         err = cudaGetLastError();
     }
@@ -1840,7 +1850,7 @@ dect_status run_chunk(const dect_plan *P, const float *m, float *x, int nimg,
         launch_fwd<NB, 0>(P, W, W.fwd, W.f[0], W.r, C, s);
     else
         k_r_zero<NB><<<(unsigned)((P->M * NB + 255) / 256), 256, 0, s>>>(W.r, m, W.beta, C, D);
-    count_launches(1);
+    count_launches(prm->warm_start ? fwd_kernels(W, W.fwd, 0) : 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
     W.bwd = 1;
     if ((e = tune_bwd<NB>(P, W, C, s)) != cudaSuccess) return fail(e);
