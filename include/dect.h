@@ -502,7 +502,7 @@ dect_status dect_plan_set_tuning(dect_plan *plan, int images, int choice);
 /*
  * Autotuner record of the forward projector A G inside dect_adm_tv, as
  * dect_plan_get_tuning gives it for A^T: the variant chosen for batch width
- * `images` and the measured median time of each (microseconds; -1 = not
+ * `images` and the measured time of each (microseconds; -1 = not
  * timed).  Variants 0-2 run one 1024-thread block per SM and a warp per ray:
  *   0 each lane gathers 4 channels of an entry (one 16-byte load); the row's
  *     table entries are loaded by the warp together and handed to the lanes
@@ -511,11 +511,13 @@ dect_status dect_plan_set_tuning(dect_plan *plan, int images, int choice);
  *     lanes receive each entry's (index, length), four entries per lane in
  *     flight; 16, 32 or 64 channels only (otherwise 0 is used),
  *   2 as 1 with two entries per lane in flight,
- *   3 the plan's line table, a lane per ray and four channels; up to 16
+ *   3 the plan's line table, a lane per ray and four channels; up to 8
  *     channels, where the geometry has the table (otherwise 2, or 0 below 16
  *     channels).
- * Timed on the set-up projection r = A f - beta m of the first ADM call
- * with that width.  Host memory: us has DECT_FWD_VARIANTS elements.
+ * Below 16 channels the choice is a rule (3 where the plan has the table,
+ * otherwise 0) and only that variant is timed; from 16 on the fastest of 0-2 is
+ * kept.  Timed on A G of the first ADM call with that width, before its first
+ * iteration.  Host memory: us has DECT_FWD_VARIANTS elements.
  */
 #define DECT_FWD_VARIANTS 4
 dect_status dect_plan_get_fwd_tuning(const dect_plan *plan, int images, int *choice,

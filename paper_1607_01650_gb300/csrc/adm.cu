@@ -25,8 +25,8 @@
 //   k_fwd    q = A G  (ray-major table)                  ; |grad G|^2, |q|^2,
 //            then the last block forms Phi^k, the stopping test and
 //            alpha^k in FP64.
-// Up to 16 channels k_line_fwd may take the place of k_fwd: A G from the line
-// table (lines.cuh), gathering from G and from a transposed copy that k_bwd
+// Up to 8 channels k_line_fwd takes the place of k_fwd where the plan has a line
+// table: A G from it (lines.cuh), gathering from G and from a transposed copy that k_bwd
 // writes beside it.
 //
 // Optional joint TV over the stacked image (both energies of a slice, channels
@@ -64,11 +64,17 @@ constexpr int kGrid = kSMs * 8;  // fixed grid of every reducing kernel
 constexpr int kFwdBlock = 1024;
 constexpr int kFwdGrid = kSMs;
 
+// Widest batch whose A G takes the line table.  At 16 channels the CSR kernels are
+// as fast inside the iteration (512^2 / 60 views: 172 us both; 1024^2 / 360: 3.30
+// against 3.61 ms; 256^2 / 60: 59 against 63) and k_bwd writes one copy of G less; at
+// 8 the line table is ahead (105 against 118 us, 1.77 against 2.14 ms, 42 against 45).
+constexpr int kLineMaxChannels = 8;
+
 // block partials held per kernel: the grid of k_line_fwd goes beyond kGrid
 template <int NB>
 __host__ __device__ constexpr int part_blocks()
 {
-    return NB <= kLineMaxImages ? kSMs * 16 : kGrid;
+    return NB <= kLineMaxChannels ? kSMs * 16 : kGrid;
 }
 
 // reduction slots; (TV, RR) and (DD, QQ) are reduced together
@@ -103,6 +109,7 @@ struct AdmConst {
     double mu_d, rho_d;  // FP64 for the step and objective
     double tol;
     int rule;
+    int dry;             // a timed A G: leave the step and the stop test alone
 };
 
 template <int NB>
@@ -717,7 +724,7 @@ __global__ void __launch_bounds__(BLK) k_bwd(const int64_t *__restrict__ colptr,
                     nrm[0].v[c] = fmaf(out.v[c], out.v[c], nrm[0].v[c]);
                 }
                 st_keep<VW>(G + o, out, pol);
-                if (NB <= kLineMaxImages && GT) st_v<VW>(GT + ((int64_t)j * C.n + i) * NB + vl * VW, out);
+                if (NB <= kLineMaxChannels && GT) st_v<VW>(GT + ((int64_t)j * C.n + i) * NB + vl * VW, out);
             }
         }
     }
@@ -728,6 +735,7 @@ __global__ void __launch_bounds__(BLK) k_bwd(const int64_t *__restrict__ colptr,
 template <int NB>
 __device__ void adm_finish(const AdmConst &C, const AdmDev &D)
 {
+    if (C.dry) return;
     const int k = *D.k;
     // joint TV: thread 2s decides for the slice (channels 2s, 2s + 1) from
     // the sums of both channels' norms; the odd threads stay idle
@@ -889,7 +897,7 @@ __global__ void __launch_bounds__(BLK) k_fwd(const int64_t *__restrict__ rowptr,
 }
 
 // ---------------------------------------------------------------------------
-// A on the line table (NB <= 16 channels).
+// A on the line table (NB <= 8 channels).
 // ---------------------------------------------------------------------------
 
 // Sums of K quantities of the thread's channel (threadIdx.x % NB) over the
@@ -1105,7 +1113,7 @@ struct Kern {
 // A variants: 0-2 the CSR table, one 1024-thread block per SM, a warp per ray:
 // 0 lanes gather 4 images of an entry; 1 lanes gather 8 images (row_dot_w),
 // four rounds of gathers in flight; 2 as 1 with two rounds (below 16 images
-// 1 and 2 fall back to 0).  3 the line table (NB <= 16; otherwise 2).
+// 1 and 2 fall back to 0).  3 the line table (NB <= 8; otherwise 2).
 constexpr int kFwdLines = 3;
 
 struct Work {
@@ -1130,7 +1138,7 @@ void launch_fwd(const dect_plan *P, const Work &W, int variant, const float *src
 {
     constexpr int GF = Kern<NB>::GF;
     const AdmDev &D = W.D;
-    if constexpr (NB <= kLineMaxImages) {
+    if constexpr (NB <= kLineMaxChannels) {
         if (variant == kFwdLines && W.GT) {
             const LineTable &T = P->lines;
             if (MODE != 1)  // (k_bwd writes G's transpose)
@@ -1287,22 +1295,25 @@ cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     return cudaSuccess;
 }
 
-// Time every A variant on the set-up projection r = A f - beta m and keep the
-// fastest in the plan.  The caller runs the set-up projection again afterwards with
-// the chosen variant (the variants sum in different orders).
+// The A variant of this width.  Below 16 channels a rule: the line table where the
+// plan has it, so that the sums, and with them the images, do not hang on a
+// timing (it is ahead at every size tried but one, 512^2 / 31 views at 8
+// channels, 76 against 71 us).  From 16 on the CSR variants are timed, as the iteration
+// runs them: A G with its norms, without the step that adm_finish forms (on the
+// set-up projection, which reads the planar measurements as well, 16 channels at
+// 1024^2 / 360 views took 4.2 ms where the iteration takes 3.3 and 4.1, and the
+// slower was kept).  G = 0 here, and q = A G is 0 before the first iteration, so
+// timing changes no result.
 template <int NB>
-cudaError_t tune_fwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_t s)
+cudaError_t tune_fwd(const dect_plan *P, Work &W, AdmConst C, cudaStream_t s)
 {
     const int idx = nb_index<NB>();
+    const int rule = W.GT ? kFwdLines : 0;
     if (P->fwd_choice[idx] < 0) {
-        // of 0-2 only 0 below 16 images
+        C.dry = 1;
         const cudaError_t e = tune_variants(
-            s, P->fwd_us[idx], P->fwd_choice[idx],
-            [&](int v) { return v == kFwdLines ? W.GT != nullptr : v == 0 || NB >= 16; },
-            [&](int v) {
-                launch_fwd<NB, 0>(P, W, v, W.f[0], W.r, C, s);
-                count_launches(fwd_kernels(W, v, 0) - 1);
-            });
+            s, P->fwd_us[idx], P->fwd_choice[idx], [&](int v) { return NB < 16 ? v == rule : v != kFwdLines; },
+            [&](int v) { launch_fwd<NB, 1>(P, W, v, W.G, W.q, C, s); });
         if (e != cudaSuccess) return e;
     }
     W.fwd = P->fwd_choice[idx];
@@ -1443,7 +1454,7 @@ cudaError_t alloc_work(const dect_plan *P, Work &W, char **base_out, const float
         W.p = (float *)take(2 * nf * 4);
         W.r = (float *)take(nr * 4);
         W.q = (float *)take(nr * 4);
-        W.GT = NB <= kLineMaxImages && P->lines.ok ? (float *)take(nf * 4) : nullptr;
+        W.GT = NB <= kLineMaxChannels && P->lines.ok ? (float *)take(nf * 4) : nullptr;
         W.beta = (float *)take(64 * 4);
         W.dbl = (double *)take(ndbl * 8);
         W.ints = (int *)take(nint * 4);
@@ -1772,6 +1783,7 @@ AdmConst adm_const(const dect_plan *P, const dect_adm_params *prm)
     C.rho_d = prm->rho;
     C.tol = prm->rel_obj_tol;
     C.rule = prm->step_rule;
+    C.dry = 0;
     return C;
 }
 
