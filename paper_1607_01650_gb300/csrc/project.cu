@@ -139,7 +139,10 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
         }
         return ok;
     };
-    float zero = 0.f;  // stays 0 while every sum is finite
+    // Whether every sum is finite.  Narrow widths add 0 times the sum, which stays 0 (a
+    // comparison each cost the cone pair 3 %), wide ones, short of registers, compare.
+    float zero = 0.f;
+    bool fine = true;
     for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
         int64_t row, b, e;
         const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
@@ -149,10 +152,13 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
         else
             acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, SITE);
 #pragma unroll
-        for (int c = 0; c < VW; ++c) zero = fmaf(acc.v[c], 0.f, zero);
+        for (int c = 0; c < VW; ++c) {
+            if constexpr (NB > 16) fine = fine && isfinite(acc.v[c]);
+            else zero = fmaf(acc.v[c], 0.f, zero);
+        }
         if (ok && grp == 0) st_v<VW>(dst + row * NB + vl * VW, acc);
     }
-    if (__syncthreads_and(zero == 0.f)) return;
+    if (__syncthreads_and(fine && zero == 0.f)) return;
     const GatherIL<NB> gather{src, src_rows, SITE};
     for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
         int64_t row, b, e;
