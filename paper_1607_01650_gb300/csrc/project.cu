@@ -21,9 +21,26 @@ constexpr int kOpBlock = 1024;  // one block per SM
 // entries meet the same lines (A^T of two images at 512^2 / 60 views: 117 -> 65
 // us against a warp per row; 4 lanes 64 us, but 20 % slower on small images;
 // cone-beam 256^2 x 64, 60 views of 64 x 368, one volume: A 1275 -> 971 us, A^T
-// 1821 -> 974; 16 volumes 3485 -> 3382 and 3864 -> 2759).
+// 1821 -> 974; 16 volumes 3485 -> 3382 and 3864 -> 2759).  A fan-beam ray's pixels lie
+// apart from its neighbours', and a warp per ray stays ahead (16 images, 512^2 / 60:
+// 214 us against 262).
 template <int NB>
 constexpr int kLanes = NB <= 16 ? 8 : 32;
+
+// Whether a row takes a whole warp.  Eight lanes take its entries four times as
+// long one after the other, so on few rows a warp each is ahead: A^T up to two turns
+// of the grid, three where a row has 256 entries or more (8 images of 96^2, 60 views:
+// 20 us against 23; 112^2, 60 views: 22 and 23; 112^2, 180 views: 32 and 35; 128^2, 60
+// views: 25 and 23), with 8 images on such rows 16 (256^2, 180 views: 87 and 96;
+// 384^2: 175 and 177); cone-beam A up to five (8 images of 128^2 x 4, 22080 rays: 34
+// and 38; 64^2 x 16, 44160 rays: 37 and 34).
+template <int NB>
+bool warp_rows(bool tiled, int nz, int64_t rows, int64_t nnz)
+{
+    if (!tiled && nz == 0) return true;  // fan-beam A
+    const int turns = !tiled ? 5 : nnz < 256 * rows ? 2 : NB == 8 ? 16 : 3;
+    return rows <= (int64_t)turns * kSMs * (kOpBlock / 32);
+}
 constexpr int kTileW = 8;  // A^T: tiles of 8 columns, so a tile's sinogram lines stay in one L1
 
 // Packing and unpacking, bound by memory.  Up to 4 images a thread takes a row of
@@ -97,21 +114,21 @@ __global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict_
     }
 }
 
-// dst[row][NB] = sum over the row's entries of len * src[index][NB], kLanes
+// dst[row][NB] = sum over the row's entries of len * src[index][NB], G
 // lanes per row.  TILED (pixel-major table of an n x n image): the block's
 // consecutive rows walk pixel tiles of 8 columns, so that pixels sharing rays
 // share an L1; otherwise rows are taken in order (adjacent rays of a view share
-// pixels).  Lanes gather 8 images of an entry above 16 images (row_dot_w), 4
-// below (row_dot_g).
+// pixels).  With a warp per row lanes gather 8 images of an entry from 16 images on
+// (row_dot_w), otherwise 4 (row_dot_g).
 //   row_dot pads a row with entries of weight 0 at index 0, whose product with a
 // value there that is not finite is not 0: a block with a sum that is not finite
 // goes over its rows once more, without padding.
-template <int NB, bool TILED>
+template <int NB, int G, bool TILED>
 __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict__ ptr, const Entry *__restrict__ ent,
                                                       int64_t rows, int n, int nz, const float *__restrict__ src,
                                                       int64_t src_rows, float *__restrict__ dst)
 {
-    constexpr int G = kLanes<NB>, VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
+    constexpr int VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
     constexpr int TW = kTileW, TH = kOpBlock / G > 64 ? kOpBlock / G / TW : 8;
     constexpr unsigned SITE = TILED ? CHK_GATHER_AT : CHK_GATHER_A;
     const int lr = threadIdx.x % G, grp = lr / LPE, vl = lr % LPE;
@@ -147,7 +164,7 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
         int64_t row, b, e;
         const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
         Vec<VW> acc;
-        if constexpr (NB > 16)
+        if constexpr (NB >= 16 && G == 32)
             acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, SITE);
         else
             acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, SITE);
@@ -187,16 +204,19 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
 
 template <int NB>
 cudaError_t pass(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t rows_out, int n, int nz, bool tiled,
-                 const float *src, float *dst, int nimg, float *buf, cudaStream_t s)
+                 int64_t nnz, const float *src, float *dst, int nimg, float *buf, cudaStream_t s)
 {
     float *in_il = buf, *out_il = buf + rows_in * NB;
     constexpr int TR = kTileRows<NB>;
     const unsigned bi = (unsigned)((rows_in + TR - 1) / TR), bo = (unsigned)((rows_out + TR - 1) / TR);
     k_to_il<NB><<<bi, kPackBlock, 0, s>>>(src, in_il, rows_in, nimg);
-    if (tiled)
-        k_rows_il<NB, true><<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, nz, in_il, rows_in, out_il);
+    auto rows = [&](auto kernel) {
+        kernel<<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, std::max(nz, 1), in_il, rows_in, out_il);
+    };
+    if (warp_rows<NB>(tiled, nz, rows_out, nnz))
+        tiled ? rows(k_rows_il<NB, 32, true>) : rows(k_rows_il<NB, 32, false>);
     else
-        k_rows_il<NB, false><<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, nz, in_il, rows_in, out_il);
+        tiled ? rows(k_rows_il<NB, kLanes<NB>, true>) : rows(k_rows_il<NB, kLanes<NB>, false>);
     k_from_il<NB><<<bo, kPackBlock, 0, s>>>(out_il, dst, rows_out, nimg);
     count_launches(3);
     return cudaGetLastError();
@@ -205,7 +225,7 @@ cudaError_t pass(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t 
 // Passes of up to 64 images over the table (ptr, ent) mapping src rows
 // (rows_in per image) to dst rows (rows_out per image).
 cudaError_t run_batched(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t rows_out, int n, int nz,
-                        bool tiled, const float *src, float *dst, int batch, cudaStream_t s)
+                        bool tiled, int64_t nnz, const float *src, float *dst, int batch, cudaStream_t s)
 {
     int width0 = 2;  // widest pass: the next power of two >= min(batch, 64), at least 2
     while (width0 < std::min(batch, kMaxBatchImages)) width0 *= 2;
@@ -216,12 +236,12 @@ cudaError_t run_batched(const int64_t *ptr, const Entry *ent, int64_t rows_in, i
         const int k = std::min(kMaxBatchImages, batch - done);
         const float *sp = src + (int64_t)done * rows_in;
         float *dp = dst + (int64_t)done * rows_out;
-        if (k <= 2) e = pass<2>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
-        else if (k <= 4) e = pass<4>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
-        else if (k <= 8) e = pass<8>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
-        else if (k <= 16) e = pass<16>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
-        else if (k <= 32) e = pass<32>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
-        else e = pass<64>(ptr, ent, rows_in, rows_out, n, nz, tiled, sp, dp, k, buf, s);
+        if (k <= 2) e = pass<2>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
+        else if (k <= 4) e = pass<4>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
+        else if (k <= 8) e = pass<8>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
+        else if (k <= 16) e = pass<16>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
+        else if (k <= 32) e = pass<32>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
+        else e = pass<64>(ptr, ent, rows_in, rows_out, n, nz, tiled, nnz, sp, dp, k, buf, s);
         done += k;
     }
     cudaError_t f = cudaFreeAsync(buf, s);
@@ -312,11 +332,16 @@ cudaError_t run_lines(const LineTable &T, const float *x, float *y, int batch, c
     return e != cudaSuccess ? e : f;
 }
 
-// images of a batch that A takes through the line table: the last pass, where it is narrow enough
+// Images of a batch that A takes through the line table: the last pass, where it is
+// narrow enough.  Above four images a small matrix does not fill the chip with the
+// table's blocks, and a warp per ray is ahead up to about 4 million elements: 16 images of
+// 64^2 / 60 views 21 us against 25, 160^2 / 60 (2.8 million) 36 against 44, 192^2 / 60
+// (4.0) 48 against 46, 256^2 / 30 (3.6) 46 both, 384^2 / 30 (8.0) 83 against 64; 8 images
+// of 160^2 / 60 26 against 29, 192^2 / 60 32 against 31.
 int line_tail(const dect_plan *p, int batch)
 {
     const int rest = batch % kMaxBatchImages;
-    return p->lines.ok && rest <= kLineMaxImages ? rest : 0;
+    return p->lines.ok && rest <= kLineMaxImages && (rest <= 4 || p->nnz >= (int64_t)1 << 22) ? rest : 0;
 }
 
 }  // namespace
@@ -325,14 +350,14 @@ cudaError_t launch_project_planar(const dect_plan *p, const float *x, float *y, 
 {
     const int tail = line_tail(p, batch), head = batch - tail;
     cudaError_t e = cudaSuccess;
-    if (head > 0) e = run_batched(p->rowptr, p->ent, p->N, p->M, p->n, std::max(p->nz, 1), false, x, y, head, s);
+    if (head > 0) e = run_batched(p->rowptr, p->ent, p->N, p->M, p->n, p->nz, false, p->nnz, x, y, head, s);
     if (e == cudaSuccess && tail > 0) e = run_lines(p->lines, x + head * p->N, y + head * p->M, tail, s);
     return e;
 }
 
 cudaError_t launch_backproject_planar(const dect_plan *p, const float *y, float *x, int batch, cudaStream_t s)
 {
-    return run_batched(p->colptr, p->tent, p->M, p->N, p->n, std::max(p->nz, 1), true, y, x, batch, s);
+    return run_batched(p->colptr, p->tent, p->M, p->N, p->n, p->nz, true, p->nnz, y, x, batch, s);
 }
 
 }  // namespace dect
