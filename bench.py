@@ -65,7 +65,7 @@ def parse():
     ap.add_argument("--fwd-variant", type=int, default=-1,
                     help="fix the A variant (0-3, see dect_plan_get_fwd_tuning) instead of autotuning")
     ap.add_argument("--tv-variant", type=int, default=-1,
-                    help="fix the TV-step variant (0-1, see dect_plan_get_tv_tuning) instead of autotuning")
+                    help="fix the TV-step variant (0-2, see dect_plan_get_tv_tuning) instead of autotuning")
     ap.add_argument("--no-stress-cnn", action="store_true",
                     help="stress workload: skip the tile-wise CNN warm start measured after the timed steps")
     ap.add_argument("--batched-otf", action="store_true",
@@ -124,7 +124,7 @@ def measured_peaks():
     return FALLBACK_HBM_GBS, "fallback"
 
 
-ADM_SOURCES = ("adm.cu", "dect_internal.cuh", "kernels.cuh")  # where k_tv, k_bwd*, k_fwd live
+ADM_SOURCES = ("adm.cu", "dect_internal.cuh", "kernels.cuh", "lines.cuh")  # where k_tv, k_bwd*, k_fwd, k_line_fwd live
 
 
 def kernel_source_hash():
@@ -136,6 +136,23 @@ def kernel_source_hash():
             h.update(name.encode())
             h.update(f.read())
     return h.hexdigest()[:16]
+
+
+def fwd_kernel_name(choice, width):
+    """Name of the A kernel of a recorded variant (dect_plan_get_fwd_tuning) at `width` channels."""
+    if choice == 3:
+        return "k_line_fwd" if width <= 8 else "k_fwd<w8,r2>"
+    return {1: "k_fwd<w8,r4>", 2: "k_fwd<w8,r2>"}.get(choice if width >= 16 else 0, "k_fwd")
+
+
+def gathered_by_a(kernel, bytes_per_launch, n, n_pixels, n_rays, nnz):
+    """(mean channels, bytes gathered from the image) of a launch of A whose algorithmic bytes dect_adm_profile
+    gives: the table, and 4 bytes per channel of every pixel read and ray written.  k_fwd gathers a pixel per
+    element of the matrix, k_line_fwd two per ray and line."""
+    lines = kernel == "k_line_fwd"
+    table = 4.0 * n_rays * n if lines else 8.0 * nnz + 8.0 * (n_rays + 1)
+    channels = (bytes_per_launch - table) / (4.0 * (n_pixels + n_rays))
+    return channels, 4.0 * channels * (2.0 * n_rays * n if lines else nnz)
 
 
 def committed_traffic(kernel, workload):
@@ -889,14 +906,8 @@ def main():
     bwd_n = sum(p.bwd_launches for p in state["prof"])
     p0 = state["prof"][-1]
     width = min(64, 1 << (2 * S - 1).bit_length())
-    choice, _ = plan.tuning(width)
-    names = ["k_bwd<tile4>", "k_bwd<tile8>", "k_bwd<tile16>", "k_bwd_win", "k_bwd<1k,8x8>", "k_bwd<1k,16x8>",
-             "k_bwd<1k,8x8,w8>", "k_bwd<1k,8x8,w8,2px>"]
-    bwd_name = names[choice] if 0 <= choice < len(names) else "k_bwd"
-    fchoice, _ = plan.fwd_tuning(width)
-    fnames = ["k_fwd", "k_fwd<w8,r4>", "k_fwd<w8,r2>"]
-    fwd_name = fnames[fchoice] if 0 <= fchoice < len(fnames) else "k_fwd"
-    # the dominant kernel: A (k_fwd), the largest share of the kernel time in
+    fwd_name = fwd_kernel_name(plan.fwd_tuning(width)[0], width)
+    # the dominant kernel: A (k_fwd or k_line_fwd), the largest share of the kernel time in
     # the ncu launch list of this workload (profiles/); with several chunks
     # in flight the event windows of A^T include the other chunk's kernels
     # and would overstate its time
@@ -915,11 +926,8 @@ def main():
 
     clocks = clk.summary()
     # the bound that applies to the table kernels: loaded data returned from
-    # L1 to registers, 128 B per cycle per SM; gathered bytes = 4 NB per entry
-    bytes_fixed = 8.0 * plan.nnz + 8.0 * ((plan.n_rays if kname.startswith("k_fwd") else plan.n_pixels) + 1)
-    per_chan = 4.0 * (plan.n_pixels + plan.n_rays) if kname.startswith("k_fwd") else 4.0 * (plan.n_rays + 3 * plan.n_pixels)
-    nb_mean = (bytes_ - bytes_fixed) / per_chan
-    gathered = 4.0 * nb_mean * plan.nnz
+    # L1 to registers, 128 B per cycle per SM
+    nb_mean, gathered = gathered_by_a(kname, bytes_, geom.n, plan.n_pixels, plan.n_rays, plan.nnz)
     sm_mhz = clocks.get("sm_mhz") or 2070.0
     l1_peak = 128.0 * 152 * sm_mhz * 1e6 / 1e9
     roofline_l1 = {"bound": "l1_writeback", "kernel": kname,
