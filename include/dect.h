@@ -149,9 +149,13 @@ dect_status dect_plan_copy_table(const dect_plan *plan, int64_t *rowptr, int32_t
  * y = A x, Eq. (1), for `batch` images: x [batch][n][n] -> y [batch][n_views][n_bins].
  * The batch runs in passes of up to 64 images: each pass copies its images
  * into a pixel-major interleaved scratch ([pixel][64]), streams the ray-major
- * table once, and copies the sums out.  FP32 multiply-add in a fixed order;
- * deterministic.  The scratch (about 4 (N + M) min(batch, 64) bytes) is
- * taken from the stream-ordered allocator and returned before the call ends.
+ * table once, and copies the sums out.  A last pass of up to 16 images streams
+ * the plan's line table instead, where the plan has it (rays that end outside the
+ * image, 4 <= n <= 4096, memory to spare; above four images from 2^22 elements
+ * on): the same lengths, rounded to FP32 on their own, pieces below 1e-10 of a line's
+ * length left out.  FP32 multiply-add in a fixed order; deterministic.  The
+ * scratch (about 4 (N + M) min(batch, 64) bytes, 8 N min(batch, 16) on the line
+ * table) is taken from the stream-ordered allocator and returned before the call ends.
  * Errors: DECT_ERR_INVALID_ARG (NULL plan/pointer, batch < 0), DECT_ERR_OOM,
  * DECT_ERR_CUDA.  batch = 0 is a no-op.
  */
@@ -163,7 +167,7 @@ dect_status dect_project(const dect_plan *plan, const float *x, float *y, int ba
  * `batch` sinograms: y [batch][n_views][n_bins] -> x [batch][n][n].
  * Gather form over the pixel-major table (rays increasing inside a pixel),
  * in passes of up to 64 sinograms interleaved as for dect_project, pixels
- * taken in 8 x 8 tiles; every pixel sums its rays in a fixed order; no
+ * taken in tiles of 8 columns; every pixel sums its rays in a fixed order; no
  * atomics, bitwise reproducible.  Scratch and errors as dect_project.
  */
 dect_status dect_backproject(const dect_plan *plan, const float *y, float *x, int batch,
@@ -478,11 +482,13 @@ dect_status dect_adm_tv_ex(const dect_plan *plan, const float *m, float *x, int 
  * c channels uses the next of these widths >= min(c, 64)), and the measured
  * time of each variant in microseconds (the median of three launches, or the
  * smaller of two where both are behind the fastest so far; -1 = not available):
- *   0-2 L1-cached gather with 4x4 / 8x8 / 16x16 pixel tiles per 256-thread block,
+ *   0-2 L1-cached gather with 4x4 (4x8 up to 8 channels) / 8x8 / 16x16 pixel tiles
+ *       per 256-thread block,
  *   3   at 16 channels eight lanes per pixel, one 1024-thread block per SM over
  *       8x32 tiles; otherwise none (falls back to 1),
  *   4-5 L1-cached gather, one 1024-thread block per SM, tiles of two / four
- *       block steps (8x8 / 16x8 pixels at 32 and 64 channels, 8x16 / 16x16 below),
+ *       block steps (8x8 / 16x8 pixels at 32 and 64 channels, 8x16 / 16x16 at 16,
+ *       8x32 / 16x32 up to 8),
  *   6-7 (16, 32 or 64 channels; otherwise 4 is used) each lane gathers 8
  *       channels of an entry (two 16-byte loads), so fewer lanes receive
  *       each entry's (index, length): 6 with the lanes and tiles of 4, 7 with
@@ -531,7 +537,7 @@ dect_status dect_plan_set_fwd_tuning(dect_plan *plan, int images, int choice);
  * Autotuner record of the TV step inside dect_adm_tv (the f and r step, the
  * multiplier step of Eq. (7), the z-shrink of Eq. (8) and p, with the TV
  * norm and |r|^2), as dect_plan_get_tuning gives it for A^T: the variant
- * chosen for batch width `images` and the measured median time of each
+ * chosen for batch width `images` and the measured time of each
  * (microseconds; -1 = not timed).
  *   0 blocks claim tiles of 16 rows from a counter and walk down their
  *     columns; the updated row is exchanged through shared memory, one

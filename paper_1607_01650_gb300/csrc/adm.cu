@@ -1127,7 +1127,7 @@ struct Work {
     float *GT;        // transposed copy of G, or of an image being projected (null: no line table at this width)
     int bwd;          // A^T variant in use
     int fwd;          // A variant in use
-    int tv;           // TV-step variant in use (0 k_tv, 1 k_tv_tma)
+    int tv;           // TV-step variant in use (0 k_tv, 1 k_tv_tma, 2 k_tv_px)
     int tv_grid;      // blocks of k_tv_tma
 };
 

@@ -61,7 +61,7 @@ struct PlsConst {
 // Sums of K values over the blocks of vector v = blockIdx.y: FP32 inside a
 // warp, FP64 across warps and blocks, always in the same order.  The vector's
 // last block (a ticket per vector) returns true, with the totals in out[] of
-// thread 0.  A vector's partials (at most a few hundred) are summed by one warp
+// thread 0.  A vector's partials (at most 1216, cg_blocks) are summed by one warp
 // per value, lanes in fixed strides, then a fixed butterfly: summing them one
 // after the other in a single thread cost 40 of the 45 us of each launch on
 // one 512^2 slice.
