@@ -520,10 +520,10 @@ dect_status dect_plan_set_tuning(dect_plan *plan, int images, int choice);
  *   3 the plan's line table, a lane per ray and four channels; up to 8
  *     channels, where the geometry has the table (otherwise 2, or 0 below 16
  *     channels).
- * Below 16 channels the choice is a rule (3 where the plan has the table,
- * otherwise 0) and only that variant is timed; from 16 on the fastest of 0-2 is
- * kept.  Timed on A G of the first ADM call with that width, before its first
- * iteration.  Host memory: us has DECT_FWD_VARIANTS elements.
+ * The choice is a rule up to 32 channels (up to 8 variant 3 where the plan has the
+ * table, otherwise 0), and only that variant is timed; at 64 the faster of 1 and 2,
+ * which sum alike: the images do not depend on it.  Timed on A G of the first ADM
+ * call with that width, before its first iteration.  Host memory: us has DECT_FWD_VARIANTS elements.
  */
 #define DECT_FWD_VARIANTS 4
 dect_status dect_plan_get_fwd_tuning(const dect_plan *plan, int images, int *choice,

@@ -64,10 +64,10 @@ constexpr int kGrid = kSMs * 8;  // fixed grid of every reducing kernel
 constexpr int kFwdBlock = 1024;
 constexpr int kFwdGrid = kSMs;
 
-// Widest batch whose A G takes the line table.  At 16 channels the CSR kernels are
-// as fast inside the iteration (512^2 / 60 views: 172 us both; 1024^2 / 360: 3.30
-// against 3.61 ms; 256^2 / 60: 59 against 63) and k_bwd writes one copy of G less; at
-// 8 the line table is ahead (105 against 118 us, 1.77 against 2.14 ms, 42 against 45).
+// Widest batch whose A G takes the line table.  At 16 channels k_fwd is ahead (512^2
+// / 60 views: 156 us against 172; 1024^2 / 360: 2.88 ms against 3.61; 256^2 / 60: 57 us
+// against 63) and as accurate, and k_bwd writes one copy of G less; at 8 the line table
+// is (105 against 118 us, 1.77 against 2.14 ms, 42 against 45).
 constexpr int kLineMaxChannels = 8;
 
 // block partials held per kernel: the grid of k_line_fwd goes beyond kGrid
@@ -857,7 +857,7 @@ __global__ void __launch_bounds__(BLK) k_fwd(const int64_t *__restrict__ rowptr,
         if constexpr (VWL > 4 && NB >= 16)
             acc = row_dot_w<NB, G_, VWL, R>(ent, b, e, lr, src, pol, C.N, CHK_GATHER_A);
         else
-            acc = row_dot<NB, G_, true>(ent, b, e, src, C.N, lr, CHK_GATHER_A);
+            acc = row_dot<NB, G_, true, false, (G_ <= 8 || NB >= 16)>(ent, b, e, src, C.N, lr, CHK_GATHER_A);
         if (ray < C.M && grp == 0) {
             if (MODE != 1) {
 #pragma unroll
@@ -1295,24 +1295,27 @@ cudaError_t tune_bwd(const dect_plan *P, Work &W, const AdmConst &C, cudaStream_
     return cudaSuccess;
 }
 
-// The A variant of this width.  Below 16 channels a rule: the line table where the
-// plan has it, so that the sums, and with them the images, do not hang on a
-// timing (it is ahead at every size tried but one, 512^2 / 31 views at 8
-// channels, 76 against 71 us).  From 16 on the CSR variants are timed, as the iteration
-// runs them: A G with its norms, without the step that adm_finish forms (on the
-// set-up projection, which reads the planar measurements as well, 16 channels at
-// 1024^2 / 360 views took 4.2 ms where the iteration takes 3.3 and 4.1, and the
-// slower was kept).  G = 0 here, and q = A G is 0 before the first iteration, so
-// timing changes no result.
+// The A variant of this width, by a rule, so that the sums and their accuracy do not
+// hang on a timing: up to 8 channels the line table where the plan has it (ahead at
+// every size tried but one, 512^2 / 31 views at 8 channels, 73 us against 71); at 16
+// and 32 variant 0, whose sums carry their rounding errors (512^2 / 60 views, 1 and 2
+// in brackets: 156 us [214] and 264 [277], images after 60 iterations 1.3e-7 [1.6e-7]
+// and 1.3e-7 [1.8e-7] from 64 bits; without that 170 us, 1.9e-7 and 262, 2.7e-7).  At 64
+// the faster of 1 and 2, which sum alike (444 to 452 us, 2.6e-7; variant 0 450, 1.4e-7).
+// The variant is timed as the iteration runs it: A G with its norms, without the step
+// that adm_finish forms (the set-up projection reads the planar measurements as
+// well: 16 channels at 1024^2 / 360 views took 4.2 ms there and 3.3 in the iteration).
+// G = 0 here, and q = A G is 0 before the first iteration, so timing changes no result.
 template <int NB>
 cudaError_t tune_fwd(const dect_plan *P, Work &W, AdmConst C, cudaStream_t s)
 {
     const int idx = nb_index<NB>();
-    const int rule = W.GT ? kFwdLines : 0;
+    const int rule = NB == 64 ? -1 : W.GT ? kFwdLines : 0;
     if (P->fwd_choice[idx] < 0) {
         C.dry = 1;
         const cudaError_t e = tune_variants(
-            s, P->fwd_us[idx], P->fwd_choice[idx], [&](int v) { return NB < 16 ? v == rule : v != kFwdLines; },
+            s, P->fwd_us[idx], P->fwd_choice[idx],
+            [&](int v) { return rule >= 0 ? v == rule : v == 1 || v == 2; },
             [&](int v) { launch_fwd<NB, 1>(P, W, v, W.G, W.q, C, s); });
         if (e != cudaSuccess) return e;
     }

@@ -270,7 +270,7 @@ __device__ __forceinline__ bool reduce_images(Vec<Batch<NB>::VW> (&v)[K], double
 // reproducible.  After the call, the lanes with group == 0 hold the row's sums.
 // Every lane of the warp must call it (rows past the end pass b = e).
 // ---------------------------------------------------------------------------
-template <int NB, int G, typename Gather, bool SBC = false>
+template <int NB, int G, typename Gather, bool SBC = false, bool PART = (G <= 8)>
 __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_g(const Entry *__restrict__ ent, int64_t b,
                                                         int64_t e, int lr, Gather gather)
 {
@@ -280,11 +280,11 @@ __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot_g(const Entry *__restrict_
     const int grp = lr / LPE, vl = lr % LPE;
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned gbase = lane & ~(unsigned)(G - 1);  // first lane of this row group
-    // a lane of a short split sums many entries: the step's are summed by
+    // PART: a lane of a short split sums many entries: the step's are summed by
     // themselves first and their sums with compensation, so that the error of A
-    // and A^T is no larger than with a warp per row (two entry groups at 16 images
-    // sum half a row each: A^T y 6.8e-8 off without, 2.8e-8 with, 4.4e-8 with a warp per row)
-    constexpr bool PART = G <= 8;
+    // and A^T is no larger than with more entry groups (two of them at 16 images and
+    // eight lanes sum half a row each: A^T y 6.8e-8 off without, 2.8e-8 with, 4.4e-8
+    // with a warp per row; two at 64 images and a warp: ADM images 4.7e-7 and 1.4e-7)
     Vec<VW> acc, lost;
     acc.zero();
     lost.zero();
@@ -472,13 +472,13 @@ struct GatherIL {  // interleaved [index][NB] in global memory, `rows` indices
     }
 };
 // src holds `rows` interleaved rows; site: the check site of its gathers.
-template <int NB, int G, bool IL, bool SBC = false>
+template <int NB, int G, bool IL, bool SBC = false, bool PART = (G <= 8)>
 __device__ __forceinline__ Vec<Batch<NB>::VW> row_dot(const Entry *__restrict__ ent, int64_t b, int64_t e,
                                                       const float *__restrict__ src, int64_t rows, int lr,
                                                       unsigned site)
 {
     static_assert(IL, "only the interleaved layout is gathered");
-    return row_dot_g<NB, G, GatherIL<NB>, SBC>(ent, b, e, lr, GatherIL<NB>{src, rows, site});
+    return row_dot_g<NB, G, GatherIL<NB>, SBC, PART>(ent, b, e, lr, GatherIL<NB>{src, rows, site});
 }
 
 }  // namespace dect
