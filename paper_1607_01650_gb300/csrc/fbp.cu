@@ -104,19 +104,6 @@ __device__ __forceinline__ double odd_tap(double k, double ds)
     return -1.0 / (pi * pi * k * k * ds * ds);
 }
 
-// The views' directions, and for k_fbp_filter_tc the cosine weights [n_bins] and the
-// taps at odd distances 2 j + 1 [n_bins / 2 + 1].
-__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap)
-{
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v < g.n_bins) cwd[v] = cos_weight(g, v);
-    if (v <= g.n_bins / 2) tap[v] = odd_tap(2.0 * v + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
-    if (v >= g.n_views) return;
-    const double th = g.start_rad + (double)v * (g.arc_rad / (double)g.n_views);
-    const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
-    vg[v] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
-}
-
 // ---------------------------------------------------------------------------
 // FP64 filter: one block per (view, image); shared memory q[nb] and the odd
 // taps.  For detectors of more than kTcMaxBins bins.
@@ -159,7 +146,7 @@ __global__ void __launch_bounds__(kFbpBlock) k_fbp_filter(const float *__restric
 // tiles.  B fragments come from a table of T's digits by n - k (Toeplitz), two
 // neighbouring taps per 32-bit word.  T's first digit is zero from d = 13 on
 // and its second from d = 183 on (1 / d^2 below half a unit of it), so tiles
-// farther from the diagonal leave out the products with it.  Up to 44 k MMAs per
+// farther from the diagonal leave out the products with it.  27 k MMAs per
 // block at 736 bins; two blocks' worth per SM at 64 images of 60 views.
 //   The sum of one weight's products is at most the sum of |T digit| over both
 // sides' taps times 128: 0.92 2^24 at 1152 bins, below 2^24 up to 1270.
@@ -173,6 +160,7 @@ struct FilterShape {
     int ld;       // row stride of a digit plane (BF16), 16 bytes off a multiple of 32
     int tn;       // words of one digit of the tap table
     int nw;       // words of a row's bits
+    size_t dig;   // bytes of the digits and taps
     size_t smem;
 };
 __host__ __device__ inline FilterShape filter_shape(int nb)
@@ -184,11 +172,13 @@ __host__ __device__ inline FilterShape filter_shape(int nb)
     f.ld = f.kpad + 8;
     f.tn = 2 * f.kpad + 32;
     f.nw = (nb + 31) / 32;
-    f.smem = (size_t)kDig * kTcRows * f.ld * 2 + (size_t)kDig * f.tn * 4 + (size_t)nb * sizeof(FF) +
-             (size_t)kTcRows * f.nw * 4;
+    const size_t digits = ((size_t)kDig * kTcRows * f.ld * 2 + (size_t)kDig * f.tn * 4 + 15) & ~(size_t)15;
+    const size_t rows = (size_t)kTcRows * nb * sizeof(double);  // of the second sums, over the digits and taps
+    f.dig = digits > rows ? digits : rows;
+    f.smem = f.dig + (size_t)nb * sizeof(FF) + (size_t)kTcRows * f.nw * 4;
     return f;
 }
-constexpr size_t kTcSmemMax = 176 * 1024;  // kTcMaxBins: 169 KB
+constexpr size_t kTcSmemMax = 176 * 1024;  // kTcMaxBins: 171 KB
 
 __device__ __forceinline__ void ldsm_a(unsigned (&r)[4], const void *p)
 {
@@ -216,10 +206,44 @@ __device__ __forceinline__ void digits(long long Q, __nv_bfloat16 (&d)[kDig])
     }
 }
 
+// The views' directions, and for k_fbp_filter_tc the cosine weights [n_bins], the taps
+// at odd distances 2 j + 1 [n_bins / 2 + 1] and the words of T's digits [kDig][tn]: word w
+// holds (T(w - kpad - 16), T(w - kpad - 17)) of the even outputs, T(x) = 1 / (2 j +
+// 1)^2, j = x - 1 for x > 0 and -x otherwise.  (Formed by every block, the digits' FP64
+// divisions were a tenth of the filter.)
+__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap, unsigned *tw)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const FilterShape F = filter_shape(g.n_bins);
+    if (t < g.n_bins) cwd[t] = cos_weight(g, t);
+    if (t <= g.n_bins / 2) tap[t] = odd_tap(2.0 * t + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
+    if (t < F.tn) {
+        __nv_bfloat16 d0[kDig], d1[kDig];
+        const int x = t - F.kpad - 16, j0 = x > 0 ? x - 1 : -x, j1 = x - 1 > 0 ? x - 2 : 1 - x;
+        const double k0 = 2.0 * j0 + 1.0, k1 = 2.0 * j1 + 1.0;
+        digits(__double2ll_rn(0x1p46 / (k0 * k0)), d0);
+        digits(__double2ll_rn(0x1p46 / (k1 * k1)), d1);
+#pragma unroll
+        for (int k = 0; k < kDig; ++k)
+            tw[k * F.tn + t] = (unsigned)__bfloat16_as_ushort(d0[k]) | ((unsigned)__bfloat16_as_ushort(d1[k]) << 16);
+    }
+    if (t >= g.n_views) return;
+    const double th = g.start_rad + (double)t * (g.arc_rad / (double)g.n_views);
+    const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
+    vg[t] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
+}
+
+// Numbers of a call that every thread would divide for.
+struct FilterConst {
+    double ds, h0;  // bin spacing at the isocentre, h(0)
+    FF ipi2, ids;   // 1 / pi^2, 1 / ds
+};
+
 __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__restrict__ m, float *__restrict__ qf,
                                                               const double *__restrict__ cwd,
-                                                              const double *__restrict__ tap, dect_geometry g, int nimg,
-                                                              int width)
+                                                              const double *__restrict__ tap,
+                                                              const uint4 *__restrict__ tw, dect_geometry g,
+                                                              FilterConst K, int nimg, int width)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ float sscale[kTcRows];  // 2^(e - 12) of the row
@@ -228,25 +252,13 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
     const FilterShape F = filter_shape(nb);
     __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16 *>(dyn);  // [digit][row][ld], the inputs of one parity
     unsigned *T = reinterpret_cast<unsigned *>(A + (size_t)kDig * kTcRows * F.ld);  // [digit][tn]
-    FF *cw = reinterpret_cast<FF *>(T + (size_t)kDig * F.tn);
+    FF *cw = reinterpret_cast<FF *>(dyn + F.dig);
     unsigned *todo = reinterpret_cast<unsigned *>(cw + nb);  // [row][nw] a bit per bin left to FP64
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t R0 = (int64_t)blockIdx.x * kTcRows, rows = (int64_t)nv * nimg;
-    const double ds = g.pitch_mm * (g.sod_mm / g.sdd_mm);
     for (int b = threadIdx.x; b < nb; b += kTcThreads) cw[b] = ff_of(cwd[b]);
     for (int b = threadIdx.x; b < kTcRows * F.nw; b += kTcThreads) todo[b] = 0u;
-    // tap table: word w holds (T(w - kpad - 16), T(w - kpad - 17)) of the even outputs,
-    // T(x) = 1 / (2 j + 1)^2, j = x - 1 for x > 0 and -x otherwise
-    for (int w = threadIdx.x; w < F.tn; w += kTcThreads) {
-        __nv_bfloat16 d0[kDig], d1[kDig];
-        const int x = w - F.kpad - 16, j0 = x > 0 ? x - 1 : -x, j1 = x - 1 > 0 ? x - 2 : 1 - x;
-        const double k0 = 2.0 * j0 + 1.0, k1 = 2.0 * j1 + 1.0;
-        digits(__double2ll_rn(0x1p46 / (k0 * k0)), d0);
-        digits(__double2ll_rn(0x1p46 / (k1 * k1)), d1);
-#pragma unroll
-        for (int k = 0; k < kDig; ++k)
-            T[k * F.tn + w] = (unsigned)__bfloat16_as_ushort(d0[k]) | ((unsigned)__bfloat16_as_ushort(d1[k]) << 16);
-    }
+    for (int w = threadIdx.x; w < kDig * F.tn / 4; w += kTcThreads) reinterpret_cast<uint4 *>(T)[w] = tw[w];
     __syncthreads();
     // a warp per row: its scale, later its digits
     const bool on = R0 + warp < rows;
@@ -275,7 +287,6 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
             slim[warp] = bad ? NAN : mx > 0.f ? ldexpf(sqrtf((float)nb), e - 23) : 0.f;
         }
     }
-    const FF ipi2 = ff_of(1.0 / (3.14159265358979323846 * 3.14159265358979323846)), ids = ff_of(1.0 / ds);
     const int gid = lane >> 2, t4 = lane & 3;
     for (int par = 0; par < 2; ++par) {  // outputs of parity par from inputs of the other
         __syncthreads();  // the scales are written; the other parity's digits have been read
@@ -339,11 +350,11 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
                     const float scale = sscale[row];
                     const FF sum = two_sum(s3.h, __fadd_rn(__fadd_rn(s1.l, __fadd_rn(s2.l, s3.l)),
                                                            fmaf(acc[t][5][c], 0x1p-40f, acc[t][4][c] * 0x1p-32f)));
-                    const FF far = ff_mul(FF{sum.h * scale, sum.l * scale}, ipi2);
+                    const FF far = ff_mul(FF{sum.h * scale, sum.l * scale}, K.ipi2);
                     const FF q = ff_mul(FF{m[((int64_t)img * nv + v) * nb + b], 0.f}, cw[b]);
                     const FF d = ff_add(FF{0.25f * q.h, 0.25f * q.l}, FF{-far.h, -far.l});
                     if (fabsf(d.h) >= slim[row]) {
-                        const FF o = ff_mul(d, ids);
+                        const FF o = ff_mul(d, K.ids);
                         qf[((int64_t)v * nb + b) * width + img] = __fadd_rn(o.h, o.l);
                     } else {
                         atomicOr(&todo[row * F.nw + (b >> 5)], 1u << (b & 31));
@@ -351,28 +362,33 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
                 }
         }
     }
-    // what is left to FP64: the row's q over the digits, a warp per output, its lanes over the taps
+    // What is left to FP64: the rows' q in place of the digits, a warp per row; then a warp
+    // per output, its lanes over the taps, 32 bins after 32 to one warp after the other.
+    if (!__syncthreads_or(lane < F.nw && todo[warp * F.nw + lane] != 0u ||
+                          lane + 32 < F.nw && todo[warp * F.nw + lane + 32] != 0u))
+        return;
+    double *q = reinterpret_cast<double *>(dyn);  // [row][nb]
+    {
+        bool any = false;
+        for (int w = lane; w < F.nw; w += 32) any |= todo[warp * F.nw + w] != 0u;
+        if (__any_sync(0xffffffffu, any))
+            for (int b = lane; b < nb; b += 32) q[warp * nb + b] = (double)mine[b] * cwd[b];
+    }
     __syncthreads();
-    double *q = reinterpret_cast<double *>(dyn);
-    const double h0 = 1.0 / (4.0 * ds * ds);
-    for (int row = 0; row < kTcRows; ++row) {
-        unsigned *bits = todo + row * F.nw;
-        if (!__syncthreads_or(threadIdx.x < F.nw && bits[threadIdx.x] != 0u)) continue;
+    for (int w = warp; w < kTcRows * F.nw; w += kTcWarps) {
+        const int row = w / F.nw;
+        const double *qr = q + row * nb;
         const int v = (int)((R0 + row) / nimg), img = (int)((R0 + row) % nimg);
-        const float *src = m + ((int64_t)img * nv + v) * nb;
-        for (int b = threadIdx.x; b < nb; b += kTcThreads) q[b] = (double)src[b] * cwd[b];
-        __syncthreads();
-        for (int w = warp; w < F.nw; w += kTcWarps)
-            for (unsigned left = bits[w]; left != 0u; left &= left - 1u) {
-                const int b = w * 32 + __ffs(left) - 1;
-                double acc = 0.0;
+        for (unsigned left = todo[w]; left != 0u; left &= left - 1u) {
+            const int b = (w - row * F.nw) * 32 + __ffs(left) - 1;
+            double acc = 0.0;
 #pragma unroll 4
-                for (int i = 1 - (b & 1) + 2 * lane; i < nb; i += 64) acc = fma(tap[abs(i - b) >> 1], q[i], acc);
+            for (int i = 1 - (b & 1) + 2 * lane; i < nb; i += 64) acc = fma(tap[abs(i - b) >> 1], qr[i], acc);
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (lane == 0)
-                    qf[((int64_t)v * nb + b) * width + img] = (float)(ds * fma(h0, q[b], acc));
-            }
+            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if (lane == 0)
+                qf[((int64_t)v * nb + b) * width + img] = (float)(K.ds * fma(K.h0, qr[b], acc));
+        }
     }
 }
 
@@ -396,20 +412,27 @@ struct BpShape {
     static constexpr int GV = LPP < 4 ? 4 : LPP, GPL = GV / LPP;  // views of a group, of a lane's geometry
 };
 
+// Numbers of a call, in two words (formed in FP64 by every thread they took 47 us of the
+// case below).
+struct BpConst {
+    int n, nv, nb;
+    FF pixel, sod, half_dth, t0;  // t0: the isocentre's bin coordinate, negated
+};
+
 template <int W>
 __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict__ qf, float *__restrict__ x,
-                                                        const ViewGeo *__restrict__ vg, dect_geometry g, FF t0, int nimg)
+                                                        const ViewGeo *__restrict__ vg, BpConst K, int nimg)
 {
     using S = BpShape<W>;
     constexpr int NV = S::IPL / S::VW;
-    const int n = g.n, nv = g.n_views, nb = g.n_bins;
+    const int n = K.n, nv = K.nv, nb = K.nb;
+    const FF sod = K.sod, half_dth = K.half_dth, t0 = K.t0;
     const int p = threadIdx.x / S::LPP, sub = threadIdx.x % S::LPP;
     const int i = blockIdx.y * S::TH + p / S::TW, j = blockIdx.x * S::TW + p % S::TW;
     const bool in = i < n && j < n;
-    const FF px = ff_of(((double)j + 0.5 - 0.5 * (double)n) * g.pixel_mm);
-    const FF py = ff_of(((double)i + 0.5 - 0.5 * (double)n) * g.pixel_mm);
-    const FF sod = ff_of(g.sod_mm);
-    const FF half_dth = ff_of(0.5 * g.arc_rad / (double)nv);
+    // (half integers below 2^23: exact)
+    const FF px = ff_mul(FF{0.5f * (float)(2 * j + 1 - n), 0.f}, K.pixel);
+    const FF py = ff_mul(FF{0.5f * (float)(2 * i + 1 - n), 0.f}, K.pixel);
     const float tmax = (float)(nb - 1);
     float acc[S::IPL];
 #pragma unroll
@@ -497,11 +520,11 @@ __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict_
 }
 
 template <int W>
-void launch_bp(const float *qf, float *x, const ViewGeo *vg, const dect_geometry &g, FF t0, int nimg, cudaStream_t s)
+void launch_bp(const float *qf, float *x, const ViewGeo *vg, const BpConst &K, int nimg, cudaStream_t s)
 {
     using S = BpShape<W>;
-    const dim3 grid((unsigned)((g.n + S::TW - 1) / S::TW), (unsigned)((g.n + S::TH - 1) / S::TH));
-    k_fbp_bp<W><<<grid, kBpBlock, 0, s>>>(qf, x, vg, g, t0, nimg);
+    const dim3 grid((unsigned)((K.n + S::TW - 1) / S::TW), (unsigned)((K.n + S::TH - 1) / S::TH));
+    k_fbp_bp<W><<<grid, kBpBlock, 0, s>>>(qf, x, vg, K, nimg);
 }
 
 }  // namespace
@@ -535,19 +558,27 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
     const size_t nr = (size_t)g.n_views * g.n_bins, qbytes = (sizeof(float) * nr * width + 255) & ~(size_t)255;
     const int nodd = g.n_bins / 2 + 1;
     char *base = nullptr;
-    DECT_CUDA(cudaMallocAsync((void **)&base,
-                              qbytes + sizeof(ViewGeo) * g.n_views + sizeof(double) * (size_t)(g.n_bins + nodd), s));
+    const FilterShape F = filter_shape(g.n_bins);
+    const size_t vbytes = sizeof(ViewGeo) * (size_t)g.n_views, wbytes = sizeof(unsigned) * (size_t)kDig * F.tn;
+    DECT_CUDA(cudaMallocAsync((void **)&base, qbytes + vbytes + wbytes + sizeof(double) * (size_t)(g.n_bins + nodd), s));
     float *qf = (float *)base;
     ViewGeo *vg = (ViewGeo *)(base + qbytes);
-    double *cwd = (double *)(vg + g.n_views), *tap = cwd + g.n_bins;
-    const FilterShape F = filter_shape(g.n_bins);
+    unsigned *tw = (unsigned *)(base + qbytes + vbytes);  // (16-byte aligned: both sizes are multiples of 32)
+    double *cwd = (double *)(base + qbytes + vbytes + wbytes), *tap = cwd + g.n_bins;
+    FilterConst K;
+    K.ds = g.pitch_mm * (g.sod_mm / g.sdd_mm);
+    K.h0 = 1.0 / (4.0 * K.ds * K.ds);
+    K.ipi2 = ff_of(1.0 / (3.14159265358979323846 * 3.14159265358979323846));
+    K.ids = ff_of(1.0 / K.ds);
     const bool tc = g.n_bins <= kTcMaxBins;
     cudaError_t e = cudaFuncSetAttribute(k_fbp_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fbp_filter_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
-    const FF t0 = ff_of(-0.5 * (double)(g.n_bins - 1) + g.det_offset_mm / g.pitch_mm);
+    const BpConst B{g.n, g.n_views, g.n_bins, ff_of(g.pixel_mm), ff_of(g.sod_mm),
+                    ff_of(0.5 * g.arc_rad / (double)g.n_views),
+                    ff_of(-0.5 * (double)(g.n_bins - 1) + g.det_offset_mm / g.pitch_mm)};
     if (e == cudaSuccess) {
-        k_fbp_tables<<<(std::max(g.n_views, g.n_bins) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap);
+        k_fbp_tables<<<(std::max({g.n_views, g.n_bins, F.tn}) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap, tw);
         count_launches(1);
     }
     for (int done = 0; done < batch && e == cudaSuccess; done += kMaxBatchImages) {
@@ -558,17 +589,17 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
         while (w < k) w *= 2;
         if (tc)
             k_fbp_filter_tc<<<(unsigned)(((int64_t)g.n_views * k + kTcRows - 1) / kTcRows), kTcThreads, F.smem, s>>>(
-                mk, qf, cwd, tap, g, k, w);
+                mk, qf, cwd, tap, (const uint4 *)tw, g, K, k, w);
         else
             k_fbp_filter<<<dim3(g.n_views, k), kFbpBlock, smem, s>>>(mk, qf, g, w);
         switch (w) {
-        case 1: launch_bp<1>(qf, xk, vg, g, t0, k, s); break;
-        case 2: launch_bp<2>(qf, xk, vg, g, t0, k, s); break;
-        case 4: launch_bp<4>(qf, xk, vg, g, t0, k, s); break;
-        case 8: launch_bp<8>(qf, xk, vg, g, t0, k, s); break;
-        case 16: launch_bp<16>(qf, xk, vg, g, t0, k, s); break;
-        case 32: launch_bp<32>(qf, xk, vg, g, t0, k, s); break;
-        default: launch_bp<64>(qf, xk, vg, g, t0, k, s); break;
+        case 1: launch_bp<1>(qf, xk, vg, B, k, s); break;
+        case 2: launch_bp<2>(qf, xk, vg, B, k, s); break;
+        case 4: launch_bp<4>(qf, xk, vg, B, k, s); break;
+        case 8: launch_bp<8>(qf, xk, vg, B, k, s); break;
+        case 16: launch_bp<16>(qf, xk, vg, B, k, s); break;
+        case 32: launch_bp<32>(qf, xk, vg, B, k, s); break;
+        default: launch_bp<64>(qf, xk, vg, B, k, s); break;
         }
         count_launches(2);
         e = cudaGetLastError();
