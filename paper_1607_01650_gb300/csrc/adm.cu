@@ -1794,7 +1794,7 @@ AdmConst adm_const(const dect_plan *P, const dect_adm_params *prm)
 // batch of NB can narrow to, each on an empty workspace (as a narrowing does
 // before the state arrives), so that chunks run side by side later find
 // their choices made and no timing sees another chunk's kernels.  m: a
-// sinogram of the plan (read by the set-up projection only).
+// sinogram of the plan.
 template <int NB>
 cudaError_t pretune(const dect_plan *P, const float *m, const AdmConst &C, cudaStream_t s)
 {

@@ -23,8 +23,8 @@
 //
 // The multi-slice ADM also runs on the plans' stored tables instead
 // (dect_adm_tv_batch_ex with DECT_PROJ_TABLE): eight lanes per ray of the
-// ray-major table for A, eight per pixel of the pixel-major table for A^T
-// (the row kernels of the single-plan ADM at two channels).
+// ray-major table for A, eight per pixel of the pixel-major table for A^T.  (The
+// single-plan ADM takes A from the line table instead, where the plan has it.)
 //
 // Multi-slice ADM.  Each slice (both energies interleaved, [pixel][2])
 // keeps its own state and scalars; one launch per ADM phase covers every
