@@ -145,14 +145,14 @@ def fwd_kernel_name(choice, width):
     return {1: "k_fwd<w8,r4>", 2: "k_fwd<w8,r2>"}.get(choice if width >= 16 else 0, "k_fwd")
 
 
-def gathered_by_a(kernel, bytes_per_launch, n, n_pixels, n_rays, nnz):
-    """(mean channels, bytes gathered from the image) of a launch of A whose algorithmic bytes dect_adm_profile
-    gives: the table, and 4 bytes per channel of every pixel read and ray written.  k_fwd gathers a pixel per
-    element of the matrix, k_line_fwd two per ray and line."""
-    lines = kernel == "k_line_fwd"
-    table = 4.0 * n_rays * n if lines else 8.0 * nnz + 8.0 * (n_rays + 1)
-    channels = (bytes_per_launch - table) / (4.0 * (n_pixels + n_rays))
-    return channels, 4.0 * channels * (2.0 * n_rays * n if lines else nnz)
+def gathered_by_a(kernel, bytes_bwd, n, n_pixels, n_rays, nnz):
+    """(mean channels, bytes gathered from the image) of a launch of A.  The channels follow from the algorithmic
+    bytes of A^T (dect_adm_profile), whose table is the same at every width a batch narrows to: the table, and 4
+    bytes per channel of every ray and two gradients read and pixel written.  k_fwd gathers a pixel per element of
+    the matrix, k_line_fwd two per ray and line; launches of a batch that has narrowed from the one to the other
+    are counted as the kernel's named."""
+    channels = (bytes_bwd - 8.0 * nnz - 8.0 * (n_pixels + 1)) / (4.0 * (n_rays + 3 * n_pixels))
+    return channels, 4.0 * channels * (2.0 * n_rays * n if kernel == "k_line_fwd" else nnz)
 
 
 def committed_traffic(kernel, workload):
@@ -927,7 +927,7 @@ def main():
     clocks = clk.summary()
     # the bound that applies to the table kernels: loaded data returned from
     # L1 to registers, 128 B per cycle per SM
-    nb_mean, gathered = gathered_by_a(kname, bytes_, geom.n, plan.n_pixels, plan.n_rays, plan.nnz)
+    nb_mean, gathered = gathered_by_a(kname, p0.table_bytes_bwd, geom.n, plan.n_pixels, plan.n_rays, plan.nnz)
     sm_mhz = clocks.get("sm_mhz") or 2070.0
     l1_peak = 128.0 * 152 * sm_mhz * 1e6 / 1e9
     roofline_l1 = {"bound": "l1_writeback", "kernel": kname,

@@ -9,11 +9,14 @@ def test_the_kernel_that_runs_is_the_one_named():
     assert bench.fwd_kernel_name(1, 8) == bench.fwd_kernel_name(0, 64) == bench.fwd_kernel_name(-1, 64) == "k_fwd"
 
 
-def test_bytes_gathered_follow_the_table():
-    n, M, nnz, nb = 512, 60 * 736, 28793597, 2
+def test_bytes_gathered_follow_the_width():
+    n, M, nnz = 512, 60 * 736, 28793597
     N = n * n
-    # the library's algorithmic bytes of a launch on either table (adm.cu, add_profile_bytes)
-    csr = 8.0 * nnz + 8.0 * (M + 1) + 4.0 * nb * (N + M)
-    lines = 4.0 * M * n + 4.0 * nb * (N + M)
-    assert bench.gathered_by_a("k_fwd", csr, n, N, M, nnz) == (nb, 4.0 * nb * nnz)
-    assert bench.gathered_by_a("k_line_fwd", lines, n, N, M, nnz) == (nb, 4.0 * nb * 2 * M * n)
+
+    def bwd(nb):  # the library's algorithmic bytes of A^T (adm.cu, add_profile_bytes)
+        return 8.0 * nnz + 8.0 * (N + 1) + 4.0 * nb * (M + 3 * N)
+
+    assert bench.gathered_by_a("k_fwd<w8,r2>", bwd(64), n, N, M, nnz) == (64, 4.0 * 64 * nnz)
+    assert bench.gathered_by_a("k_line_fwd", bwd(2), n, N, M, nnz) == (2, 4.0 * 2 * 2 * M * n)
+    # half of the launches narrowed to 2 channels, where A has another table: 33 on average
+    assert bench.gathered_by_a("k_fwd<w8,r2>", (bwd(64) + bwd(2)) / 2, n, N, M, nnz)[0] == 33
