@@ -82,10 +82,39 @@ __global__ void __launch_bounds__(kPackBlock) k_to_il(const float *__restrict__ 
     }
 }
 
+// The table and the interleaved images that k_rows_il has summed.
+struct RowTable {
+    const int64_t *ptr;
+    const Entry *ent;
+    const float *src;
+    int64_t src_rows;
+    unsigned site;
+};
+
+// v, image c of a row of sums; where it is not finite, the row's sum without the
+// padded entries of row_dot, whose product 0 times a value at index 0 that is not
+// finite is not 0.  (Tested in k_rows_il itself the comparison cost ptxas the order of
+// its gathers: A of 16 volumes of 256^2 x 64 3.16 -> 4.00 ms, A^T of 64 images at
+// 1024^2 / 360 views 10.3 -> 11.9.)
+template <int NB>
+__device__ __forceinline__ float unpadded(float v, const RowTable &T, int64_t row, int c)
+{
+    if (isfinite(v)) return v;
+    float s = 0.f;
+#pragma unroll 1
+    for (int64_t k = T.ptr[row], e = T.ptr[row + 1]; k < e; ++k) {
+        const Entry en = ld_entry(T.ent + k);
+        int at = en.x;
+        if (!DECT_IDX_OK(at, T.src_rows, T.site)) at = 0;
+        s = fmaf(__int_as_float(en.y), T.src[(int64_t)at * NB + c], s);
+    }
+    return s;
+}
+
 // interleaved src [rows][NB] -> planar dst [nimg][rows]
 template <int NB>
-__global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict__ src, float *__restrict__ dst,
-                                                        int64_t rows, int nimg)
+__global__ void __launch_bounds__(kPackBlock, 8) k_from_il(const float *__restrict__ src, float *__restrict__ dst,
+                                                           int64_t rows, int nimg, RowTable T)
 {
     constexpr int VW = Batch<NB>::VW, TR = kTileRows<NB>;
     const int64_t r0 = (int64_t)blockIdx.x * TR;
@@ -95,21 +124,25 @@ __global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict_
         const Vec<VW> v = ld_il<VW>(src + row * NB);
 #pragma unroll
         for (int c = 0; c < NB; ++c)
-            if (c < nimg) dst[(int64_t)c * rows + row] = v.v[c];
+            if (c < nimg) dst[(int64_t)c * rows + row] = unpadded<NB>(v.v[c], T, row, c);
     } else {
         __shared__ float tile[TR][NB + 1];
         const int nr = (int)(rows - r0 < TR ? rows - r0 : TR);
+        float zero = 0.f;  // stays 0 while every sum is finite
 #pragma unroll 4
         for (int e = threadIdx.x; e < nr * (NB / 4); e += kPackBlock) {
             const int r = e / (NB / 4), c = e % (NB / 4) * 4;
             const Vec<4> v = ld_il<4>(src + (r0 + r) * NB + c);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) tile[r][c + k] = v.v[k];
+            for (int k = 0; k < 4; ++k) {
+                tile[r][c + k] = v.v[k];
+                zero = fmaf(v.v[k], 0.f, zero);
+            }
         }
-        __syncthreads();
+        const bool fine = __syncthreads_and(zero == 0.f);
         for (int e = threadIdx.x; e < TR * nimg; e += kPackBlock) {
             const int r = e % TR, c = e / TR;
-            if (r < nr) dst[(int64_t)c * rows + r0 + r] = tile[r][c];
+            if (r < nr) dst[(int64_t)c * rows + r0 + r] = fine ? tile[r][c] : unpadded<NB>(tile[r][c], T, r0 + r, c);
         }
     }
 }
@@ -119,10 +152,8 @@ __global__ void __launch_bounds__(kPackBlock) k_from_il(const float *__restrict_
 // consecutive rows walk pixel tiles of 8 columns, so that pixels sharing rays
 // share an L1; otherwise rows are taken in order (adjacent rays of a view share
 // pixels).  With a warp per row lanes gather 8 images of an entry from 16 images on
-// (row_dot_w), otherwise 4 (row_dot_g).
-//   row_dot pads a row with entries of weight 0 at index 0, whose product with a
-// value there that is not finite is not 0: a block with a sum that is not finite
-// goes over its rows once more, without padding.
+// (row_dot_w), otherwise 4 (row_dot_g).  Rows are padded with entries of weight 0 at
+// index 0: where the value there is not finite, k_from_il forms the sum again.
 template <int NB, int G, bool TILED>
 __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict__ ptr, const Entry *__restrict__ ent,
                                                       int64_t rows, int n, int nz, const float *__restrict__ src,
@@ -130,16 +161,15 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
 {
     constexpr int VW = Batch<NB>::VW, LPE = Batch<NB>::CPB;
     constexpr int TW = kTileW, TH = kOpBlock / G > 64 ? kOpBlock / G / TW : 8;
-    constexpr unsigned SITE = TILED ? CHK_GATHER_AT : CHK_GATHER_A;
     const int lr = threadIdx.x % G, grp = lr / LPE, vl = lr % LPE;
     const int64_t rpb = kOpBlock / G;
     const int tiles_x = (n + TW - 1) / TW, tiles_y = (n + TH - 1) / TH;
     const int64_t per_slice = (int64_t)tiles_x * tiles_y * TW * TH;
     const int64_t vrows = TILED ? per_slice * nz : rows;
     const unsigned long long pol = l2_evict_last_policy();
-    // row v of the block's walk: its index (false: none) and its entries [b, e)
-    auto locate = [&](int64_t v, int64_t &row, int64_t &b, int64_t &e) {
-        row = v;
+    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
+        const int64_t v = v0 + threadIdx.x / G;
+        int64_t row = v;
         bool ok = v < vrows;
         if (TILED && ok) {  // slice k, tile of the slice, pixel of the tile
             const int64_t k = v / per_slice, vs = v % per_slice;
@@ -149,56 +179,17 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
             ok = i < n && j < n;
             row = (k * n + i) * n + j;
         }
-        b = e = 0;
+        int64_t b = 0, e = 0;
         if (ok) {
             b = ptr[row];
             e = ptr[row + 1];
         }
-        return ok;
-    };
-    // Whether every sum is finite.  Narrow widths add 0 times the sum, which stays 0 (a
-    // comparison each cost the cone pair 3 %), wide ones, short of registers, compare.
-    float zero = 0.f;
-    bool fine = true;
-    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
-        int64_t row, b, e;
-        const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
         Vec<VW> acc;
         if constexpr (NB >= 16 && G == 32)
-            acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, SITE);
+            acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
         else
-            acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, SITE);
-#pragma unroll
-        for (int c = 0; c < VW; ++c) {
-            if constexpr (NB > 16) fine = fine && isfinite(acc.v[c]);
-            else zero = fmaf(acc.v[c], 0.f, zero);
-        }
+            acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
         if (ok && grp == 0) st_v<VW>(dst + row * NB + vl * VW, acc);
-    }
-    if (__syncthreads_and(fine && zero == 0.f)) return;
-    const GatherIL<NB> gather{src, src_rows, SITE};
-    for (int64_t v0 = (int64_t)blockIdx.x * rpb; v0 < vrows; v0 += (int64_t)gridDim.x * rpb) {
-        int64_t row, b, e;
-        const bool ok = locate(v0 + threadIdx.x / G, row, b, e);
-        Vec<VW> acc;
-        acc.zero();
-        for (int64_t k = b + grp; k < e; k += G / LPE) {
-            const Entry en = ld_entry(ent + k);
-            const Vec<VW> xv = gather(en.x, vl);
-#pragma unroll
-            for (int c = 0; c < VW; ++c) acc.v[c] = fmaf(__int_as_float(en.y), xv.v[c], acc.v[c]);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int off = LPE; off < G; off <<= 1)
-#pragma unroll
-            for (int c = 0; c < VW; ++c) acc.v[c] += __shfl_xor_sync(0xffffffffu, acc.v[c], off);
-        if (ok && grp == 0) {
-            float *o = dst + row * NB + vl * VW;  // written by this thread
-#pragma unroll
-            for (int c = 0; c < VW; ++c)
-                if (!isfinite(o[c])) o[c] = acc.v[c];
-        }
     }
 }
 
@@ -217,7 +208,8 @@ cudaError_t pass(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t 
         tiled ? rows(k_rows_il<NB, 32, true>) : rows(k_rows_il<NB, 32, false>);
     else
         tiled ? rows(k_rows_il<NB, kLanes<NB>, true>) : rows(k_rows_il<NB, kLanes<NB>, false>);
-    k_from_il<NB><<<bo, kPackBlock, 0, s>>>(out_il, dst, rows_out, nimg);
+    const RowTable T{ptr, ent, in_il, rows_in, tiled ? CHK_GATHER_AT : CHK_GATHER_A};
+    k_from_il<NB><<<bo, kPackBlock, 0, s>>>(out_il, dst, rows_out, nimg, T);
     count_launches(3);
     return cudaGetLastError();
 }
