@@ -151,8 +151,8 @@ dect_status dect_plan_copy_table(const dect_plan *plan, int64_t *rowptr, int32_t
  * into a pixel-major interleaved scratch ([pixel][64]), streams the ray-major
  * table once, and copies the sums out.  A last pass of up to 16 images streams
  * the plan's line table instead, where the plan has it (rays that end outside the
- * image, 4 <= n <= 4096, memory to spare; above four images from 2^22 elements
- * on): the same lengths, rounded to FP32 on their own, pieces below 1e-10 of a line's
+ * image, 4 <= n <= 4096, memory to spare; above four images from 3.5 million
+ * elements on): the same lengths, rounded to FP32 on their own, pieces below 1e-10 of a line's
  * length left out.  FP32 multiply-add in a fixed order; deterministic.  The
  * scratch (about 4 (N + M) min(batch, 64) bytes, 8 N min(batch, 16) on the line
  * table) is taken from the stream-ordered allocator and returned before the call ends.

@@ -326,14 +326,15 @@ cudaError_t run_lines(const LineTable &T, const float *x, float *y, int batch, c
 
 // Images of a batch that A takes through the line table: the last pass, where it is
 // narrow enough.  Above four images a small matrix does not fill the chip with the
-// table's blocks, and a warp per ray is ahead up to about 4 million elements: 16 images of
-// 64^2 / 60 views 21 us against 25, 160^2 / 60 (2.8 million) 36 against 44, 192^2 / 60
-// (4.0) 48 against 46, 256^2 / 30 (3.6) 46 both, 384^2 / 30 (8.0) 83 against 64; 8 images
-// of 160^2 / 60 26 against 29, 192^2 / 60 32 against 31.
+// table's blocks, and a warp per ray is ahead up to about 3.5 million elements: 16 images
+// of 64^2 / 60 views 21 us against 25, 160^2 / 60 (2.8 million) 36 against 44, 256^2 / 30
+// (3.6) 46 both, 192^2 / 60 (4.0) 48 against 46, 384^2 / 30 (8.0) 83 against 64; 8 images of
+// 160^2 / 60 26 against 29, 256^2 / 30 30 both, 192^2 / 60 32 against 31.
+constexpr int64_t kLineElements = 3500000;
 int line_tail(const dect_plan *p, int batch)
 {
     const int rest = batch % kMaxBatchImages;
-    return p->lines.ok && rest <= kLineMaxImages && (rest <= 4 || p->nnz >= (int64_t)1 << 22) ? rest : 0;
+    return p->lines.ok && rest <= kLineMaxImages && (rest <= 4 || p->nnz >= kLineElements) ? rest : 0;
 }
 
 }  // namespace

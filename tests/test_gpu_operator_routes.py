@@ -2,7 +2,7 @@
 
 A^T of narrow passes takes a warp per pixel up to 9728 pixels (14592 where a pixel
 meets 256 rays or more, 77824 of 8 images) and eight lanes beyond; A takes the line
-table, above four images from 2^22 elements on.  Cone-beam A takes a warp per ray up
+table, above four images from 3.5 million elements on.  Cone-beam A takes a warp per ray up
 to 24320 rays.  Tolerance 1e-5 relative L2, that of the projector tests.
 """
 import numpy as np
@@ -26,7 +26,7 @@ SIZES = {
     "120": (120, 150, 170), "121": (121, 150, 170),    # 14400 and 14641 pixels of about 270 rays
     "120 short rows": (120, 140, 170),                 # about 250 rays
     "278": (278, 160, 400), "279": (279, 160, 400),    # 77284 and 77841 pixels of about 290 rays
-    "below 2^22": (168, 110, 160), "above 2^22": (168, 120, 160),
+    "below 3.5 million": (168, 90, 160), "above 3.5 million": (168, 100, 160),
 }
 
 
@@ -35,7 +35,7 @@ def test_the_sizes_lie_where_they_are_meant_to():
     assert nnz["98"] < 256 * 9604
     assert nnz["120"] >= 256 * 120 ** 2 and nnz["121"] >= 256 * 121 ** 2 and nnz["120 short rows"] < 256 * 120 ** 2
     assert nnz["278"] >= 256 * 278 ** 2 and nnz["279"] >= 256 * 279 ** 2
-    assert nnz["below 2^22"] < 2 ** 22 <= nnz["above 2^22"] < 1.2 * 2 ** 22
+    assert nnz["below 3.5 million"] < 3.5e6 <= nnz["above 3.5 million"] < 4e6
 
 
 @pytest.mark.parametrize("name", sorted(SIZES))
