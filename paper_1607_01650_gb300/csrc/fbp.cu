@@ -211,10 +211,12 @@ __device__ __forceinline__ void digits(long long Q, __nv_bfloat16 (&d)[kDig])
 // holds (T(w - kpad - 16), T(w - kpad - 17)) of the even outputs, T(x) = 1 / (2 j +
 // 1)^2, j = x - 1 for x > 0 and -x otherwise.  (Formed by every block, the digits' FP64
 // divisions were a tenth of the filter.)
-__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap, unsigned *tw)
+// And the pixel coordinates along an axis [n].
+__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap, unsigned *tw, FF *pos)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const FilterShape F = filter_shape(g.n_bins);
+    if (t < g.n) pos[t] = ff_of(((double)t + 0.5 - 0.5 * (double)g.n) * g.pixel_mm);
     if (t < g.n_bins) cwd[t] = cos_weight(g, t);
     if (t <= g.n_bins / 2) tap[t] = odd_tap(2.0 * t + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
     if (t < F.tn) {
@@ -364,9 +366,7 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
     }
     // What is left to FP64: the rows' q in place of the digits, a warp per row; then a warp
     // per output, its lanes over the taps, 32 bins after 32 to one warp after the other.
-    if (!__syncthreads_or(lane < F.nw && todo[warp * F.nw + lane] != 0u ||
-                          lane + 32 < F.nw && todo[warp * F.nw + lane + 32] != 0u))
-        return;
+    __syncthreads();  // every warp has set its bits and read the digits
     double *q = reinterpret_cast<double *>(dyn);  // [row][nb]
     {
         bool any = false;
@@ -416,12 +416,13 @@ struct BpShape {
 // case below).
 struct BpConst {
     int n, nv, nb;
-    FF pixel, sod, half_dth, t0;  // t0: the isocentre's bin coordinate, negated
+    FF sod, half_dth, t0;  // t0: the isocentre's bin coordinate, negated
 };
 
 template <int W>
 __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict__ qf, float *__restrict__ x,
-                                                        const ViewGeo *__restrict__ vg, BpConst K, int nimg)
+                                                        const ViewGeo *__restrict__ vg, const FF *__restrict__ pos,
+                                                        BpConst K, int nimg)
 {
     using S = BpShape<W>;
     constexpr int NV = S::IPL / S::VW;
@@ -430,9 +431,7 @@ __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict_
     const int p = threadIdx.x / S::LPP, sub = threadIdx.x % S::LPP;
     const int i = blockIdx.y * S::TH + p / S::TW, j = blockIdx.x * S::TW + p % S::TW;
     const bool in = i < n && j < n;
-    // (half integers below 2^23: exact)
-    const FF px = ff_mul(FF{0.5f * (float)(2 * j + 1 - n), 0.f}, K.pixel);
-    const FF py = ff_mul(FF{0.5f * (float)(2 * i + 1 - n), 0.f}, K.pixel);
+    const FF px = pos[min(j, n - 1)], py = pos[min(i, n - 1)];
     const float tmax = (float)(nb - 1);
     float acc[S::IPL];
 #pragma unroll
@@ -520,11 +519,11 @@ __global__ void __launch_bounds__(kBpBlock, 2) k_fbp_bp(const float *__restrict_
 }
 
 template <int W>
-void launch_bp(const float *qf, float *x, const ViewGeo *vg, const BpConst &K, int nimg, cudaStream_t s)
+void launch_bp(const float *qf, float *x, const ViewGeo *vg, const FF *pos, const BpConst &K, int nimg, cudaStream_t s)
 {
     using S = BpShape<W>;
     const dim3 grid((unsigned)((K.n + S::TW - 1) / S::TW), (unsigned)((K.n + S::TH - 1) / S::TH));
-    k_fbp_bp<W><<<grid, kBpBlock, 0, s>>>(qf, x, vg, K, nimg);
+    k_fbp_bp<W><<<grid, kBpBlock, 0, s>>>(qf, x, vg, pos, K, nimg);
 }
 
 }  // namespace
@@ -560,11 +559,13 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
     char *base = nullptr;
     const FilterShape F = filter_shape(g.n_bins);
     const size_t vbytes = sizeof(ViewGeo) * (size_t)g.n_views, wbytes = sizeof(unsigned) * (size_t)kDig * F.tn;
-    DECT_CUDA(cudaMallocAsync((void **)&base, qbytes + vbytes + wbytes + sizeof(double) * (size_t)(g.n_bins + nodd), s));
+    DECT_CUDA(cudaMallocAsync((void **)&base,
+                              qbytes + vbytes + wbytes + sizeof(double) * (size_t)(g.n_bins + nodd) + sizeof(FF) * g.n, s));
     float *qf = (float *)base;
     ViewGeo *vg = (ViewGeo *)(base + qbytes);
     unsigned *tw = (unsigned *)(base + qbytes + vbytes);  // (16-byte aligned: both sizes are multiples of 32)
     double *cwd = (double *)(base + qbytes + vbytes + wbytes), *tap = cwd + g.n_bins;
+    FF *pos = (FF *)(tap + nodd);
     FilterConst K;
     K.ds = g.pitch_mm * (g.sod_mm / g.sdd_mm);
     K.h0 = 1.0 / (4.0 * K.ds * K.ds);
@@ -574,11 +575,11 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
     cudaError_t e = cudaFuncSetAttribute(k_fbp_filter, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fbp_filter_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
-    const BpConst B{g.n, g.n_views, g.n_bins, ff_of(g.pixel_mm), ff_of(g.sod_mm),
-                    ff_of(0.5 * g.arc_rad / (double)g.n_views),
+    const BpConst B{g.n, g.n_views, g.n_bins, ff_of(g.sod_mm), ff_of(0.5 * g.arc_rad / (double)g.n_views),
                     ff_of(-0.5 * (double)(g.n_bins - 1) + g.det_offset_mm / g.pitch_mm)};
     if (e == cudaSuccess) {
-        k_fbp_tables<<<(std::max({g.n_views, g.n_bins, F.tn}) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap, tw);
+        k_fbp_tables<<<(std::max({g.n, g.n_views, g.n_bins, F.tn}) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap, tw,
+                                                                                                pos);
         count_launches(1);
     }
     for (int done = 0; done < batch && e == cudaSuccess; done += kMaxBatchImages) {
@@ -593,13 +594,13 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
         else
             k_fbp_filter<<<dim3(g.n_views, k), kFbpBlock, smem, s>>>(mk, qf, g, w);
         switch (w) {
-        case 1: launch_bp<1>(qf, xk, vg, B, k, s); break;
-        case 2: launch_bp<2>(qf, xk, vg, B, k, s); break;
-        case 4: launch_bp<4>(qf, xk, vg, B, k, s); break;
-        case 8: launch_bp<8>(qf, xk, vg, B, k, s); break;
-        case 16: launch_bp<16>(qf, xk, vg, B, k, s); break;
-        case 32: launch_bp<32>(qf, xk, vg, B, k, s); break;
-        default: launch_bp<64>(qf, xk, vg, B, k, s); break;
+        case 1: launch_bp<1>(qf, xk, vg, pos, B, k, s); break;
+        case 2: launch_bp<2>(qf, xk, vg, pos, B, k, s); break;
+        case 4: launch_bp<4>(qf, xk, vg, pos, B, k, s); break;
+        case 8: launch_bp<8>(qf, xk, vg, pos, B, k, s); break;
+        case 16: launch_bp<16>(qf, xk, vg, pos, B, k, s); break;
+        case 32: launch_bp<32>(qf, xk, vg, pos, B, k, s); break;
+        default: launch_bp<64>(qf, xk, vg, pos, B, k, s); break;
         }
         count_launches(2);
         e = cudaGetLastError();

@@ -57,6 +57,25 @@ def test_every_bin_of_rows_of_every_range(nb):
         assert (err <= 8 * 2.0 ** -24 * np.abs(want)).all(), (k, int((err / np.abs(want)).argmax()))
 
 
+@pytest.mark.parametrize("nb", [101, 150, 172, 199, 232])
+def test_rows_with_few_bins_left_to_fp64(nb):
+    """64 CT-like rows with air beside the object, in four blocks of 16: a bin in a hundred is summed again."""
+    g = _geometry(nb)
+    rng = np.random.default_rng(nb)
+    b = np.arange(nb) - 0.5 * (nb - 1)
+    m = np.empty((64, nb), np.float32)
+    for k in range(64):
+        rad = rng.uniform(0.2, 0.45) * nb
+        p = 0.02 * 2 * np.sqrt(np.maximum(rad ** 2 - (b - rng.uniform(-0.05, 0.05) * nb) ** 2, 0)) * 100 / nb
+        m[k] = -np.log(np.maximum(rng.poisson(2e5 * np.exp(-p)), 1) / 2e5)
+    plan, mt = dect.Plan(g), torch.tensor(m[:, None], device="cuda")
+    want = np.pi * np.stack([oracle.fbp_filter(g, r[None].astype(np.float64))[0] for r in m])
+    for _ in range(5):
+        x = dect.fbp(plan, mt).cpu().numpy()
+        got = np.stack([_bins(g, r) for r in x])
+        assert (np.abs(got - want) <= 8 * 2.0 ** -24 * np.abs(want)).all()
+
+
 def test_rows_share_a_block_with_rows_of_other_ranges():
     """Rows that are left to FP64 in whole, in part and not at all beside one another give what they give alone."""
     g = _geometry(300)
