@@ -30,15 +30,13 @@ constexpr int kLanes = NB <= 16 ? 8 : 32;
 // Whether a row takes a whole warp.  Eight lanes take its entries four times as
 // long one after the other, so on few rows a warp each is ahead: A^T up to two turns
 // of the grid, three where a row has 256 entries or more (8 images of 96^2, 60 views:
-// 20 us against 23; 112^2, 60 views: 22 and 23; 112^2, 180 views: 32 and 35; 128^2, 60
-// views: 25 and 23), with 8 images on such rows 16 (256^2, 180 views: 87 and 96;
-// 384^2: 175 and 177); cone-beam A up to five (8 images of 128^2 x 4, 22080 rays: 34
+// 20 us against 23; 112^2, 60 views: 22 and 23; 112^2, 180 views: 33 and 35; 128^2, 60
+// views: 25 and 23); cone-beam A up to five (8 images of 128^2 x 4, 22080 rays: 34
 // and 38; 64^2 x 16, 44160 rays: 37 and 34).
-template <int NB>
 bool warp_rows(bool tiled, int nz, int64_t rows, int64_t nnz)
 {
     if (!tiled && nz == 0) return true;  // fan-beam A
-    const int turns = !tiled ? 5 : nnz < 256 * rows ? 2 : NB == 8 ? 16 : 3;
+    const int turns = !tiled ? 5 : nnz < 256 * rows ? 2 : 3;
     return rows <= (int64_t)turns * kSMs * (kOpBlock / 32);
 }
 constexpr int kTileW = 8;  // A^T: tiles of 8 columns, so a tile's sinogram lines stay in one L1
@@ -151,8 +149,8 @@ __global__ void __launch_bounds__(kPackBlock, 8) k_from_il(const float *__restri
 // lanes per row.  TILED (pixel-major table of an n x n image): the block's
 // consecutive rows walk pixel tiles of 8 columns, so that pixels sharing rays
 // share an L1; otherwise rows are taken in order (adjacent rays of a view share
-// pixels).  With a warp per row lanes gather 8 images of an entry from 16 images on
-// (row_dot_w), otherwise 4 (row_dot_g).  Rows are padded with entries of weight 0 at
+// pixels).  Lanes gather 8 images of an entry above 16 images (row_dot_w), 4
+// below (row_dot_g, its partial sums with their rounding errors).  Rows are padded with entries of weight 0 at
 // index 0: where the value there is not finite, k_from_il forms the sum again.
 template <int NB, int G, bool TILED>
 __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict__ ptr, const Entry *__restrict__ ent,
@@ -185,10 +183,10 @@ __global__ void __launch_bounds__(kOpBlock) k_rows_il(const int64_t *__restrict_
             e = ptr[row + 1];
         }
         Vec<VW> acc;
-        if constexpr (NB >= 16 && G == 32)
+        if constexpr (NB > 16)
             acc = row_dot_w<NB, G, 8, 2>(ent, b, e, lr, src, pol, src_rows, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
         else
-            acc = row_dot<NB, G, true>(ent, b, e, src, src_rows, lr, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
+            acc = row_dot<NB, G, true, false, true>(ent, b, e, src, src_rows, lr, TILED ? CHK_GATHER_AT : CHK_GATHER_A);
         if (ok && grp == 0) st_v<VW>(dst + row * NB + vl * VW, acc);
     }
 }
@@ -204,7 +202,7 @@ cudaError_t pass(const int64_t *ptr, const Entry *ent, int64_t rows_in, int64_t 
     auto rows = [&](auto kernel) {
         kernel<<<kSMs, kOpBlock, 0, s>>>(ptr, ent, rows_out, n, std::max(nz, 1), in_il, rows_in, out_il);
     };
-    if (warp_rows<NB>(tiled, nz, rows_out, nnz))
+    if (warp_rows(tiled, nz, rows_out, nnz))
         tiled ? rows(k_rows_il<NB, 32, true>) : rows(k_rows_il<NB, 32, false>);
     else
         tiled ? rows(k_rows_il<NB, kLanes<NB>, true>) : rows(k_rows_il<NB, kLanes<NB>, false>);
