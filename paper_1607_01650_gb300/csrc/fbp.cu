@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
 // view share an L1.  The lanes of a pixel form the geometry of different views
 // and hand it round by shuffles.  Per pixel and view two bins x W x 4 bytes
 // come back from L1, which bounds the pass: 64 images of 512^2 from 60 views
-// are 8 GB, 200 us at the L1 rate (128 bytes per cycle and SM); measured 363
+// are 8 GB, 200 us at the L1 rate (128 bytes per cycle and SM); measured 332
 // us (10.4 ms with FP64 geometry repeated for every four images).
 // ---------------------------------------------------------------------------
 constexpr int kBpBlock = 512;
@@ -412,8 +412,8 @@ struct BpShape {
     static constexpr int GV = LPP < 4 ? 4 : LPP, GPL = GV / LPP;  // views of a group, of a lane's geometry
 };
 
-// Numbers of a call, in two words (formed in FP64 by every thread they took 47 us of the
-// case below).
+// Numbers of a call, in two words (these and the pixel coordinates, formed in FP64 by
+// every thread, took 47 us of the above case).
 struct BpConst {
     int n, nv, nb;
     FF sod, half_dth, t0;  // t0: the isocentre's bin coordinate, negated
