@@ -211,15 +211,21 @@ __device__ __forceinline__ void digits(long long Q, __nv_bfloat16 (&d)[kDig])
 // holds (T(w - kpad - 16), T(w - kpad - 17)) of the even outputs, T(x) = 1 / (2 j +
 // 1)^2, j = x - 1 for x > 0 and -x otherwise.  (Formed by every block, the digits' FP64
 // divisions were a tenth of the filter.)
-// And the pixel coordinates along an axis [n].
-__global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap, unsigned *tw, FF *pos)
+// And the pixel coordinates along an axis [n].  A table per blockIdx.y: one after the
+// other in a thread their FP64 divisions and sines took 12 us.
+constexpr int kTables = 4, kTableBlock = 64;
+__global__ void __launch_bounds__(kTableBlock) k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *tap,
+                                                            unsigned *tw, FF *pos)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * kTableBlock + threadIdx.x;
     const FilterShape F = filter_shape(g.n_bins);
-    if (t < g.n) pos[t] = ff_of(((double)t + 0.5 - 0.5 * (double)g.n) * g.pixel_mm);
-    if (t < g.n_bins) cwd[t] = cos_weight(g, t);
-    if (t <= g.n_bins / 2) tap[t] = odd_tap(2.0 * t + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
-    if (t < F.tn) {
+    if (blockIdx.y == 0) {
+        if (t < g.n_bins) cwd[t] = cos_weight(g, t);
+        if (t < g.n) pos[t] = ff_of(((double)t + 0.5 - 0.5 * (double)g.n) * g.pixel_mm);
+    } else if (blockIdx.y == 1) {
+        if (t <= g.n_bins / 2) tap[t] = odd_tap(2.0 * t + 1.0, g.pitch_mm * (g.sod_mm / g.sdd_mm));
+    } else if (blockIdx.y == 2) {
+        if (t >= F.tn) return;
         __nv_bfloat16 d0[kDig], d1[kDig];
         const int x = t - F.kpad - 16, j0 = x > 0 ? x - 1 : -x, j1 = x - 1 > 0 ? x - 2 : 1 - x;
         const double k0 = 2.0 * j0 + 1.0, k1 = 2.0 * j1 + 1.0;
@@ -228,11 +234,12 @@ __global__ void k_fbp_tables(dect_geometry g, ViewGeo *vg, double *cwd, double *
 #pragma unroll
         for (int k = 0; k < kDig; ++k)
             tw[k * F.tn + t] = (unsigned)__bfloat16_as_ushort(d0[k]) | ((unsigned)__bfloat16_as_ushort(d1[k]) << 16);
+    } else {
+        if (t >= g.n_views) return;
+        const double th = g.start_rad + (double)t * (g.arc_rad / (double)g.n_views);
+        const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
+        vg[t] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
     }
-    if (t >= g.n_views) return;
-    const double th = g.start_rad + (double)t * (g.arc_rad / (double)g.n_views);
-    const double c = cos(th), s = sin(th), k = g.sdd_mm / g.pitch_mm;  // SOD / ds
-    vg[t] = ViewGeo{ff_of(-s * k), ff_of(c * k), ff_of(-c), ff_of(-s)};
 }
 
 // Numbers of a call that every thread would divide for.
@@ -290,7 +297,9 @@ __global__ void __launch_bounds__(kTcThreads) k_fbp_filter_tc(const float *__res
         }
     }
     const int gid = lane >> 2, t4 = lane & 3;
-    for (int par = 0; par < 2; ++par) {  // outputs of parity par from inputs of the other
+    // outputs of parity par from inputs of the other: both, or (two blocks per 16 rows) one
+    const int par0 = gridDim.y == 2 ? (int)blockIdx.y : 0, par1 = gridDim.y == 2 ? par0 + 1 : 2;
+    for (int par = par0; par < par1; ++par) {
         __syncthreads();  // the scales are written; the other parity's digits have been read
         for (int i = lane; i < F.kpad; i += 32) {
             __nv_bfloat16 d[kDig];
@@ -578,8 +587,9 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
     const BpConst B{g.n, g.n_views, g.n_bins, ff_of(g.sod_mm), ff_of(0.5 * g.arc_rad / (double)g.n_views),
                     ff_of(-0.5 * (double)(g.n_bins - 1) + g.det_offset_mm / g.pitch_mm)};
     if (e == cudaSuccess) {
-        k_fbp_tables<<<(std::max({g.n, g.n_views, g.n_bins, F.tn}) + 255) / 256, 256, 0, s>>>(g, vg, cwd, tap, tw,
-                                                                                                pos);
+        const int most = std::max({g.n, g.n_views, g.n_bins, F.tn});
+        k_fbp_tables<<<dim3((unsigned)((most + kTableBlock - 1) / kTableBlock), kTables), kTableBlock, 0, s>>>(
+            g, vg, cwd, tap, tw, pos);
         count_launches(1);
     }
     for (int done = 0; done < batch && e == cudaSuccess; done += kMaxBatchImages) {
@@ -588,10 +598,13 @@ extern "C" dect_status dect_fbp(const dect_plan *plan, const float *m, float *x,
         float *xk = x + (int64_t)done * plan->N;
         int w = 1;
         while (w < k) w *= 2;
-        if (tc)
-            k_fbp_filter_tc<<<(unsigned)(((int64_t)g.n_views * k + kTcRows - 1) / kTcRows), kTcThreads, F.smem, s>>>(
+        if (tc) {
+            // few rows leave most of the chip idle: a block per parity then (call on one image of
+            // 512^2 / 60 views, 8 blocks instead of 4: 186 -> 147 us)
+            const unsigned blocks = (unsigned)(((int64_t)g.n_views * k + kTcRows - 1) / kTcRows);
+            k_fbp_filter_tc<<<dim3(blocks, blocks <= (unsigned)kSMs / 2 ? 2 : 1), kTcThreads, F.smem, s>>>(
                 mk, qf, cwd, tap, (const uint4 *)tw, g, K, k, w);
-        else
+        } else
             k_fbp_filter<<<dim3(g.n_views, k), kFbpBlock, smem, s>>>(mk, qf, g, w);
         switch (w) {
         case 1: launch_bp<1>(qf, xk, vg, pos, B, k, s); break;

@@ -102,3 +102,14 @@ def test_pixel_weights_are_rounded_once(n, batch):
     for k in range(batch):
         want = np.pi * r * r * 2.0 ** k / 4
         assert (np.abs(x[k, n // 2] - want) <= 2.0 ** -24 * (1 + 2.0 ** -20) * want).all()
+
+
+@pytest.mark.parametrize("nv", [19, 20])
+def test_a_block_per_parity_and_one_for_both(nv):
+    """64 images of 19 views make 76 blocks of 16 rows, the most that are split by parity; of 20 views 80."""
+    g = synth.tiny_geometry(n=21, nv=nv, nb=35, px=1.0, start=0.3, det_offset=0.2)
+    m = np.random.default_rng(nv).standard_normal((64, nv, 35)).astype(np.float32)
+    x = dect.fbp(dect.Plan(g), torch.tensor(m, device="cuda")).cpu().numpy()
+    for k in range(0, 64, 9):  # tolerance of test_gpu_fbp.py
+        want = oracle.fbp(g, m[k].astype(np.float64))
+        assert np.linalg.norm(x[k] - want) <= 1e-5 * np.linalg.norm(want)
